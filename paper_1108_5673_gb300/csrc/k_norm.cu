@@ -4,6 +4,9 @@
 //
 //   M[a][b] = (1/N_gen) sum_{j in accepted MC} conj(A_a(j)) A_b(j).
 //
+// Serves the samples whose amplitudes leave the tensor-core kernel's range
+// (k_norm_tc.cu) and PWA_NORM_KERNEL=fp64.
+//
 // Exactness: a product of two floats is exact in double, so every term is
 // formed exactly and summed in FP64; the matrix carries ~1e-15 relative
 // rounding, far below what the NLL needs (V^H M V ~ N_data).

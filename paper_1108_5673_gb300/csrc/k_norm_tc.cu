@@ -20,31 +20,54 @@
 // digits s and t of rows p and q is c c' 2^(r_p + r_q - 8(s + t)): within one
 // accumulator entry (p, q) of one digit pair all products are integer
 // multiples of one quantum and at most 2^14 of it, so the tensor cores' FP32
-// sum over 512 events (at most 2^23 quanta) is exact.
+// sum over 1024 events (at most 2^24 quanta) is exact.
 //
-// Digit blocks D_st[p][q] = sum_j t_s(p, j) t_t(q, j). The main MMA takes A =
-// rows [X1; X2; X3] (digits 1-3 of every row, 3R <= 128 rows) and B = rows
-// [X1; ...; X5] (5R columns): the blocks s <= 3, t <= 5, exact, drained every
-// 512 events into float-float sums per CTA. The blocks with s >= 4, t <= 3
-// are their transposes (D_ts[q][p] = D_st[p][q], exactly). A second MMA takes
-// A = [X4; X5] and B = X4: the blocks (4,4) and (5,4) (and (4,5) as the
-// transpose of (5,4)), below 2^-36 of the leading ones, accumulated in FP32
-// over the whole launch (one-sided roundings of at most 2^-12 of their size
-// per CTA). Every pair but (5,5) is kept: per event and real entry of G the
-// error is at most 2^-41 (|x_p| 2^r_q [|x_q| < 2^(r_q - 17)] + |x_q| 2^r_p
-// [|x_p| < 2^(r_p - 17)]) + 2^(r_p + r_q - 61), with unbiased signs apart
-// from the last term.
+// Digit blocks D_st[p][q] = sum_j t_s(p, j) t_t(q, j), R rows each, from at
+// most two MMAs per tile on the same digits in shared memory. The first takes
+// as many digits as fit M = 128 rows (S1 = 5 up to 12 waves, 3 up to 20, 2 up
+// to 32) against all five; the second the next two digits against the rest
+// (none, [X4; X5] against X4, [X3; X4] against [X3; X4; X5]). An M = 128 MMA
+// reads its 128 A rows whatever the number of columns, which is what a small
+// model's tile costs, hence one MMA where everything fits. With D_ts =
+// D_st^T these are all pairs (all but (5,5) beyond 12 waves), all exact,
+// drained every 1024 events:
+//   G = T + U + U^T, T the products whose transposes are among them too (a
+//   symmetric sum), U the others,
+// so that one sum W = T/2 + U per (row, column) serves, G = W + W^T: float-
+// float for the first MMA's blocks, plain FP32 for the second's, which are
+// below 2^-32 of the leading one. Per event and real entry of G the error is
+// at most 2^-41 (|x_p| 2^r_q [|x_q| < 2^(r_q - 17)] + |x_q| 2^r_p [|x_p| <
+// 2^(r_p - 17)]) + 2^(r_p + r_q - 61), with unbiased signs apart from the last
+// term. Measured against an exact Gram matrix (inputs on a 2^-22 grid): 0.6-
+// 1.5e-16 of M at 4-48 waves, 1-10M events; FP64 sums of the exact products
+// give 4-5e-16.
 //
-// Per CTA (persistent, one per SM): a TMA warp streams 64-event tiles of the
-// 2N MC planes; four consumer warps (tile j to warp j % 4, each with two TMA
-// stages and one digit buffer of its own) write the digits K-major with
-// 128-byte swizzle (rows (s - 1) R + p, one 64-event K-atom); one thread
-// issues the two MMAs (kind::f16, M = 128, K = 16; four steps per tile), the
-// main one into one of two accumulators in tensor memory (alternating every
-// eight tiles); eight drain warps (two per lane quarter, half of the columns
-// each) add the main accumulator into float-float sums. The CTA's share of M
-// goes to global memory with the CTA index innermost; norm_tc_finalize adds
-// the CTAs in a fixed order, divides by N_gen and fills the Hermitian matrix.
+// More than 32 waves: the accumulators no longer fit tensor memory, so the
+// waves are cut into three blocks and three launches take two blocks each
+// (two TMA boxes per tile); between them every pair of waves is covered, at
+// twice the one-pass traffic and digit work.
+//
+// Per CTA (persistent, one per SM), sixteen warps (128 registers a thread): a
+// TMA warp streams 64-event tiles of the planes; six consumer warps in GROUPS
+// groups (tile j to group j mod GROUPS, its row pairs shared by the group's
+// warps: one-warp groups for the few rows of a small model, so that several
+// tiles are in flight, three-warp groups from 16 waves on) write the digits
+// K-major with 128-byte swizzle into a ring of digit buffers; one thread
+// issues the MMAs (kind::f16, K = 16, four steps per tile); eight drain warps
+// (two per lane quarter, half of each block's columns) add the accumulators
+// into W. Up to 20 waves two accumulator sets alternate; beyond, one set, whose
+// two MMAs hand over separately, so that the first MMA of the next period
+// runs while the second accumulator is drained. The CTA's share of M goes to
+// global memory with the CTA index innermost; norm_tc_finalize adds the CTAs
+// in a fixed order, divides by N_gen and fills the Hermitian matrix.
+//
+// Bound: the digit split (30 packed FP32 operations per two rows and four
+// events, on six warps) and the MMAs, about 1300 and 1024 cycles per tile at
+// 32 waves, overlapping in part. Per call of pwa_build_norm: 10M x 32 in 0.94
+// ms (2.7 TB/s of amplitudes), 5M x 20 in 0.35 ms, 10M x 12 in 0.41 ms, 4M x
+// 48 in 1.18 ms; before, with one-warp consumers per tile, 0.49 ms at 5M x 20
+// and 0.63 at 10M x 12, and on the FP64 pipe beyond 20 waves 81 ms at 10M x
+// 32 and 69 ms at 4M x 48.
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -52,50 +75,68 @@ namespace pwa {
 namespace {
 
 constexpr int kNTE = 64;         // events per tile (one K-atom)
-constexpr int kNCons = 4;        // consumer warps
-constexpr int kNSPC = 2;         // TMA stages per consumer warp
-constexpr int kNDrain = 8;       // drain warps (warps 4..11: lane quarter = warp % 4)
-constexpr int kNFirstDrain = 4;
-constexpr int kNWarps = 14;      // 0 TMA, 1 MMA, 2-3 and 12-13 consumers, 4-11 drain
+constexpr int kNCons = 6;        // consumer warps
+constexpr int kNDrain = 8;       // drain warps (warps 2..9: lane quarter = warp % 4)
+constexpr int kNFirstDrain = 2;
+constexpr int kNFirstCons = kNFirstDrain + kNDrain;
+constexpr int kNWarps = kNFirstCons + kNCons;  // 0 TMA, 1 MMA, 2-9 drain, 10-15 consumers
 constexpr int kNThreads = kNWarps * 32;
 constexpr int kNDigits = 5;
-constexpr int kNPeriod = 8;      // tiles per accumulation period (512 events: sums < 2^23)
+constexpr int kNPeriod = 16;     // tiles per accumulation period (1024 events: sums <= 2^24)
 constexpr uint32_t kNTmemCols = 512;
 constexpr int kNFinMaxRounds = 8;    // CTAs up to 32 x 8
-
-__device__ __forceinline__ int consumer_index(int warp)
-{
-    return warp < kNFirstDrain ? warp - 2 : warp - (kNFirstDrain + kNDrain) + 2;
-}
+constexpr int kNMaxOnePass = 32;     // waves of one launch
 
 constexpr int round_up16(int x) { return (x + 15) / 16 * 16; }
-constexpr int round_up32(int x) { return (x + 31) / 32 * 32; }
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int cmin(int a, int b) { return a < b ? a : b; }
 
 template <int NW>
 struct NormTcCfg {
-    static constexpr int R = 2 * NW;                    // real rows (padded waves)
-    static constexpr int N1 = round_up16(kNDigits * R); // main MMA: B = digits 1-5
-    static constexpr int N2 = round_up16(R);            // second MMA: B = digit 4
-    // buffer rows: the digits, the main B operand's padding, and the 128 rows
-    // the second MMA's A operand reads from row 3R on
-    static constexpr int BUFROWS = cmax(cmax(N1, 3 * R + 128), 128);
-    static constexpr uint32_t JBYTES = BUFROWS * 128;   // one 64-event K-atom of every row
+    static constexpr int R = 2 * NW;                         // real rows (padded waves)
+    // digits in the first MMA's A operand; the second MMA takes digits S1 + 1
+    // and S1 + 2 against B2 digits from S1 + 1 on (none when S1 = 5)
+    static constexpr int S1 = NW <= 12 ? 5 : NW <= 20 ? 3 : 2;
+    static constexpr int B2 = S1 == 5 ? 0 : S1 == 3 ? 1 : 3;
+    static constexpr int N1 = round_up16(kNDigits * R);      // columns of the first MMA: digits 1-5
+    static constexpr int N2 = round_up16(B2 * R);            // of the second
+    static constexpr int NI1 = N1 > 256 ? N1 / 2 : N1;       // one instruction's columns
+    static constexpr int WPG = NW <= 8 ? 1 : NW <= 12 ? 2 : 3;  // warps per consumer group
+    static constexpr int GROUPS = kNCons / WPG;
+    static constexpr int ITERS = (NW + WPG - 1) / WPG;       // row pairs per warp and tile
+    static constexpr int NBUF = NW <= 12 ? 6 : 4;
+    static constexpr int NACC = 2 * (N1 + N2) <= (int)kNTmemCols ? 2 : 1;
+    // buffer rows: the digits, the B operands' padding, and the 128 rows that
+    // each A operand reads
+    static constexpr int BUFROWS =
+        cmax(cmax(N1, 128), B2 ? cmax(S1 * R + N2, S1 * R + 128) : 0);
+    static constexpr uint32_t JBYTES = BUFROWS * 128;        // one 64-event K-atom of every row
     static constexpr uint32_t STAGE_BYTES = R * kNTE * 4;
-    static constexpr int STAGES = kNCons * kNSPC;
-    static constexpr uint32_t ACC1 = round_up32(N1);    // column of the second main accumulator
-    static constexpr uint32_t ACCX = 2 * ACC1;          // column of the small-block accumulator
-    static constexpr size_t SMEM = (size_t)kNCons * JBYTES + (size_t)STAGES * STAGE_BYTES + 1024;
-    // the CTA's sums as doubles, T[3R][R], U[3R][R] and X[2R][R], reuse the digit buffers
-    static constexpr size_t SUMS_BYTES = (size_t)8 * R * R * sizeof(double);
-    static_assert(3 * R <= 128, "digits 1-3 of every row fill M = 128");
-    static_assert(N1 <= 256 && N2 <= 256, "N of the MMA");
-    static_assert(ACCX + N2 <= kNTmemCols, "tensor memory");
-    static_assert(NW % 4 == 0, "drain in 4-column steps");
-    static_assert(JBYTES % 1024 == 0 && STAGE_BYTES % 1024 == 0 && (3 * R) % 8 == 0,
-                  "swizzle atoms stay 1 KB aligned");
+    static constexpr int STAGES =
+        cmin(18, (int)((224 * 1024 - NBUF * JBYTES) / STAGE_BYTES)) / GROUPS * GROUPS;
+    static constexpr size_t SMEM = (size_t)NBUF * JBYTES + (size_t)STAGES * STAGE_BYTES + 1024;
+    // the CTA's sums W[S1 R][R] as doubles reuse the digit buffers
+    static constexpr size_t SUMS_BYTES = (size_t)S1 * R * R * sizeof(double);
+    static_assert(S1 * R <= 128, "S1 digits of every row fit M = 128");
+    static_assert(NI1 % 16 == 0 && NI1 <= 256 && N2 <= 256 && N1 % NI1 == 0, "N of the MMA");
+    static_assert(NACC * (N1 + N2) <= (int)kNTmemCols, "tensor memory");
+    static_assert(NW % 4 == 0, "drain in 4-column steps, 8-row swizzle atoms per digit");
+    // Stages and buffers belong to one group each: a group's parity wait on
+    // the phase of use k is then on a barrier whose use k - 1 it consumed
+    // itself. Shared ones would let a wait pass one phase too early, because
+    // copies can land out of order and groups can drift apart.
+    static_assert(STAGES >= GROUPS && STAGES % GROUPS == 0 && NBUF % GROUPS == 0, "owned rings");
+    static_assert(JBYTES % 1024 == 0 && STAGE_BYTES % 1024 == 0, "swizzle atoms stay 1 KB aligned");
     static_assert(SMEM <= 227 * 1024, "shared memory");
-    static_assert(SUMS_BYTES <= (size_t)kNCons * JBYTES, "sums fit in the digit buffers");
+    static_assert(SUMS_BYTES <= (size_t)NBUF * JBYTES, "sums fit in the digit buffers");
+};
+
+// The waves of one launch: box k of blk waves starts at wave first[k]; local
+// wave w is wave first[w / blk] + w % blk (past the model's end: a zero wave).
+struct NormBlocks {
+    int n_box, blk, first[2];
+    __host__ __device__ int local() const { return n_box * blk; }
+    __host__ __device__ int global(int w) const { return w < blk ? first[0] + w : first[1] + w - blk; }
 };
 
 // Byte offset of (row, byte b of the row) in a K-major operand with 128-byte
@@ -116,14 +157,14 @@ __device__ __forceinline__ uint32_t to_bf16x2(float lo, float hi)
     return r;
 }
 
-__device__ __forceinline__ f2 lds2_f2(const float *p) { return *reinterpret_cast<const f2 *>(p); }
-
-__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v)
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b)
 {
-    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+    // no memory clobber: loads of the next rows may move above it; the proxy
+    // fence that follows the stores is ordered after them (both volatile)
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b));
 }
 
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t *r)
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -157,75 +198,88 @@ __device__ __forceinline__ float first_digit_constant(float amax)
 template <int NW>
 __device__ __forceinline__ void tmem_row_half(uint32_t taddr, uint32_t (&v)[NW])
 {
+    if constexpr (NW % 16 == 0) {
 #pragma unroll
-    for (int c4 = 0; c4 < NW / 4; ++c4) {
-        uint32_t r4[4];
-        tmem_ld4(taddr + (uint32_t)(4 * c4), r4);
+        for (int c = 0; c < NW / 16; ++c)
+            tmem_ld16(taddr + (uint32_t)(16 * c), *reinterpret_cast<uint32_t(*)[16]>(v + 16 * c));
+    } else if constexpr (NW % 8 == 0) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            v[4 * c4 + i] = r4[i];
+        for (int c = 0; c < NW / 8; ++c)
+            tmem_ld8(taddr + (uint32_t)(8 * c), *reinterpret_cast<uint32_t(*)[8]>(v + 8 * c));
+    } else {
+#pragma unroll
+        for (int c = 0; c < NW / 4; ++c)
+            tmem_ld4(taddr + (uint32_t)(4 * c), v + 4 * c);
     }
 }
 
 template <int NW>
 __global__ void __launch_bounds__(kNThreads, 1)
     norm_tc_kernel(const __grid_constant__ CUtensorMap map, const float *__restrict__ amax,
-                   int n_waves, int n_tiles, double *__restrict__ part, int *status)
+                   int n_waves, NormBlocks blocks, int n_tiles, double *__restrict__ part,
+                   int *status)
 {
     using C = NormTcCfg<NW>;
-    constexpr int R = C::R, STAGES = C::STAGES;
+    constexpr int R = C::R, S1 = C::S1, STAGES = C::STAGES, NBUF = C::NBUF, NACC = C::NACC;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const uint32_t jbase = smem_u32(base);
-    float *stages = reinterpret_cast<float *>(base + (size_t)kNCons * C::JBYTES);
-    __shared__ uint64_t full[STAGES], empty[STAGES], jfull[kNCons], jempty[kNCons];
-    __shared__ uint64_t accfull[2], accempty[2], g_done;
+    float *stages = reinterpret_cast<float *>(base + (size_t)NBUF * C::JBYTES);
+    __shared__ uint64_t full[STAGES], empty[STAGES], jfull[NBUF], jempty[NBUF];
+    __shared__ uint64_t accfull[2 * NACC], accempty[2 * NACC], g_done;
     __shared__ float s_sig[R];
     __shared__ uint32_t tmem_base;
     __shared__ int s_flags;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tiles of this CTA: blockIdx.x + j gridDim.x, j < n_my; tile j goes to
-    // consumer j % kNCons, to its stage (j / kNCons) % kNSPC and its buffer
+    // consumer group j % GROUPS, TMA stage j % STAGES, digit buffer j % NBUF
     const int n_my =
         (n_tiles > (int)blockIdx.x) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const uint32_t stage_tx = 2u * (uint32_t)n_waves * kNTE * 4u;
-    auto stage_of = [](int j) { return (j % kNCons) * kNSPC + (j / kNCons) % kNSPC; };
-    auto use_of = [](int j) { return (uint32_t)((j / kNCons) / kNSPC); };
+    const int box_rows = 2 * blocks.blk;
+    const uint32_t stage_tx = (uint32_t)(blocks.n_box * box_rows) * kNTE * 4u;
     const int n_first = n_my < STAGES ? n_my : STAGES;
+    auto issue = [&](int j) {
+        const int s = j % STAGES;
+        float *dst = stages + (size_t)s * (C::STAGE_BYTES / 4);
+        const int x = ((int)blockIdx.x + j * (int)gridDim.x) * kNTE;
+        mbar_arrive_expect_tx(&full[s], stage_tx);
+        for (int k = 0; k < blocks.n_box; ++k)
+            tma_load_2d(dst + k * box_rows * kNTE, &map, x, 2 * blocks.first[k], &full[s]);
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&empty[s], C::WPG);
         }
-        for (int c = 0; c < kNCons; ++c) {
-            mbar_init(&jfull[c], 1);
-            mbar_init(&jempty[c], 1);
+        for (int b = 0; b < NBUF; ++b) {
+            mbar_init(&jfull[b], C::WPG);
+            mbar_init(&jempty[b], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < 2 * NACC; ++b) {
             mbar_init(&accfull[b], 1);
             mbar_init(&accempty[b], kNDrain);
         }
         mbar_init(&g_done, 1);
         fence_barrier_init();
         s_flags = 0;
-        for (int j = 0; j < n_first; ++j) {
-            mbar_arrive_expect_tx(&full[stage_of(j)], stage_tx);
-            tma_load_2d(stages + (size_t)stage_of(j) * (C::STAGE_BYTES / 4), &map,
-                        ((int)blockIdx.x + j * (int)gridDim.x) * kNTE, 0, &full[stage_of(j)]);
-        }
+        for (int j = 0; j < n_first; ++j)
+            issue(j);
     }
     // rows of padded waves are never written by TMA: zero them once; so are
     // the buffer rows past the digits, which the MMAs read as padding
+    const int in_rows = blocks.n_box * box_rows;
     for (int s = 0; s < STAGES; ++s)
-        for (int i = 2 * n_waves * kNTE + threadIdx.x; i < R * kNTE; i += blockDim.x)
+        for (int i = in_rows * kNTE + threadIdx.x; i < R * kNTE; i += blockDim.x)
             stages[(size_t)s * (C::STAGE_BYTES / 4) + i] = 0.f;
-    for (int c = 0; c < kNCons; ++c)
+    for (int b = 0; b < NBUF; ++b)
         for (uint32_t i = kNDigits * R * 32 + threadIdx.x; i < C::JBYTES / 4; i += blockDim.x)
-            reinterpret_cast<uint32_t *>(base + (size_t)c * C::JBYTES)[i] = 0u;
-    if (threadIdx.x < R)
-        s_sig[threadIdx.x] =
-            (threadIdx.x / 2 < n_waves) ? first_digit_constant(amax[threadIdx.x / 2]) : 1.5f * 32768.f;
+            reinterpret_cast<uint32_t *>(base + (size_t)b * C::JBYTES)[i] = 0u;
+    if (threadIdx.x < R) {
+        const int w = threadIdx.x / 2;
+        const int g = w < blocks.local() ? blocks.global(w) : n_waves;
+        s_sig[threadIdx.x] = g < n_waves ? first_digit_constant(amax[g]) : 1.5f * 32768.f;
+    }
     if (warp == 1)
         tmem_alloc(&tmem_base, kNTmemCols);
     fence_async_smem();
@@ -240,56 +294,70 @@ __global__ void __launch_bounds__(kNThreads, 1)
         if (lane == 0) {
             int j = n_first;
             for (; j < n_my; ++j) {
-                const int s = stage_of(j);
-                const uint32_t u = use_of(j);
-                if (u > 0 && !mbar_wait(&empty[s], (u & 1) ^ 1)) {
+                if (!mbar_wait(&empty[j % STAGES], (uint32_t)(j / STAGES - 1) & 1)) {
                     flags |= FLAG_TIMEOUT;
                     break;
                 }
-                mbar_arrive_expect_tx(&full[s], stage_tx);
-                tma_load_2d(stages + (size_t)s * (C::STAGE_BYTES / 4), &map,
-                            ((int)blockIdx.x + j * (int)gridDim.x) * kNTE, 0, &full[s]);
+                issue(j);
             }
             // no copy may still be landing in shared memory when the CTA exits
             for (int q = (j > STAGES ? j - STAGES : 0); q < j; ++q)
-                if (!mbar_wait(&full[stage_of(q)], use_of(q) & 1))
+                if (!mbar_wait(&full[q % STAGES], (uint32_t)(q / STAGES) & 1))
                     flags |= FLAG_TIMEOUT;
         }
     } else if (warp == 1) {
         // ---- MMA issuer ----------------------------------------------------
         if (lane == 0) {
-            const uint32_t id1 = umma_idesc_bf16(128, C::N1, 0, 0);
+            const uint32_t id1 = umma_idesc_bf16(128, C::NI1, 0, 0);
             const uint32_t id2 = umma_idesc_bf16(128, C::N2, 0, 0);
             const uint64_t dK = umma_desc_sw128(0, 16, 1024);
-            const uint32_t row4 = 3u * R * 128u;  // byte offset of digit 4's rows
+            const uint32_t row2 = (uint32_t)(S1 * R) * 128u;  // byte offset of digit S1 + 1's rows
             bool ok = true;
             for (int j = 0; j < n_my; ++j) {
-                const int c = j % kNCons;
-                if (!mbar_wait(&jfull[c], (uint32_t)(j / kNCons) & 1)) {
+                const int b = j % NBUF;
+                if (!mbar_wait(&jfull[b], (uint32_t)(j / NBUF) & 1)) {
                     ok = false;
                     break;
                 }
-                const int P = j / kNPeriod, ab = P & 1;
+                const int P = j / kNPeriod, set = P % NACC;
                 const bool first = (j % kNPeriod) == 0;
-                // accumulator ab is free once period P - 2 has been drained
-                if (first && P >= 2 && !mbar_wait(&accempty[ab], (uint32_t)((P >> 1) - 1) & 1)) {
+                const bool last = (j % kNPeriod) == kNPeriod - 1 || j == n_my - 1;
+                const uint32_t jb = jbase + (uint32_t)b * C::JBYTES;
+                const uint32_t acc1 = tmem + (uint32_t)set * (C::N1 + C::N2), acc2 = acc1 + C::N1;
+                // an accumulator is free once the period NACC before has been drained
+                if (first && P >= NACC && !mbar_wait(&accempty[2 * set], (uint32_t)(P / NACC - 1) & 1)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t jb = jbase + (uint32_t)c * C::JBYTES;
 #pragma unroll
                 for (int ks = 0; ks < kNTE / 16; ++ks) {
                     const uint32_t a = jb + (uint32_t)ks * 32;  // 16 events = 32 bytes of a row
-                    umma_bf16(tmem + (uint32_t)ab * C::ACC1, dK + (a >> 4), dK + (a >> 4), id1,
-                              (first && ks == 0) ? 0u : 1u);
-                    umma_bf16(tmem + C::ACCX, dK + ((a + row4) >> 4), dK + ((a + row4) >> 4), id2,
-                              (j == 0 && ks == 0) ? 0u : 1u);
+#pragma unroll
+                    for (int h = 0; h < C::N1 / C::NI1; ++h)
+                        umma_bf16(acc1 + (uint32_t)(h * C::NI1), dK + (a >> 4),
+                                  dK + ((a + (uint32_t)(h * C::NI1) * 128u) >> 4), id1,
+                                  (first && ks == 0) ? 0u : 1u);
                 }
-                // on completion the consumer's buffer is free again
-                umma_commit(&jempty[c]);
-                if ((j % kNPeriod) == kNPeriod - 1 || j == n_my - 1)
-                    umma_commit(&accfull[ab]);
+                if (last)
+                    umma_commit(&accfull[2 * set]);
+                if constexpr (C::B2 > 0) {
+                    if (first && P >= NACC &&
+                        !mbar_wait(&accempty[2 * set + 1], (uint32_t)(P / NACC - 1) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+    #pragma unroll
+                    for (int ks = 0; ks < kNTE / 16; ++ks) {
+                        const uint32_t a = jb + row2 + (uint32_t)ks * 32;
+                        umma_bf16(acc2, dK + (a >> 4), dK + (a >> 4), id2, (first && ks == 0) ? 0u : 1u);
+                    }
+                }
+                // on completion the digit buffer is free again
+                umma_commit(&jempty[b]);
+                if (C::B2 > 0 && last)
+                    umma_commit(&accfull[2 * set + 1]);
             }
             umma_commit(&g_done);
             // tensor memory is released only after every product has finished
@@ -298,101 +366,112 @@ __global__ void __launch_bounds__(kNThreads, 1)
             if (!ok)
                 flags |= FLAG_TIMEOUT;
         }
-    } else if (warp >= kNFirstDrain && warp < kNFirstDrain + kNDrain) {
+    } else if (warp < kNFirstCons) {
         // ---- drain: lane quarter q, rows m = 32 q + lane, columns half h ----
-        // Row m < 3R is digit s = m / R + 1 of row p = m % R. T1 sums the
-        // blocks t = 1..3 (columns (t - 1) R ...), T2 the blocks t = 4, 5.
+        // Row m holds row p = m % R of digit m / R of each MMA's A operand;
+        // block t of an accumulator is columns t R ... of it. Blocks whose
+        // transpose is among the products too count half (T/2): t < S1 of the
+        // first MMA, the A digits' own of the second.
         const int q = warp & 3, h = (warp - kNFirstDrain) >> 2, m = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         constexpr int HC = NW / 2;  // packed column pairs per thread and block (NW columns)
-        f2 h1[HC], l1[HC], h2[HC], l2[HC];
+        constexpr int CH = NW <= 24 ? NW : 16;  // columns read at a time
+        const f2 HALF = pk2(0.5f, 0.5f);
+        // B2 = 1: D_44 counts half, D_54 (rows of the second A digit) in full
+        const float w54 = m < R ? 0.5f : 1.0f;
+        const f2 W54 = pk2(w54, w54);
+        // (wh, wl): the first MMA's blocks; w2: the second's, below 2^-32 of the
+        // leading one (2^-48 for B2 = 1), whose FP32 roundings are below 2^-56.
+        // Added to (wh, wl) they would fall below its last bit, one-sidedly.
+        f2 wh[HC], wl[HC], w2[C::B2 > 0 ? HC : 1];
 #pragma unroll
         for (int c = 0; c < HC; ++c)
-            h1[c] = l1[c] = h2[c] = l2[c] = 0ull;
+            wh[c] = wl[c] = 0ull;
+#pragma unroll
+        for (int c = 0; c < (C::B2 > 0 ? HC : 1); ++c)
+            w2[c] = 0ull;
         const int n_periods = (n_my + kNPeriod - 1) / kNPeriod;
-        for (int P = 0; P < n_periods; ++P) {
-            const int ab = P & 1;
-            if (!mbar_wait(&accfull[ab], (uint32_t)(P >> 1) & 1)) {
-                flags |= FLAG_TIMEOUT;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t acc = tmem + lane_addr + (uint32_t)ab * C::ACC1 + (uint32_t)(h * NW);
+        bool ok = true;
+        for (int P = 0; P < n_periods && ok; ++P) {
+            const int set = P % NACC;
 #pragma unroll
-            for (int t = 1; t <= kNDigits; ++t) {
-                uint32_t v[NW];
-                tmem_row_half<NW>(acc + (uint32_t)((t - 1) * R), v);
-                tmem_ld_wait();
-                if (t == kNDigits) {
-                    // every column is in registers: the accumulator may be reused
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0)
-                        mbar_arrive(&accempty[ab]);
+            for (int half = 0; half < (C::B2 > 0 ? 2 : 1); ++half) {
+                if (!mbar_wait(&accfull[2 * set + half], (uint32_t)(P / NACC) & 1)) {
+                    flags |= FLAG_TIMEOUT;
+                    ok = false;
+                    break;
                 }
+                tc_fence_after();
+                const uint32_t acc = tmem + lane_addr + (uint32_t)set * (C::N1 + C::N2) +
+                                     (half ? (uint32_t)C::N1 : 0u) + (uint32_t)(h * NW);
+                const int n_blocks = half ? C::B2 : kNDigits;
 #pragma unroll
-                for (int c = 0; c < HC; ++c) {
-                    const f2 x = pk2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
-                    if (t <= 3)
-                        two_sum2(h1[c], l1[c], x);
-                    else
-                        two_sum2(h2[c], l2[c], x);
+                for (int t = 0; t < n_blocks; ++t) {
+#pragma unroll
+                    for (int c0 = 0; c0 < NW; c0 += CH) {
+                        uint32_t v[CH];
+                        tmem_row_half<CH>(acc + (uint32_t)(t * R + c0), v);
+                        tmem_ld_wait();
+                        if (t == n_blocks - 1 && c0 + CH == NW) {
+                            // every column is in registers: the accumulator may be reused
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0)
+                                mbar_arrive(&accempty[2 * set + half]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < CH / 2; ++i) {
+                            const int c = c0 / 2 + i;
+                            const f2 x = pk2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                            if (half == 0)
+                                two_sum2(wh[c], wl[c], t < S1 ? mul2(x, HALF) : x);
+                            else if (C::B2 == 1)
+                                w2[c] = fma2(x, W54, w2[c]);
+                            else
+                                w2[c] = t < 2 ? fma2(x, HALF, w2[c]) : add2(w2[c], x);
+                        }
+                    }
                 }
             }
         }
         // ---- this CTA's share of M -----------------------------------------
-        // T[s][p][q] = sum_{t <= 5} D_st[p][q], U[s][p][q] = sum_{t = 4, 5}
-        // D_st[p][q] (s <= 3) and X[s - 4][p][q] = D_s4[p][q] (s = 4, 5) go
-        // through shared memory (the digit buffers are free once the last
-        // period is drained: every MMA has completed); then
-        //   G[p][q] = sum_s T[s][p][q] + sum_s U[s][q][p]
-        //           + X[0][p][q] + X[1][p][q] + X[1][q][p].
-        double *Ts = reinterpret_cast<double *>(base);
-        double *Us = Ts + 3 * R * R;
-        double *Xs = Us + 3 * R * R;
-        if (m < 3 * R) {
+        // W goes through shared memory (the digit buffers are free once the
+        // last period is drained: every MMA has completed); then G[p][q] =
+        // sum over the digit rows d < S1 of W[dR + p][q] + W[dR + q][p].
+        double *Ws = reinterpret_cast<double *>(base);
+        if (m < S1 * R) {
 #pragma unroll
             for (int c = 0; c < HC; ++c) {
-                float a0, a1, b0, b1, c0, c1, d0, d1;
-                upk2(h1[c], a0, a1);
-                upk2(l1[c], b0, b1);
-                upk2(h2[c], c0, c1);
-                upk2(l2[c], d0, d1);
-                const int col = h * NW + 2 * c;
-                const double u0 = (double)c0 + (double)d0, u1 = (double)c1 + (double)d1;
-                Ts[m * R + col] = ((double)a0 + (double)b0) + u0;
-                Ts[m * R + col + 1] = ((double)a1 + (double)b1) + u1;
-                Us[m * R + col] = u0;
-                Us[m * R + col + 1] = u1;
-            }
-        }
-        {
-            // the small blocks, accumulated over the whole launch
-            uint32_t v[NW];
-            tmem_row_half<NW>(tmem + lane_addr + C::ACCX + (uint32_t)(h * NW), v);
-            tmem_ld_wait();
-            if (m < 2 * R) {
-#pragma unroll
-                for (int c = 0; c < NW; ++c)
-                    Xs[m * R + h * NW + c] = (double)__uint_as_float(v[c]);
+                float a0, a1, b0, b1;
+                upk2(wh[c], a0, a1);
+                upk2(wl[c], b0, b1);
+                double x0 = (double)a0 + (double)b0, x1 = (double)a1 + (double)b1;
+                if (C::B2 > 0 && m < 2 * R) {
+                    float d0, d1;
+                    upk2(w2[C::B2 > 0 ? c : 0], d0, d1);
+                    x0 += (double)d0;
+                    x1 += (double)d1;
+                }
+                Ws[m * R + h * NW + 2 * c] = x0;
+                Ws[m * R + h * NW + 2 * c + 1] = x1;
             }
         }
         asm volatile("bar.sync 1, %0;" ::"r"(kNDrain * 32) : "memory");
-        // entries e of the upper triangle (a <= b) of M, real and imaginary parts
-        const int E = n_waves * (n_waves + 1) / 2;
+        // entries e of the upper triangle (a <= b) of the local waves, real and imaginary parts
+        const int nl = blocks.local(), E = nl * (nl + 1) / 2;
         for (int ec = (warp - kNFirstDrain) * 32 + lane; ec < 2 * E; ec += kNDrain * 32) {
             const int e = ec >> 1, comp = ec & 1;
             int a = 0, o = e;
-            while (o >= n_waves - a) {
-                o -= n_waves - a;
+            while (o >= nl - a) {
+                o -= nl - a;
                 ++a;
             }
             const int b = a + o;
             auto G = [&](int p, int r) {
-                double v = Xs[p * R + r] + (Xs[(R + p) * R + r] + Xs[(R + r) * R + p]);
+                double v = 0.0;
 #pragma unroll
-                for (int d = 0; d < 3; ++d)
-                    v += Ts[(d * R + p) * R + r] + Us[(d * R + r) * R + p];
+                for (int d = 0; d < S1; ++d)
+                    v += Ws[(d * R + p) * R + r] + Ws[(d * R + r) * R + p];
                 return v;
             };
             const double v = comp == 0 ? G(2 * a, 2 * b) + G(2 * a + 1, 2 * b + 1)
@@ -400,51 +479,69 @@ __global__ void __launch_bounds__(kNThreads, 1)
             part[(size_t)ec * gridDim.x + blockIdx.x] = v;
         }
     } else {
-        // ---- consumers: warp c takes tiles j = c, c + kNCons, ... ----------
-        const int c = consumer_index(warp);
-        const uint32_t jb = jbase + (uint32_t)c * C::JBYTES;
-        const uint32_t cb = (uint32_t)lane * 4;  // this lane's events 2 lane, 2 lane + 1
-        const f2 STEP = pk2(0x1p-8f, 0x1p-8f);
-        for (int j = c; j < n_my; j += kNCons) {
-            const int st = stage_of(j);
-            if (!mbar_wait(&full[st], use_of(j) & 1)) {
+        // ---- consumers: group g takes tiles j = g, g + GROUPS, ... ----------
+        // A half warp holds one row of the tile (four events a lane); warp w of
+        // the group takes row pairs w, w + WPG, ...
+        const int cw = warp - kNFirstCons, g = cw / C::WPG, wg = cw % C::WPG;
+        const int half = lane >> 4, l16 = lane & 15;
+        for (int j = g; j < n_my; j += C::GROUPS) {
+            const int st = j % STAGES, b = j % NBUF, k = j / NBUF;
+            if (!mbar_wait(&full[st], (uint32_t)(j / STAGES) & 1)) {
                 flags |= FLAG_TIMEOUT;
                 break;
             }
-            const float *T = stages + (size_t)st * (C::STAGE_BYTES / 4) + 2 * lane;
-            f2 x[R];
+            const float *T = stages + (size_t)st * (C::STAGE_BYTES / 4) + 4 * l16;
+            float4 xs[C::ITERS];
 #pragma unroll
-            for (int p = 0; p < R; ++p)
-                x[p] = lds2_f2(T + p * kNTE);
+            for (int it = 0; it < C::ITERS; ++it) {
+                const int rp = wg + it * C::WPG;
+                if (rp < NW)
+                    xs[it] = *reinterpret_cast<const float4 *>(T + (2 * rp + half) * kNTE);
+            }
             // the amplitudes are in registers: the stage may be refilled
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(&empty[st]);
-            // this warp's buffer is free once the products of its previous tile are done
-            const int k = j / kNCons;
-            if (k > 0 && !mbar_wait(&jempty[c], (uint32_t)(k - 1) & 1)) {
+            // the buffer is free once the products of its previous tile are done
+            if (k > 0 && !mbar_wait(&jempty[b], (uint32_t)(k - 1) & 1)) {
                 flags |= FLAG_TIMEOUT;
                 break;
             }
+            const uint32_t jb = jbase + (uint32_t)b * C::JBYTES;
 #pragma unroll
-            for (int p = 0; p < R; ++p) {
-                f2 z = x[p];
-                f2 S = pk2(s_sig[p], s_sig[p]);
+            for (int it = 0; it < C::ITERS; ++it) {
+                const int rp = wg + it * C::WPG;
+                if (rp < NW) {
+                    const int p = 2 * rp + half;
+                    const float sig = s_sig[p];
+                    const f2 S0 = pk2(sig, sig);
+                    f2 z0 = pk2(xs[it].x, xs[it].y), z1 = pk2(xs[it].z, xs[it].w);
+                    const uint32_t dst = jb + sw128(p, (uint32_t)l16 * 8);
+                    float step = 1.0f;
 #pragma unroll
-                for (int d = 0; d < kNDigits; ++d) {
-                    const f2 t = sub2(add2(z, S), S);  // z rounded to a multiple of 2^(r - 8(d+1))
-                    z = sub2(z, t);                    // exact remainder
-                    float t0, t1;
-                    upk2(t, t0, t1);
-                    st_shared_u32(jb + sw128(d * R + p, cb), to_bf16x2(t0, t1));
-                    S = mul2(S, STEP);
+                    for (int d = 0; d < kNDigits; ++d) {
+                        // z rounded to a multiple of 2^(r - 8(d+1)): z + S - S with S =
+                        // S0 2^-8d (the products by powers of two are exact), and the
+                        // exact remainder
+                        const f2 up = pk2(step, step), dn = pk2(-step, -step);
+                        const f2 t0 = fma2(S0, dn, fma2(S0, up, z0));
+                        const f2 t1 = fma2(S0, dn, fma2(S0, up, z1));
+                        z0 = sub2(z0, t0);
+                        z1 = sub2(z1, t1);
+                        float a0, a1, a2, a3;
+                        upk2(t0, a0, a1);
+                        upk2(t1, a2, a3);
+                        st_shared_v2(dst + (uint32_t)(d * R) * 128u, to_bf16x2(a0, a1),
+                                     to_bf16x2(a2, a3));
+                        step *= 0x1p-8f;
+                    }
                 }
             }
             // generic-proxy writes become visible to the tensor core, then signal
             fence_async_smem();
             __syncwarp();
             if (lane == 0)
-                mbar_arrive(&jfull[c]);
+                mbar_arrive(&jfull[b]);
         }
     }
     if (flags)
@@ -459,24 +556,27 @@ __global__ void __launch_bounds__(kNThreads, 1)
     }
 }
 
-// M from the CTAs' shares: one warp per (entry, part) of the upper triangle;
-// lane k adds CTAs k, k + 32, ... (all loads issued first), then a fixed
-// shuffle tree; divided by N_gen, written to (a, b) and conjugated to (b, a),
-// the diagonal's imaginary part zero. With a timeout flagged, M is NaN.
-__global__ void norm_tc_finalize(const double *__restrict__ part, int grid, int N, double n_gen,
-                                 const int *status, double *__restrict__ M)
+// M from the CTAs' shares: one warp per (entry, part) of the launch's upper
+// triangle; lane k adds CTAs k, k + 32, ... (all loads issued first), then a
+// fixed shuffle tree; divided by N_gen, written to (a, b) and conjugated to
+// (b, a), the diagonal's imaginary part zero. With a timeout flagged, M is NaN.
+__global__ void norm_tc_finalize(const double *__restrict__ part, int grid, int N,
+                                 NormBlocks blocks, double n_gen, const int *status,
+                                 double *__restrict__ M)
 {
     const int ec = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int E = N * (N + 1) / 2;
+    const int nl = blocks.local(), E = nl * (nl + 1) / 2;
     if (ec >= 2 * E)
         return;
     const int e = ec >> 1, comp = ec & 1;
-    int a = 0, o = e;
-    while (o >= N - a) {
-        o -= N - a;
-        ++a;
+    int la = 0, o = e;
+    while (o >= nl - la) {
+        o -= nl - la;
+        ++la;
     }
-    const int b = a + o;
+    const int a = blocks.global(la), b = blocks.global(la + o);
+    if (a >= N || b >= N)
+        return;
     const double *pe = part + (size_t)ec * grid;
     double x[kNFinMaxRounds];
 #pragma unroll
@@ -503,8 +603,9 @@ __global__ void norm_tc_finalize(const double *__restrict__ part, int grid, int 
 }
 
 template <int NW>
-cudaError_t norm_tc_nw(const CUtensorMap *map, const Planes &mc, const float *amax, double n_gen,
-                       double *part, int grid, int *status, double *M, cudaStream_t s)
+cudaError_t norm_tc_nw(const CUtensorMap *map, const Planes &mc, const NormBlocks &blocks,
+                       const float *amax, double n_gen, double *part, int grid, int *status,
+                       double *M, cudaStream_t s)
 {
     using C = NormTcCfg<NW>;
     const int n_tiles = (int)((mc.n + kNTE - 1) / kNTE);
@@ -516,28 +617,45 @@ cudaError_t norm_tc_nw(const CUtensorMap *map, const Planes &mc, const float *am
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess)
         return e;
-    norm_tc_kernel<NW><<<grid, kNThreads, C::SMEM, s>>>(*map, amax, mc.n_waves, n_tiles, part,
-                                                        status);
+    norm_tc_kernel<NW><<<grid, kNThreads, C::SMEM, s>>>(*map, amax, mc.n_waves, blocks, n_tiles,
+                                                        part, status);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    const int E2 = mc.n_waves * (mc.n_waves + 1);
-    norm_tc_finalize<<<(E2 + 7) / 8, 256, 0, s>>>(part, grid, mc.n_waves, n_gen, status, M);
+    const int E2 = blocks.local() * (blocks.local() + 1);
+    norm_tc_finalize<<<(E2 + 7) / 8, 256, 0, s>>>(part, grid, mc.n_waves, blocks, n_gen, status, M);
     return cudaGetLastError();
 }
 
-int norm_tc_nw_of(int n_waves)
+// waves per block: all of them in one launch, or a third
+int norm_tc_block(int n_waves) { return n_waves <= kNMaxOnePass ? n_waves : (n_waves + 2) / 3; }
+
+cudaError_t norm_tc_pass(const CUtensorMap *map, const Planes &mc, const NormBlocks &blocks,
+                         const float *amax, double n_gen, double *part, int grid, int *status,
+                         double *M, cudaStream_t s)
 {
-    for (int p : {4, 8, 12, 16, 20})
-        if (n_waves <= p)
-            return p;
-    return -1;
+    const int n = blocks.local();
+    if (n <= 4)
+        return norm_tc_nw<4>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    if (n <= 8)
+        return norm_tc_nw<8>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    if (n <= 12)
+        return norm_tc_nw<12>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    if (n <= 16)
+        return norm_tc_nw<16>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    if (n <= 20)
+        return norm_tc_nw<20>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    if (n <= 24)
+        return norm_tc_nw<24>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
+    return norm_tc_nw<32>(map, mc, blocks, amax, n_gen, part, grid, status, M, s);
 }
 
 }  // namespace
 
-bool norm_tc_available(int n_waves) { return n_waves >= 1 && norm_tc_nw_of(n_waves) > 0; }
+bool norm_tc_available(int n_waves) { return n_waves >= 1 && n_waves <= kMaxWaves; }
 
 int norm_tc_box_events() { return kNTE; }
+
+int norm_tc_box_rows(int n_waves) { return 2 * norm_tc_block(n_waves); }
 
 bool norm_tc_scale_ok(float amax)
 {
@@ -548,23 +666,28 @@ bool norm_tc_scale_ok(float amax)
 
 size_t norm_tc_partials_doubles(int n_waves, int grid)
 {
-    return (size_t)grid * n_waves * (n_waves + 1);
+    const int n = n_waves <= kNMaxOnePass ? n_waves : 2 * norm_tc_block(n_waves);
+    return (size_t)grid * n * (n + 1);
 }
 
 cudaError_t launch_build_norm_tc(const CUtensorMap *map, const Planes &mc, const float *amax,
                                  double n_gen, double *partials, int grid, int *status, double *M,
                                  cudaStream_t s)
 {
-    if (mc.n < 1)
+    if (mc.n < 1 || !norm_tc_available(mc.n_waves))
         return cudaErrorInvalidValue;
-    switch (norm_tc_nw_of(mc.n_waves)) {
-    case 4: return norm_tc_nw<4>(map, mc, amax, n_gen, partials, grid, status, M, s);
-    case 8: return norm_tc_nw<8>(map, mc, amax, n_gen, partials, grid, status, M, s);
-    case 12: return norm_tc_nw<12>(map, mc, amax, n_gen, partials, grid, status, M, s);
-    case 16: return norm_tc_nw<16>(map, mc, amax, n_gen, partials, grid, status, M, s);
-    case 20: return norm_tc_nw<20>(map, mc, amax, n_gen, partials, grid, status, M, s);
-    default: return cudaErrorNotSupported;
-    }
+    const int blk = norm_tc_block(mc.n_waves);
+    if (blk == mc.n_waves)
+        return norm_tc_pass(map, mc, NormBlocks{1, blk, {0, 0}}, amax, n_gen, partials, grid, status,
+                            M, s);
+    for (int i = 0; i < 3; ++i)
+        for (int k = i + 1; k < 3; ++k) {
+            const cudaError_t e = norm_tc_pass(map, mc, NormBlocks{2, blk, {i * blk, k * blk}}, amax,
+                                               n_gen, partials, grid, status, M, s);
+            if (e != cudaSuccess)
+                return e;
+        }
+    return cudaSuccess;
 }
 
 }  // namespace pwa

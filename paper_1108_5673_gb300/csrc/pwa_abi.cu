@@ -1684,8 +1684,8 @@ int pwa_build_norm(pwa_ctx *c, double *M_out)
     if (!c->loaded)
         return fail(c, PWA_ESTATE, "pwa_load_events must come first");
     DeviceGuard g(c->device);
-    // The tensor-core kernel serves up to 20 waves when every wave's scale is
-    // in its range; the FP64 kernel everything else (or PWA_NORM_KERNEL=fp64).
+    // The tensor-core kernel when every wave's scale is in its range; the FP64
+    // kernel everything else (or PWA_NORM_KERNEL=fp64).
     bool tc = norm_tc_available(c->N);
     if (const char *v = getenv("PWA_NORM_KERNEL"))
         if (strcmp(v, "fp64") == 0)
@@ -1699,7 +1699,7 @@ int pwa_build_norm(pwa_ctx *c, double *M_out)
     if (tc) {
         CUtensorMap map;
         CK(c, encode_planes_map(&map, c->mc.ptr, c->mc.n, c->mc.pitch, 2 * c->N,
-                                norm_tc_box_events(), 2 * c->N));
+                                norm_tc_box_events(), norm_tc_box_rows(c->N)));
         const int grid = c->num_sms;
         const size_t nd = norm_tc_partials_doubles(c->N, grid);
         double *scratch = nullptr;
