@@ -1268,15 +1268,11 @@ static int finish_load(pwa_ctx *c, int rc, int64_t n_data, int64_t n_mc_acc, dou
 
 // ---- amplitudes on the device --------------------------------------------
 
-// Checks the wave list and converts it (with N_lm) into the device table at
-// *d_waves (allocated here, freed by the caller); *max_m = max |m|.
-static int upload_waves(pwa_ctx *c, const pwa_wave *waves, GenWave **d_waves, int *max_m)
+// Checks the wave list and builds the generator's table.
+static int check_waves(pwa_ctx *c, const pwa_wave *waves, GenTable *table)
 {
-    *d_waves = nullptr;
     if (!waves)
         return fail(c, PWA_EINVAL, "null wave list");
-    std::vector<GenWave> h(c->N);
-    *max_m = 0;
     for (int a = 0; a < c->N; ++a) {
         const pwa_wave &w = waves[a];
         const int am = w.m < 0 ? -w.m : w.m;
@@ -1285,26 +1281,16 @@ static int upload_waves(pwa_ctx *c, const pwa_wave *waves, GenWave **d_waves, in
                         w.m, ampgen_max_l());
         if (!(w.mass > 0) || !(w.width > 0) || !std::isfinite(w.mass) || !std::isfinite(w.width))
             return fail(c, PWA_EINVAL, "wave %d: mass and width must be positive and finite", a);
-        double ratio = 1.0;  // (l - |m|)! / (l + |m|)!
-        for (int k = w.l - am + 1; k <= w.l + am; ++k)
-            ratio /= k;
-        h[a] = GenWave{w.mass, w.width, std::sqrt((2.0 * w.l + 1.0) / (4.0 * 3.14159265358979323846) * ratio),
-                       w.l, w.m};
-        *max_m = std::max(*max_m, am);
     }
-    int rc = dev_alloc(c, (void **)d_waves, c->N * sizeof(GenWave), "wave table");
-    if (rc)
-        return rc;
-    CK(c, cudaMemcpyAsync(*d_waves, h.data(), c->N * sizeof(GenWave), cudaMemcpyHostToDevice,
-                          c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
+    ampgen_table(waves, c->N, table);
     return PWA_OK;
 }
 
 // Generates the amplitudes of n events (kin host or device) into `out`
 // (device): SoA planes of `pitch` floats, or event-major complex64.
-static int generate(pwa_ctx *c, const GenWave *d_waves, int max_m, const double *kin, int64_t n,
-                    float *out, bool soa, int64_t pitch)
+// PWA_AMPGEN_KERNEL=fp64 evaluates everything in FP64.
+static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_t n, float *out,
+                    bool soa, int64_t pitch)
 {
     const double *dk = kin;
     double *staging = nullptr;
@@ -1324,8 +1310,9 @@ static int generate(pwa_ctx *c, const GenWave *d_waves, int max_m, const double 
         }
         dk = staging;
     }
-    cudaError_t e = launch_amp_gen(dk, n, c->N, d_waves, max_m, out, soa, pitch, c->num_sms * 8,
-                                   c->stream);
+    const char *kv = getenv("PWA_AMPGEN_KERNEL");
+    cudaError_t e = launch_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, soa,
+                                   pitch, c->num_sms, c->stream);
     cudaError_t e2 = cudaStreamSynchronize(c->stream);
     if (staging)
         cudaFree(staging);
@@ -1348,19 +1335,16 @@ int pwa_compute_amplitudes(pwa_ctx *c, const pwa_wave *waves, const double *kin,
     if (n < 1 || n > ((int64_t)1 << 31) - 1024)
         return fail(c, PWA_EINVAL, "n=%lld outside [1, 2^31 - 1024]", (long long)n);
     DeviceGuard g(c->device);
-    GenWave *dw;
-    int max_m;
-    int rc = upload_waves(c, waves, &dw, &max_m);
-    if (rc) {
-        dev_free(dw);
+    GenTable table{};
+    int rc = check_waves(c, waves, &table);
+    if (rc)
         return rc;
-    }
     const bool on_dev = is_device_pointer(out);
     float *dout = static_cast<float *>(out);
     if (!on_dev)
         rc = dev_alloc(c, (void **)&dout, (size_t)n * c->N * 8, "amplitudes");
     if (!rc)
-        rc = generate(c, dw, max_m, kin, n, dout, false, 0);
+        rc = generate(c, table, kin, n, dout, false, 0);
     if (!rc && !on_dev) {
         cudaError_t e = cudaMemcpy(out, dout, (size_t)n * c->N * 8, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess)
@@ -1368,7 +1352,6 @@ int pwa_compute_amplitudes(pwa_ctx *c, const pwa_wave *waves, const double *kin,
     }
     if (!on_dev)
         dev_free(dout);
-    dev_free(dw);
     return rc;
 }
 
@@ -1390,13 +1373,10 @@ int pwa_load_events_generated(pwa_ctx *c, const pwa_wave *waves, const double *d
         return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events");
     DeviceGuard g(c->device);
     cudaStreamSynchronize(c->stream);
-    GenWave *dw;
-    int max_m;
-    int rc = upload_waves(c, waves, &dw, &max_m);
-    if (rc) {
-        dev_free(dw);
+    GenTable table{};
+    int rc = check_waves(c, waves, &table);
+    if (rc)
         return rc;
-    }
     free_sample(c);
     c->n_lambda = 1;
     const int N = c->N;
@@ -1411,9 +1391,8 @@ int pwa_load_events_generated(pwa_ctx *c, const pwa_wave *waves, const double *d
                        cudaSuccess)
             rc = fail(c, PWA_ECUDA, "memset");
         if (!rc)
-            rc = generate(c, dw, max_m, which == 0 ? data_kin : mc_kin, n, p.ptr, true, p.pitch);
+            rc = generate(c, table, which == 0 ? data_kin : mc_kin, n, p.ptr, true, p.pitch);
     }
-    dev_free(dw);
     return finish_load(c, rc, n_data, n_mc_acc, n_mc_gen);
 }
 

@@ -494,16 +494,37 @@ cudaError_t launch_nll_res_tma(const CUtensorMap *dmap, const CUtensorMap *mmap,
                                const float *amax, int grid, cudaStream_t s);
 
 // k_ampgen.cu: amplitudes BW(m; M, G) Y_l^m(theta, phi) from per-event
-// kinematics kin [n][3] = (m, cos theta, phi) (device), FP64, rounded to float;
-// out as SoA planes (Re A_a at plane 2a of `pitch` floats) or, soa = false,
-// event-major complex64 [n][N].
-struct GenWave {
+// kinematics kin [n][3] = (m, cos theta, phi) (device), each component the
+// float nearest to its FP64 value; out as SoA planes (Re A_a at plane 2a of
+// `pitch` floats) or, soa = false, event-major complex64 [n][N]. fp64_only
+// evaluates everything in FP64.
+struct alignas(16) GenPair {
+    float h0, h1, l0, l1;  // a float pair h + l, each twice (for two events)
+};
+struct alignas(16) GenWave {
+    GenPair m2, g, g2, nrm;    // M^2, +-M G, (M G)^2, +-norm (the signs of m < 0)
     double mass, width, norm;  // norm = sqrt((2l + 1)/(4 pi) (l - |m|)!/(l + |m|)!)
-    int l, m;
+    int l, m, index;  // index: the wave's place in the caller's list
+    int m_inc;        // a new |m|: by how much it grew; -1: the same |m|
+    int l_steps;      // recurrence steps in l before this wave
+    int new_y;        // (l, m) differs from the wave before
+    unsigned conj;    // sign bit: the imaginary part is negated (m < 0)
+};
+struct GenStep {
+    GenPair a, b;     // (2l - 1)/(l - m), (l + m - 1)/(l - m)
+};
+constexpr int kGenMaxSteps = 160;  // 16 + 15 + ... + 1 = 136 for every m up to 16
+struct GenTable {
+    GenWave w[kMaxWaves];  // in order of (|m|, l)
+    GenStep steps[kGenMaxSteps];
+    int n_steps;
+    int fp64_only;         // a mass or width outside the float-float range
 };
 int ampgen_max_l();
-cudaError_t launch_amp_gen(const double *kin, int64_t n, int N, const GenWave *waves, int max_m,
-                           float *out, bool soa, int64_t pitch, int grid, cudaStream_t s);
+// waves checked by the caller (0 <= |m| <= l <= ampgen_max_l())
+void ampgen_table(const pwa_wave *waves, int N, GenTable *table);
+cudaError_t launch_amp_gen(const double *kin, int64_t n, int N, const GenTable &table, bool fp64_only,
+                           float *out, bool soa, int64_t pitch, int num_sms, cudaStream_t s);
 
 // k_ampgen_cov.cu: covariant tensor amplitudes of J/psi -> gamma X, X -> K+ K-
 // from p3 [n][9] (photon, K+, K- 3-momenta, device), 4 incoherent components
