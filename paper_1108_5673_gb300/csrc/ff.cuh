@@ -6,11 +6,13 @@
 // value is a pair of events in packed FP32 (f2), so that one instruction
 // serves both.
 //
-// Error model: with |l| <= 2^-21 |h| in every operand, a product's relative
-// error is below 2^-42.4 (the dropped l l' and the roundings of the low part),
-// and a sum's absolute error is below 2^-44 (|a| + |b|). Products of the
-// high parts must stay above 2^-100 in size for the split to be exact; the
-// callers check their results against thresholds that ensure it.
+// Error model, relative to the operands' sizes: a product of normalised pairs
+// (|l| <= 2^-24 |h|) 2^-45.4 (the dropped l l' and the two roundings of the low
+// part), 2^-44.5 with one operand that is not (|l| <= 2^-22 |h|), 2^-43.7 with
+// both; a sum 2^-46.4 of |a| + |b|; a b +- c d 2^-44.5 of |a b| + |c d|; the
+// reciprocal and the square root 2^-45. Products of the high parts must stay
+// above 2^-100 in size for the split to be exact; the callers check their
+// results against thresholds that ensure it.
 #pragma once
 
 #include "pwa_internal.cuh"

@@ -14,7 +14,7 @@
 // and an event whose inputs leave the float-float range, go to a queue per
 // warp and are evaluated in FP64 a warp's worth at a time: one by one, by the
 // lane concerned, they took as long as the rest (1.35 ms in all). Measured at
-// 5M x 20: 0.70 ms (1.3 TB/s of the 0.92 GB), at 2M x 40 with l up to 10: 0.98
+// 5M x 20: 0.69 ms (1.3 TB/s of the 0.92 GB), at 2M x 40 with l up to 10: 0.98
 // ms against 7.6, at 5M x 4: 0.22 ms against 1.48; bound by instruction issue
 // (57% of the slots, most of the rest packed FP32 instructions that take two).
 //
@@ -99,7 +99,7 @@ __device__ __forceinline__ double reduce(double phi, int &k, bool &ok)
     return fma(-kd, 6.12323399573676588614e-17, r);
 }
 
-// e^{i phi} to 2^-42
+// e^{i phi} to 2^-43.5
 __device__ __forceinline__ void expi(double phi0, double phi1, ff &c, ff &s, bool &ok0, bool &ok1)
 {
     int k0, k1;
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kGenThreads, 4)
                 }
                 p1 = pmm;
                 p2 = ff_dup(0.f, 0.f);
-                e1 = mul2(dup2((float)am * 0x1p-41f), abs2(pmm.h));
+                e1 = mul2(dup2((float)am * 0x1p-43f), abs2(pmm.h));
                 e2 = 0ull;
             }
             for (int k = 0; k < W.l_steps; ++k, ++step) {
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kGenThreads, 4)
                 const ff xp = ff_norm(ff_mul(x, p1));
                 const ff u = ff_mul(sa, xp), v = ff_mul(sb, p2);
                 const ff sm = ff_two_diff(u.h, v.h);
-                const f2 eps = dup2(0x1p-41f);
+                const f2 eps = dup2(0x1p-43f);
                 const f2 ex = fma2(abs2(x.h), e1, mul2(eps, abs2(xp.h)));
                 const f2 eq = fma2(sa.h, ex, fma2(sb.h, e2, mul2(eps, abs2(v.h))));
                 p2 = p1;
@@ -250,9 +250,9 @@ __global__ void __launch_bounds__(kGenThreads, 4)
                 upk2(ay, a0, a1);
                 y0 = a0 >= 0x1p-60f && ok0;
                 y1 = a1 >= 0x1p-60f && ok1;
-                // the relative errors of the products (2^-40) and of e^{i m phi}
-                // (m 2^-41), and P's
-                y_err = fma2(ay, dup2(fmaf((float)am, 0x1p-41f, 0x1p-40f)),
+                // the relative errors of the products (2^-42.2 in all) and of
+                // e^{i m phi} (m 2^-42.7), and P's
+                y_err = fma2(ay, dup2(fmaf((float)am, 0x1p-42f, 0x1p-42f)),
                              mul2(mul2(dup2(1.001f), abs2(nrm.h)), e1));
             }
             // A = y (D + i G) e^{i m phi} / (D^2 + G^2); for m < 0 the conjugate of
@@ -334,13 +334,6 @@ __global__ void __launch_bounds__(kGenThreads, 4)
         drain(n);
 }
 
-// a double as the nearest float and the remainder
-GenPair pair_of(double x)
-{
-    const float h = (float)x, l = (float)(x - (double)h);
-    return {h, h, l, l};
-}
-
 }  // namespace
 
 int ampgen_max_l() { return kMaxL; }
@@ -381,16 +374,16 @@ void ampgen_table(const pwa_wave *waves, int N, GenTable *t)
         for (; cur_l < s.l; ++cur_l) {
             const int l = cur_l + 1;
             t->steps[t->n_steps++] =
-                GenStep{pair_of((2.0 * l - 1.0) / (l - am)), pair_of((l + am - 1.0) / (l - am))};
+                GenStep{gen_pair((2.0 * l - 1.0) / (l - am)), gen_pair((l + am - 1.0) / (l - am))};
         }
         const double g = s.mass * s.width;
         // scales whose squares would leave the float range in D^2 + G^2
         if (!(g * g >= 0x1p-80 && g * g <= 0x1p80 && s.mass * s.mass <= 0x1p60))
             t->fp64_only = 1;
-        w.m2 = pair_of(s.mass * s.mass);
-        w.g = pair_of(s.m < 0 ? -g : g);
-        w.g2 = pair_of(g * g);
-        w.nrm = pair_of(s.m < 0 && (am & 1) ? -w.norm : w.norm);
+        w.m2 = gen_pair(s.mass * s.mass);
+        w.g = gen_pair(s.m < 0 ? -g : g);
+        w.g2 = gen_pair(g * g);
+        w.nrm = gen_pair(s.m < 0 && (am & 1) ? -w.norm : w.norm);
         w.conj = s.m < 0 ? 0x80000000u : 0u;
         w.new_y = k == 0 || s.l != t->w[k - 1].l || s.m != t->w[k - 1].m;
     }

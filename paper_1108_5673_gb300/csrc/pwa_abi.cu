@@ -1398,33 +1398,28 @@ int pwa_load_events_generated(pwa_ctx *c, const pwa_wave *waves, const double *d
 
 // ---- covariant amplitudes ------------------------------------------------
 
-// Checks the covariant wave list and uploads it to *d_waves (freed by the caller).
-static int upload_cov_waves(pwa_ctx *c, const pwa_cov_wave *waves, CovWave **d_waves)
+// Checks the covariant wave list and builds the generator's table.
+static int check_cov_waves(pwa_ctx *c, const pwa_cov_wave *waves, CovTable *table)
 {
-    *d_waves = nullptr;
     if (!waves)
         return fail(c, PWA_EINVAL, "null wave list");
-    std::vector<CovWave> h(c->N);
     for (int a = 0; a < c->N; ++a) {
         const pwa_cov_wave &w = waves[a];
         if (w.spin != 0 && w.spin != 2)
             return fail(c, PWA_EINVAL, "wave %d: spin %d is neither 0 nor 2", a, w.spin);
         if (!(w.mass > 0) || !(w.width > 0) || !std::isfinite(w.mass) || !std::isfinite(w.width))
             return fail(c, PWA_EINVAL, "wave %d: mass and width must be positive and finite", a);
-        h[a] = CovWave{w.mass, w.width, w.spin};
     }
-    int rc = dev_alloc(c, (void **)d_waves, c->N * sizeof(CovWave), "wave table");
-    if (rc)
-        return rc;
-    CK(c, cudaMemcpyAsync(*d_waves, h.data(), c->N * sizeof(CovWave), cudaMemcpyHostToDevice,
-                          c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
+    cov_table(waves, c->N, table);
     return PWA_OK;
 }
 
-// Covariant amplitudes of n events (p3 host or device) into `out` (device,
-// event-major [n][4][N] complex64).
-static int generate_cov(pwa_ctx *c, const CovWave *d_waves, const double *p3, int64_t n, float *out)
+// Covariant amplitudes of n events (p3 host or device) into `out` (device) in
+// the layout `mode`, their maxima into amax (may be null, zeroed). Returns
+// after the kernel has finished. PWA_AMPGEN_KERNEL=fp64 evaluates everything
+// in FP64.
+static int generate_cov(pwa_ctx *c, const CovTable &table, const double *p3, int64_t n, float *out,
+                        int mode, int64_t pitch, float *amax)
 {
     const double *dk = p3;
     double *staging = nullptr;
@@ -1444,7 +1439,9 @@ static int generate_cov(pwa_ctx *c, const CovWave *d_waves, const double *p3, in
         }
         dk = staging;
     }
-    cudaError_t e = launch_cov_amp_gen(dk, n, c->N, d_waves, out, false, 0, c->num_sms * 8, c->stream);
+    const char *kv = getenv("PWA_AMPGEN_KERNEL");
+    cudaError_t e = launch_cov_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, mode,
+                                       pitch, amax, c->num_sms, c->stream);
     cudaError_t e2 = cudaStreamSynchronize(c->stream);
     if (staging)
         cudaFree(staging);
@@ -1467,19 +1464,17 @@ int pwa_compute_covariant_amplitudes(pwa_ctx *c, const pwa_cov_wave *waves, cons
     if (n < 1 || n > ((int64_t)1 << 31) - 1024)
         return fail(c, PWA_EINVAL, "n=%lld outside [1, 2^31 - 1024]", (long long)n);
     DeviceGuard g(c->device);
-    CovWave *dw;
-    int rc = upload_cov_waves(c, waves, &dw);
-    if (rc) {
-        dev_free(dw);
+    CovTable table{};
+    int rc = check_cov_waves(c, waves, &table);
+    if (rc)
         return rc;
-    }
     const size_t bytes = (size_t)n * 4 * c->N * 8;
     const bool on_dev = is_device_pointer(out);
     float *dout = static_cast<float *>(out);
     if (!on_dev)
         rc = dev_alloc(c, (void **)&dout, bytes, "amplitudes");
     if (!rc)
-        rc = generate_cov(c, dw, p3, n, dout);
+        rc = generate_cov(c, table, p3, n, dout, kCovEventMajor, 0, nullptr);
     if (!rc && !on_dev) {
         cudaError_t e = cudaMemcpy(out, dout, bytes, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess)
@@ -1487,91 +1482,50 @@ int pwa_compute_covariant_amplitudes(pwa_ctx *c, const pwa_cov_wave *waves, cons
     }
     if (!on_dev)
         dev_free(dout);
-    dev_free(dw);
     return rc;
 }
 
-// The amplitudes of both samples go through device buffers of this call into
-// the incoherent loader (which copies them into its planes), so that every
-// check and store that loader makes applies unchanged.
-int pwa_load_events_covariant(pwa_ctx *c, const pwa_cov_wave *waves, const double *data_p3,
-                              int64_t n_data, const double *mc_p3, int64_t n_mc_acc,
-                              double n_mc_gen)
-{
-    if (!c)
-        return PWA_EINVAL;
-    if (!data_p3 || !mc_p3)
-        return fail(c, PWA_EINVAL, "null momenta");
-    if (n_data < 1 || n_mc_acc < 1)
-        return fail(c, PWA_EINVAL, "n_data=%lld and n_mc_acc=%lld must be >= 1",
-                    (long long)n_data, (long long)n_mc_acc);
-    if (n_data > ((int64_t)1 << 31) - 1024 || n_mc_acc * 4 > ((int64_t)1 << 31) - 1024)
-        return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events (MC: 4 x events)");
-    DeviceGuard g(c->device);
-    CovWave *dw;
-    int rc = upload_cov_waves(c, waves, &dw);
-    float *amp[2] = {nullptr, nullptr};
-    const int64_t n[2] = {n_data, n_mc_acc};
-    for (int k = 0; k < 2 && !rc; ++k) {
-        rc = dev_alloc(c, (void **)&amp[k], (size_t)n[k] * 4 * c->N * 8, "amplitudes");
-        if (!rc)
-            rc = generate_cov(c, dw, k == 0 ? data_p3 : mc_p3, n[k], amp[k]);
-    }
-    dev_free(dw);
-    if (!rc)
-        rc = pwa_load_events_incoherent(c, 4, amp[0], n_data, amp[1], n_mc_acc, n_mc_gen, PWA_C64);
-    cudaStreamSynchronize(c->stream);
-    dev_free(amp[0]);
-    dev_free(amp[1]);
-    return rc;
-}
+}  // extern "C"
 
-int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, int64_t n_data,
-                               const void *mc_amp, int64_t n_mc_acc, double n_mc_gen,
-                               int amp_dtype)
+// An incoherent sample of L components: checks, stores, maxima and tensor maps
+// around `fill`, which writes the amplitudes. fill(mc, planes, amax): mc false,
+// the data planes (plane 2 (l N + a) = Re A_a^l); mc true, n_mc_acc L pseudo-
+// events of N waves, so that M sums the products over components as well as
+// over events. It may leave the maxima of |Re| + |Im| per wave in amax (zeroed,
+// [N]) and then returns them as done through *have_max.
+template <typename Fill>
+static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, double n_mc_gen,
+                           Fill fill)
 {
-    if (!c)
-        return PWA_EINVAL;
-    if (n_lambda == 1)
-        return pwa_load_events(c, data_amp, n_data, mc_amp, n_mc_acc, n_mc_gen, amp_dtype);
-    if (n_lambda < 1 || n_lambda > incoh_max_components())
-        return fail(c, PWA_EINVAL, "n_lambda=%d outside [1, %d]", n_lambda, incoh_max_components());
-    if (!data_amp || !mc_amp)
-        return fail(c, PWA_EINVAL, "null amplitude pointer");
-    if (n_data < 1 || n_mc_acc < 1)
-        return fail(c, PWA_EINVAL, "n_data=%lld and n_mc_acc=%lld must be >= 1",
-                    (long long)n_data, (long long)n_mc_acc);
+    const int N = c->N;
     if (!(n_mc_gen >= (double)n_mc_acc))
         return fail(c, PWA_EINVAL, "n_mc_gen=%g must be >= n_mc_acc=%lld", n_mc_gen,
                     (long long)n_mc_acc);
-    if (amp_dtype != PWA_C64 && amp_dtype != PWA_C128)
-        return fail(c, PWA_EINVAL, "amp_dtype=%d is neither PWA_C64 nor PWA_C128", amp_dtype);
-    if (n_data > ((int64_t)1 << 31) - 1024 || n_mc_acc * n_lambda > ((int64_t)1 << 31) - 1024)
-        return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events (MC: events x n_lambda)");
     if (c->cfg.forms & PWA_FORM_TC)
         return fail(c, PWA_ENOTSUP, "the tensor-core form takes coherent samples only");
-    if ((c->cfg.forms & PWA_FORM_AMP) && c->N > incoh_max_waves(n_lambda))
+    if ((c->cfg.forms & PWA_FORM_AMP) && N > incoh_max_waves(L))
         return fail(c, PWA_ENOTSUP, "the direct form takes up to %d waves at n_lambda=%d",
-                    incoh_max_waves(n_lambda), n_lambda);
+                    incoh_max_waves(L), L);
     DeviceGuard g(c->device);
     cudaStreamSynchronize(c->stream);
     free_sample(c);
-    const int N = c->N, L = n_lambda;
-    // data: [n][L][N] complex = n events of L N waves, plane 2 (l N + a) = Re A_a^l
-    Planes &d = c->data;
-    d.n = n_data;
-    d.n_waves = L * N;
-    d.pitch = round_up(n_data, 256);
-    int rc = dev_alloc(c, (void **)&d.ptr, (size_t)2 * L * N * d.pitch * sizeof(float), "planes");
-    if (!rc && cudaMemsetAsync(d.ptr, 0, (size_t)2 * L * N * d.pitch * sizeof(float), c->stream) !=
-                   cudaSuccess)
-        rc = fail(c, PWA_ECUDA, "memset");
-    if (!rc)
-        rc = pack_rows(c, data_amp, n_data, amp_dtype, L * N, d.ptr, d.pitch);
-    // MC: the same bytes read as n L pseudo-events of N waves, so that M sums
-    // the products over components as well as over events
-    if (!rc)
-        rc = load_planes(c, mc_amp, n_mc_acc * L, amp_dtype, &c->mc);
+    int rc = PWA_OK;
+    bool have_max[2] = {false, false};
+    for (int mc = 0; mc < 2 && !rc; ++mc) {
+        Planes &d = mc ? c->mc : c->data;
+        float *amax = mc ? c->mc_amax : c->amax;
+        d.n = mc ? n_mc_acc * L : n_data;
+        d.n_waves = mc ? N : L * N;
+        d.pitch = round_up(d.n, 256);
+        const size_t bytes = (size_t)2 * d.n_waves * d.pitch * sizeof(float);
+        rc = dev_alloc(c, (void **)&d.ptr, bytes, "planes");
+        if (!rc && (cudaMemsetAsync(d.ptr, 0, bytes, c->stream) != cudaSuccess ||
+                    cudaMemsetAsync(amax, 0, N * sizeof(float), c->stream) != cudaSuccess))
+            rc = fail(c, PWA_ECUDA, "memset");
+        if (!rc)
+            rc = fill(mc != 0, d, amax, &have_max[mc]);
+    }
+    const Planes &d = c->data;
     if (!rc && (c->cfg.forms & PWA_FORM_TABLE)) {
         c->table_pitch = d.pitch;
         rc = dev_alloc(c, (void **)&c->table, (size_t)N * N * c->table_pitch * sizeof(float),
@@ -1599,14 +1553,10 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
     const char *kv = getenv("PWA_INCOH_KERNEL");
     const bool tma = (c->cfg.forms & PWA_FORM_AMP) && incoh_tma_available(N, L) &&
                      !(kv && strcmp(kv, "generic") == 0);
-    if (!rc && cudaMemsetAsync(c->amax, 0, N * sizeof(float), c->stream) != cudaSuccess)
-        rc = fail(c, PWA_ECUDA, "memset");
-    // the MC planes hold n_mc_acc L pseudo-events of N waves: their maxima
-    // scale the tensor-core build of M
-    if (!rc && (cudaMemsetAsync(c->mc_amax, 0, N * sizeof(float), c->stream) != cudaSuccess ||
-                launch_amp_max(c->mc, c->mc_amax, c->stream) != cudaSuccess))
+    // the maxima over the MC pseudo-events scale the tensor-core build of M
+    if (!rc && !have_max[1] && launch_amp_max(c->mc, c->mc_amax, c->stream) != cudaSuccess)
         rc = fail(c, PWA_ECUDA, "MC amplitude maxima");
-    if (!rc && tma) {
+    if (!rc && tma && !have_max[0]) {
         float *dmax = nullptr;
         rc = dev_alloc(c, (void **)&dmax, (size_t)L * N * sizeof(float), "component maxima");
         std::vector<float> hmax((size_t)L * N), amax(N, 0.f);
@@ -1626,9 +1576,6 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(c->amax, amax.data(), N * sizeof(float), cudaMemcpyHostToDevice,
                                     c->stream);
-            if (e == cudaSuccess)
-                e = encode_planes_map(&c->data_map, d.ptr, n_data, d.pitch, 2 * L * N,
-                                      incoh_tma_box_events(), 2 * L * N);
             if (e != cudaSuccess)
                 rc = fail(c, PWA_ECUDA, "incoherent direct-form set-up: %s", cudaGetErrorString(e));
         }
@@ -1636,6 +1583,12 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
             cudaStreamSynchronize(c->stream);
             cudaFree(dmax);
         }
+    }
+    if (!rc && tma) {
+        const cudaError_t e = encode_planes_map(&c->data_map, d.ptr, n_data, d.pitch, 2 * L * N,
+                                                incoh_tma_box_events(), 2 * L * N);
+        if (e != cudaSuccess)
+            rc = fail(c, PWA_ECUDA, "incoherent direct-form set-up: %s", cudaGetErrorString(e));
     }
     if (!rc) {
         cudaError_t e = cudaStreamSynchronize(c->stream);
@@ -1654,6 +1607,65 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
     c->loaded = true;
     c->has_norm = false;
     return PWA_OK;
+}
+
+extern "C" {
+
+// The amplitudes of both samples are generated straight into the planes that
+// the direct form and M read, with their maxima (an event-major copy, its
+// packing and a pass for the maxima took 1.0 of 6.4 ms at 1M + 2.5M events x
+// 12 waves).
+int pwa_load_events_covariant(pwa_ctx *c, const pwa_cov_wave *waves, const double *data_p3,
+                              int64_t n_data, const double *mc_p3, int64_t n_mc_acc,
+                              double n_mc_gen)
+{
+    if (!c)
+        return PWA_EINVAL;
+    if (!data_p3 || !mc_p3)
+        return fail(c, PWA_EINVAL, "null momenta");
+    if (n_data < 1 || n_mc_acc < 1)
+        return fail(c, PWA_EINVAL, "n_data=%lld and n_mc_acc=%lld must be >= 1",
+                    (long long)n_data, (long long)n_mc_acc);
+    if (n_data > ((int64_t)1 << 31) - 1024 || n_mc_acc * 4 > ((int64_t)1 << 31) - 1024)
+        return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events (MC: 4 x events)");
+    CovTable table{};
+    int rc = check_cov_waves(c, waves, &table);
+    if (rc)
+        return rc;
+    return load_incoherent(c, 4, n_data, n_mc_acc, n_mc_gen,
+                           [&](bool mc, const Planes &d, float *amax, bool *have_max) {
+                               *have_max = true;
+                               return generate_cov(c, table, mc ? mc_p3 : data_p3,
+                                                   mc ? n_mc_acc : n_data, d.ptr,
+                                                   mc ? kCovPseudoEvents : kCovPlanes, d.pitch, amax);
+                           });
+}
+
+int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, int64_t n_data,
+                               const void *mc_amp, int64_t n_mc_acc, double n_mc_gen,
+                               int amp_dtype)
+{
+    if (!c)
+        return PWA_EINVAL;
+    if (n_lambda == 1)
+        return pwa_load_events(c, data_amp, n_data, mc_amp, n_mc_acc, n_mc_gen, amp_dtype);
+    if (n_lambda < 1 || n_lambda > incoh_max_components())
+        return fail(c, PWA_EINVAL, "n_lambda=%d outside [1, %d]", n_lambda, incoh_max_components());
+    if (!data_amp || !mc_amp)
+        return fail(c, PWA_EINVAL, "null amplitude pointer");
+    if (n_data < 1 || n_mc_acc < 1)
+        return fail(c, PWA_EINVAL, "n_data=%lld and n_mc_acc=%lld must be >= 1",
+                    (long long)n_data, (long long)n_mc_acc);
+    if (amp_dtype != PWA_C64 && amp_dtype != PWA_C128)
+        return fail(c, PWA_EINVAL, "amp_dtype=%d is neither PWA_C64 nor PWA_C128", amp_dtype);
+    if (n_data > ((int64_t)1 << 31) - 1024 || n_mc_acc * n_lambda > ((int64_t)1 << 31) - 1024)
+        return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events (MC: events x n_lambda)");
+    // the MC's bytes read as n L pseudo-events of N waves
+    return load_incoherent(c, n_lambda, n_data, n_mc_acc, n_mc_gen,
+                           [&](bool mc, const Planes &d, float *, bool *) {
+                               return pack_rows(c, mc ? mc_amp : data_amp, d.n, amp_dtype, d.n_waves,
+                                                d.ptr, d.pitch);
+                           });
 }
 
 int pwa_build_norm(pwa_ctx *c, double *M_out)

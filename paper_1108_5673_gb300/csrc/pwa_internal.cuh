@@ -501,6 +501,12 @@ cudaError_t launch_nll_res_tma(const CUtensorMap *dmap, const CUtensorMap *mmap,
 struct alignas(16) GenPair {
     float h0, h1, l0, l1;  // a float pair h + l, each twice (for two events)
 };
+// a double as the nearest float and the remainder
+inline GenPair gen_pair(double x)
+{
+    const float h = (float)x, l = (float)(x - (double)h);
+    return {h, h, l, l};
+}
 struct alignas(16) GenWave {
     GenPair m2, g, g2, nrm;    // M^2, +-M G, (M G)^2, +-norm (the signs of m < 0)
     double mass, width, norm;  // norm = sqrt((2l + 1)/(4 pi) (l - |m|)!/(l + |m|)!)
@@ -528,14 +534,27 @@ cudaError_t launch_amp_gen(const double *kin, int64_t n, int N, const GenTable &
 
 // k_ampgen_cov.cu: covariant tensor amplitudes of J/psi -> gamma X, X -> K+ K-
 // from p3 [n][9] (photon, K+, K- 3-momenta, device), 4 incoherent components
-// per event; out as event-major [n][4][N] complex64 or, soa, the planes of an
-// incoherent sample (plane 2 (l N + a) = Re A_a^l of `pitch` floats).
-struct CovWave {
+// per event, each the float nearest to its FP64 value. out by mode:
+// event-major [n][4][N] complex64; the planes of an incoherent sample (plane
+// 2 (l N + a) = Re A_a^l of `pitch` floats); or n 4 pseudo-events of N waves
+// (plane 2a = Re A_a at event 4i + l; pitch a multiple of 4). amax (may be
+// null, zeroed by the caller): [N] max over events and components of |Re| +
+// |Im|. fp64_only evaluates everything in FP64.
+enum { kCovEventMajor = 0, kCovPlanes = 1, kCovPseudoEvents = 2 };
+struct alignas(16) CovWave {
+    GenPair m2, g, g2;  // M^2, M G, (M G)^2
     double mass, width;
-    int spin;  // 0 or 2
+    int spin;           // 0 or 2
+    int index;
 };
-cudaError_t launch_cov_amp_gen(const double *p3, int64_t n, int N, const CovWave *waves, float *out,
-                               bool soa, int64_t pitch, int grid, cudaStream_t s);
+struct CovTable {
+    CovWave w[kMaxWaves];
+    int fp64_only;      // a mass or width outside the float-float range
+};
+void cov_table(const pwa_cov_wave *waves, int N, CovTable *table);
+cudaError_t launch_cov_amp_gen(const double *p3, int64_t n, int N, const CovTable &table, bool fp64_only,
+                               float *out, int mode, int64_t pitch, float *amax, int num_sms,
+                               cudaStream_t s);
 
 // k_nll_incoh.cu: direct form with an incoherent sum over n_lambda components;
 // d holds 2 n_lambda N planes (plane 2 (l N + a) = Re A_a^l). Same scratch,
