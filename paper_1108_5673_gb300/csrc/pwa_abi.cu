@@ -239,8 +239,11 @@ void free_sample(pwa_ctx *c)
 
 // Copy n events of nw complex waves (event-major, host or device) into the
 // 2 nw planes starting at dst (pitch floats apart): device sources are packed
-// directly; host sources go through a bounded device staging buffer.
-int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *dst, int64_t pitch)
+// directly; host sources go through a bounded device staging buffer. amax
+// (may be null; [n_max], zeroed by the caller) takes the waves' maxima, wave w
+// at w mod n_max.
+int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *dst, int64_t pitch,
+              float *amax, int n_max)
 {
     if (nw == 0 || n == 0)
         return PWA_OK;
@@ -248,7 +251,7 @@ int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *
     if (is_device_pointer(src)) {
         if (int rc = device_input_ready(c))
             return rc;
-        CK(c, launch_pack(src, dtype, n, nw, dst, pitch, c->stream));
+        CK(c, launch_pack(src, dtype, n, nw, dst, pitch, amax, n_max, c->num_sms, c->stream));
         return PWA_OK;
     }
     const int64_t chunk = (int64_t)((64u << 20) / esz) > 0 ? (int64_t)((64u << 20) / esz) : 1;
@@ -261,7 +264,8 @@ int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *
         cudaError_t e = cudaMemcpyAsync(staging, static_cast<const char *>(src) + s * esz, m * esz,
                                         cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess)
-            e = launch_pack(staging, dtype, m, nw, dst + s, pitch, c->stream);
+            e = launch_pack(staging, dtype, m, nw, dst + s, pitch, amax, n_max, c->num_sms,
+                            c->stream);
         if (e != cudaSuccess) {
             cudaStreamSynchronize(c->stream);
             cudaFree(staging);
@@ -276,18 +280,30 @@ int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *
     return PWA_OK;
 }
 
-// Copy one sample into planes [2N][pitch].
-int load_planes(pwa_ctx *c, const void *src, int64_t n, int dtype, Planes *out)
+// Zeroes the events past n of `rows` planes (the events below n are written by
+// the kernels that fill the planes).
+int zero_tails(pwa_ctx *c, float *planes, int64_t n, int64_t pitch, int rows)
+{
+    if (n < pitch)
+        CK(c, cudaMemset2DAsync(planes + n, pitch * sizeof(float), 0, (pitch - n) * sizeof(float),
+                                rows, c->stream));
+    return PWA_OK;
+}
+
+// Copy one sample into planes [2N][pitch], its waves' maxima into amax [N].
+int load_planes(pwa_ctx *c, const void *src, int64_t n, int dtype, Planes *out, float *amax)
 {
     const int N = c->N;
     out->n = n;
     out->n_waves = N;
     out->pitch = round_up(n, 256);
     int rc = dev_alloc(c, (void **)&out->ptr, (size_t)2 * N * out->pitch * sizeof(float), "planes");
+    if (!rc)
+        rc = zero_tails(c, out->ptr, n, out->pitch, 2 * N);
     if (rc)
         return rc;
-    CK(c, cudaMemsetAsync(out->ptr, 0, (size_t)2 * N * out->pitch * sizeof(float), c->stream));
-    return pack_rows(c, src, n, dtype, N, out->ptr, out->pitch);
+    CK(c, cudaMemsetAsync(amax, 0, N * sizeof(float), c->stream));
+    return pack_rows(c, src, n, dtype, N, out->ptr, out->pitch, amax, N);
 }
 
 // n doubles (host or device) rounded to floats at dst.
@@ -320,22 +336,26 @@ int load_floats(pwa_ctx *c, const double *src, int64_t n, float *dst)
     return PWA_OK;
 }
 
-// One sample of the free-resonance form: planes [1 + 2N][pitch] + padding.
+// One sample of the free-resonance form: planes [1 + 2N][pitch] + padding; the
+// maxima of |Y_a|_1 (free waves) and |A_a|_1 into amax [N] where they exceed it.
 int load_res_sample(pwa_ctx *c, int R, const double *m, const void *Y, const void *Afix, int64_t n,
-                    int dtype, float **out, int64_t *pitch)
+                    int dtype, float **out, int64_t *pitch, float *amax)
 {
     const int N = c->N;
     *pitch = round_up(n, 256);
-    const size_t bytes = ((size_t)(1 + 2 * N) * *pitch + 256) * sizeof(float);
-    int rc = dev_alloc(c, (void **)out, bytes, "resonance planes");
+    const size_t all = (size_t)(1 + 2 * N) * *pitch;
+    int rc = dev_alloc(c, (void **)out, (all + 256) * sizeof(float), "resonance planes");
+    if (!rc)
+        rc = zero_tails(c, *out, n, *pitch, 1 + 2 * N);
     if (rc)
         return rc;
-    CK(c, cudaMemsetAsync(*out, 0, bytes, c->stream));
+    CK(c, cudaMemsetAsync(*out + all, 0, 256 * sizeof(float), c->stream));
     if ((rc = load_floats(c, m, n, *out)))
         return rc;
-    if ((rc = pack_rows(c, Y, n, dtype, R, *out + *pitch, *pitch)))
+    if ((rc = pack_rows(c, Y, n, dtype, R, *out + *pitch, *pitch, amax, R)))
         return rc;
-    return pack_rows(c, Afix, n, dtype, N - R, *out + (size_t)(1 + 2 * R) * *pitch, *pitch);
+    return pack_rows(c, Afix, n, dtype, N - R, *out + (size_t)(1 + 2 * R) * *pitch, *pitch, amax + R,
+                     N - R);
 }
 
 
@@ -673,11 +693,16 @@ int pwa_load_resonance_events(pwa_ctx *c, int n_free, const double *m_data, cons
     DeviceGuard g(c->device);
     cudaStreamSynchronize(c->stream);
     free_res(c);
-    int rc = load_res_sample(c, n_free, m_data, Y_data, Afix_data, n_data, amp_dtype, &c->res_data,
-                             &c->res_data_pitch);
+    // per-wave maxima over both samples bound the TMA-fed kernel's exact product split
+    int rc = dev_alloc(c, (void **)&c->res_amax, N * sizeof(float), "resonance maxima");
+    if (!rc && cudaMemsetAsync(c->res_amax, 0, N * sizeof(float), c->stream) != cudaSuccess)
+        rc = fail(c, PWA_ECUDA, "memset");
+    if (!rc)
+        rc = load_res_sample(c, n_free, m_data, Y_data, Afix_data, n_data, amp_dtype, &c->res_data,
+                             &c->res_data_pitch, c->res_amax);
     if (!rc)
         rc = load_res_sample(c, n_free, m_mc, Y_mc, Afix_mc, n_mc_acc, amp_dtype, &c->res_mc,
-                             &c->res_mc_pitch);
+                             &c->res_mc_pitch, c->res_amax);
     const size_t npart = res_partials_doubles(N, n_free, c->num_sms * kResMaxBlocksPerSm);
     const size_t nio = 4 * (size_t)N + 4 * (size_t)n_free + 2;
     if (!rc)
@@ -689,52 +714,17 @@ int pwa_load_resonance_events(pwa_ctx *c, int n_free, const double *m_data, cons
         c->h_res = nullptr;
         rc = fail(c, PWA_ENOMEM, "pinned host buffer");
     }
-    // The TMA-fed kernel (PWA_RES_KERNEL=generic selects the per-event one):
-    // per-wave maxima over both samples bound its exact product split.
+    // The TMA-fed kernel (PWA_RES_KERNEL=generic selects the per-event one).
     const char *kv = getenv("PWA_RES_KERNEL");
     const bool tma = res_tma_available(N, n_free) && !(kv && strcmp(kv, "generic") == 0);
     if (!rc && tma) {
-        float *tmp = nullptr;
-        rc = dev_alloc(c, (void **)&c->res_amax, N * sizeof(float), "resonance maxima");
-        if (!rc)
-            rc = dev_alloc(c, (void **)&tmp, N * sizeof(float), "resonance maxima");
-        cudaError_t e = cudaSuccess;
-        if (!rc) {
-            const Planes pd{c->res_data + c->res_data_pitch, c->res_data_pitch, n_data, N};
-            const Planes pm{c->res_mc + c->res_mc_pitch, c->res_mc_pitch, n_mc_acc, N};
-            e = cudaMemsetAsync(c->res_amax, 0, N * sizeof(float), c->stream);
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(tmp, 0, N * sizeof(float), c->stream);
-            if (e == cudaSuccess)
-                e = launch_amp_max(pd, c->res_amax, c->stream);
-            if (e == cudaSuccess)
-                e = launch_amp_max(pm, tmp, c->stream);
-            std::vector<float> h1(N), h2(N);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(h1.data(), c->res_amax, N * sizeof(float), cudaMemcpyDeviceToHost,
-                                    c->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(h2.data(), tmp, N * sizeof(float), cudaMemcpyDeviceToHost,
-                                    c->stream);
-            if (e == cudaSuccess)
-                e = cudaStreamSynchronize(c->stream);
-            for (int k = 0; k < N && e == cudaSuccess; ++k)
-                h1[k] = std::max(h1[k], h2[k]);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(c->res_amax, h1.data(), N * sizeof(float), cudaMemcpyHostToDevice,
-                                    c->stream);
-            if (e == cudaSuccess)
-                e = cudaStreamSynchronize(c->stream);
-            if (e == cudaSuccess)
-                e = encode_planes_map(&c->res_dmap, c->res_data, n_data, c->res_data_pitch, 1 + 2 * N,
-                                      res_tma_box_events(), 1 + 2 * N);
-            if (e == cudaSuccess)
-                e = encode_planes_map(&c->res_mmap, c->res_mc, n_mc_acc, c->res_mc_pitch, 1 + 2 * N,
-                                      res_tma_box_events(), 1 + 2 * N);
-            if (e != cudaSuccess)
-                rc = fail(c, PWA_ECUDA, "free-resonance set-up: %s", cudaGetErrorString(e));
-        }
-        dev_free(tmp);
+        cudaError_t e = encode_planes_map(&c->res_dmap, c->res_data, n_data, c->res_data_pitch,
+                                          1 + 2 * N, res_tma_box_events(), 1 + 2 * N);
+        if (e == cudaSuccess)
+            e = encode_planes_map(&c->res_mmap, c->res_mc, n_mc_acc, c->res_mc_pitch, 1 + 2 * N,
+                                  res_tma_box_events(), 1 + 2 * N);
+        if (e != cudaSuccess)
+            rc = fail(c, PWA_ECUDA, "free-resonance set-up: %s", cudaGetErrorString(e));
     }
     if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess)
         rc = fail(c, PWA_ECUDA, "loading the resonance samples");
@@ -1178,15 +1168,15 @@ int pwa_load_events(pwa_ctx *c, const void *data_amp, int64_t n_data, const void
     cudaStreamSynchronize(c->stream);
     free_sample(c);
     c->n_lambda = 1;
-    int rc = load_planes(c, data_amp, n_data, amp_dtype, &c->data);
+    int rc = load_planes(c, data_amp, n_data, amp_dtype, &c->data, c->amax);
     if (!rc)
-        rc = load_planes(c, mc_amp, n_mc_acc, amp_dtype, &c->mc);
+        rc = load_planes(c, mc_amp, n_mc_acc, amp_dtype, &c->mc, c->mc_amax);
     return finish_load(c, rc, n_data, n_mc_acc, n_mc_gen);
 }
 
-// After the data and MC planes of a coherent sample are filled (rc = the
-// status so far): the table, the tensor-core store, the amplitude maxima and
-// the direct form's tensor map; then the sample is marked loaded.
+// After the data and MC planes of a coherent sample and their maxima are
+// filled (rc = the status so far): the table, the tensor-core store and the
+// tensor maps; then the sample is marked loaded.
 static int finish_load(pwa_ctx *c, int rc, int64_t n_data, int64_t n_mc_acc, double n_mc_gen)
 {
     if (!rc && (c->cfg.forms & PWA_FORM_TABLE)) {
@@ -1223,13 +1213,6 @@ static int finish_load(pwa_ctx *c, int rc, int64_t n_data, int64_t n_mc_acc, dou
         }
     }
     if (!rc) {
-        cudaError_t e = cudaMemsetAsync(c->amax, 0, c->N * sizeof(float), c->stream);
-        if (e == cudaSuccess)
-            e = launch_amp_max(c->data, c->amax, c->stream);
-        if (e != cudaSuccess)
-            rc = fail(c, PWA_ECUDA, "amplitude maxima: %s", cudaGetErrorString(e));
-    }
-    if (!rc) {
         cudaError_t e = encode_planes_map(&c->data_map, c->data.ptr, c->data.n, c->data.pitch,
                                           2 * c->N, amp_box_events(c->N), amp_box_rows(c->N));
         // the MC sample's map and maxima serve the projection weights
@@ -1242,10 +1225,6 @@ static int finish_load(pwa_ctx *c, int rc, int64_t n_data, int64_t n_mc_acc, dou
                                   hess_tc_box_events(), 2 * c->N);
             c->hess_tc = e == cudaSuccess;
         }
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(c->mc_amax, 0, c->N * sizeof(float), c->stream);
-        if (e == cudaSuccess)
-            e = launch_amp_max(c->mc, c->mc_amax, c->stream);
         if (e != cudaSuccess)
             rc = fail(c, PWA_ECUDA, "tensor map encode failed");
     }
@@ -1387,11 +1366,14 @@ int pwa_load_events_generated(pwa_ctx *c, const pwa_wave *waves, const double *d
         p.n_waves = N;
         p.pitch = round_up(n, 256);
         rc = dev_alloc(c, (void **)&p.ptr, (size_t)2 * N * p.pitch * sizeof(float), "planes");
-        if (!rc && cudaMemsetAsync(p.ptr, 0, (size_t)2 * N * p.pitch * sizeof(float), c->stream) !=
-                       cudaSuccess)
-            rc = fail(c, PWA_ECUDA, "memset");
+        if (!rc)
+            rc = zero_tails(c, p.ptr, n, p.pitch, 2 * N);
         if (!rc)
             rc = generate(c, table, which == 0 ? data_kin : mc_kin, n, p.ptr, true, p.pitch);
+        float *amax = which == 0 ? c->amax : c->mc_amax;
+        if (!rc && (cudaMemsetAsync(amax, 0, N * sizeof(float), c->stream) != cudaSuccess ||
+                    launch_amp_max(p, amax, c->stream) != cudaSuccess))
+            rc = fail(c, PWA_ECUDA, "amplitude maxima");
     }
     return finish_load(c, rc, n_data, n_mc_acc, n_mc_gen);
 }
@@ -1491,8 +1473,8 @@ int pwa_compute_covariant_amplitudes(pwa_ctx *c, const pwa_cov_wave *waves, cons
 // around `fill`, which writes the amplitudes. fill(mc, planes, amax): mc false,
 // the data planes (plane 2 (l N + a) = Re A_a^l); mc true, n_mc_acc L pseudo-
 // events of N waves, so that M sums the products over components as well as
-// over events. It may leave the maxima of |Re| + |Im| per wave in amax (zeroed,
-// [N]) and then returns them as done through *have_max.
+// over events; amax (zeroed, [N]) takes max |Re A_a| + |Im A_a| over events and
+// components.
 template <typename Fill>
 static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, double n_mc_gen,
                            Fill fill)
@@ -1510,7 +1492,6 @@ static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, 
     cudaStreamSynchronize(c->stream);
     free_sample(c);
     int rc = PWA_OK;
-    bool have_max[2] = {false, false};
     for (int mc = 0; mc < 2 && !rc; ++mc) {
         Planes &d = mc ? c->mc : c->data;
         float *amax = mc ? c->mc_amax : c->amax;
@@ -1519,11 +1500,12 @@ static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, 
         d.pitch = round_up(d.n, 256);
         const size_t bytes = (size_t)2 * d.n_waves * d.pitch * sizeof(float);
         rc = dev_alloc(c, (void **)&d.ptr, bytes, "planes");
-        if (!rc && (cudaMemsetAsync(d.ptr, 0, bytes, c->stream) != cudaSuccess ||
-                    cudaMemsetAsync(amax, 0, N * sizeof(float), c->stream) != cudaSuccess))
+        if (!rc)
+            rc = zero_tails(c, d.ptr, d.n, d.pitch, 2 * d.n_waves);
+        if (!rc && cudaMemsetAsync(amax, 0, N * sizeof(float), c->stream) != cudaSuccess)
             rc = fail(c, PWA_ECUDA, "memset");
         if (!rc)
-            rc = fill(mc != 0, d, amax, &have_max[mc]);
+            rc = fill(mc != 0, d, amax);
     }
     const Planes &d = c->data;
     if (!rc && (c->cfg.forms & PWA_FORM_TABLE)) {
@@ -1546,44 +1528,12 @@ static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, 
                 rc = fail(c, PWA_ECUDA, "table build: %s", cudaGetErrorString(e));
         }
     }
-    // The TMA-fed kernel (N_pad L <= 48) bounds its exact product split by
-    // amax[a] = max over components and events of |Re A_a^l| + |Im A_a^l|; it
-    // reads all 2 L n planes as one box per tile. PWA_INCOH_KERNEL=generic
+    // The TMA-fed kernel (N_pad L <= 48) bounds its exact product split by amax;
+    // it reads all 2 L n planes as one box per tile. PWA_INCOH_KERNEL=generic
     // selects the one-event-per-thread kernel instead.
     const char *kv = getenv("PWA_INCOH_KERNEL");
     const bool tma = (c->cfg.forms & PWA_FORM_AMP) && incoh_tma_available(N, L) &&
                      !(kv && strcmp(kv, "generic") == 0);
-    // the maxima over the MC pseudo-events scale the tensor-core build of M
-    if (!rc && !have_max[1] && launch_amp_max(c->mc, c->mc_amax, c->stream) != cudaSuccess)
-        rc = fail(c, PWA_ECUDA, "MC amplitude maxima");
-    if (!rc && tma && !have_max[0]) {
-        float *dmax = nullptr;
-        rc = dev_alloc(c, (void **)&dmax, (size_t)L * N * sizeof(float), "component maxima");
-        std::vector<float> hmax((size_t)L * N), amax(N, 0.f);
-        cudaError_t e = cudaSuccess;
-        if (!rc) {
-            e = cudaMemsetAsync(dmax, 0, (size_t)L * N * sizeof(float), c->stream);
-            if (e == cudaSuccess)
-                e = launch_amp_max(d, dmax, c->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(hmax.data(), dmax, (size_t)L * N * sizeof(float),
-                                    cudaMemcpyDeviceToHost, c->stream);
-            if (e == cudaSuccess)
-                e = cudaStreamSynchronize(c->stream);
-            for (int l = 0; l < L && e == cudaSuccess; ++l)
-                for (int a = 0; a < N; ++a)
-                    amax[a] = std::max(amax[a], hmax[(size_t)l * N + a]);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(c->amax, amax.data(), N * sizeof(float), cudaMemcpyHostToDevice,
-                                    c->stream);
-            if (e != cudaSuccess)
-                rc = fail(c, PWA_ECUDA, "incoherent direct-form set-up: %s", cudaGetErrorString(e));
-        }
-        if (dmax) {
-            cudaStreamSynchronize(c->stream);
-            cudaFree(dmax);
-        }
-    }
     if (!rc && tma) {
         const cudaError_t e = encode_planes_map(&c->data_map, d.ptr, n_data, d.pitch, 2 * L * N,
                                                 incoh_tma_box_events(), 2 * L * N);
@@ -1633,8 +1583,7 @@ int pwa_load_events_covariant(pwa_ctx *c, const pwa_cov_wave *waves, const doubl
     if (rc)
         return rc;
     return load_incoherent(c, 4, n_data, n_mc_acc, n_mc_gen,
-                           [&](bool mc, const Planes &d, float *amax, bool *have_max) {
-                               *have_max = true;
+                           [&](bool mc, const Planes &d, float *amax) {
                                return generate_cov(c, table, mc ? mc_p3 : data_p3,
                                                    mc ? n_mc_acc : n_data, d.ptr,
                                                    mc ? kCovPseudoEvents : kCovPlanes, d.pitch, amax);
@@ -1662,9 +1611,9 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
         return fail(c, PWA_EINVAL, "samples are limited to 2^31 - 1024 events (MC: events x n_lambda)");
     // the MC's bytes read as n L pseudo-events of N waves
     return load_incoherent(c, n_lambda, n_data, n_mc_acc, n_mc_gen,
-                           [&](bool mc, const Planes &d, float *, bool *) {
+                           [&](bool mc, const Planes &d, float *amax) {
                                return pack_rows(c, mc ? mc_amp : data_amp, d.n, amp_dtype, d.n_waves,
-                                                d.ptr, d.pitch);
+                                                d.ptr, d.pitch, amax, c->N);
                            });
 }
 

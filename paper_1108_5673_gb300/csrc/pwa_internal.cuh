@@ -404,8 +404,10 @@ cudaError_t encode_planes_map(CUtensorMap *map, const float *base, int64_t n, in
                               int rows, int box_x, int box_y);
 
 // k_pack.cu
+// amax (may be null): amax[w mod n_max] = max of itself and |Re A_w| + |Im A_w|
+// over the events, so that several calls may share it (zeroed before the first)
 cudaError_t launch_pack(const void *src, int dtype, int64_t n, int n_waves, float *planes,
-                        int64_t pitch, cudaStream_t s);
+                        int64_t pitch, float *amax, int n_max, int num_sms, cudaStream_t s);
 cudaError_t launch_table_build(const Planes &amp, float *table, int64_t table_pitch,
                                cudaStream_t s);
 // amax[a] = max_i |Re A_a(i)| + |Im A_a(i)| (amax must be zeroed first)
