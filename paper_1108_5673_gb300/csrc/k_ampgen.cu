@@ -401,9 +401,11 @@ cudaError_t launch_amp_gen(const double *kin, int64_t n, int N, const GenTable &
     if (soa) {
         amp_gen_kernel<true><<<grid, kGenThreads, 0, s>>>(kin, n, N, table, fp64_only, out, pitch);
     } else {
-        const size_t smem = (size_t)2 * kGenThreads * (N | 1) * sizeof(float2);
+        const auto rows = [](int waves) { return (size_t)2 * kGenThreads * (waves | 1) * sizeof(float2); };
+        const size_t smem = rows(N);
+        // the same limit at every call: contexts in other threads launch it too
         const cudaError_t e = cudaFuncSetAttribute(
-            amp_gen_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            amp_gen_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows(kMaxWaves));
         if (e != cudaSuccess)
             return e;
         amp_gen_kernel<false><<<grid, kGenThreads, smem, s>>>(kin, n, N, table, fp64_only, out, 0);

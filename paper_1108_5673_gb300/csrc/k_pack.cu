@@ -20,6 +20,13 @@ namespace {
 
 constexpr int kPackWarps = 8;
 constexpr int kPackUnroll = 8;  // loads in flight per lane
+constexpr int kPackMaxWaves = 2 * kMaxWaves;  // an incoherent sample's waves times components
+
+constexpr size_t pack_smem(int n_waves, int n_max)
+{
+    return ((size_t)kPackWarps * 2 * n_waves * 33 + n_max) * sizeof(float);
+}
+static_assert(pack_smem(kPackMaxWaves, kPackMaxWaves) <= 227 * 1024, "shared memory");
 
 // One warp takes 32 events: their rows are contiguous in the source, so they
 // are read 32 elements at a time (a load's lanes next to each other, eight
@@ -103,9 +110,10 @@ template <typename T2>
 cudaError_t pack(const void *src, int64_t n, int N, float *planes, int64_t pitch, float *amax,
                  int n_max, int num_sms, cudaStream_t s)
 {
-    const size_t smem = ((size_t)kPackWarps * 2 * N * 33 + n_max) * sizeof(float);
+    const size_t smem = pack_smem(N, n_max);
+    // the same limit at every call: contexts in other threads launch it too
     cudaError_t e = cudaFuncSetAttribute(pack_kernel<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         (int)pack_smem(kPackMaxWaves, kPackMaxWaves));
     if (e != cudaSuccess)
         return e;
     // as many blocks as shared memory (and 2048 threads an SM) keeps resident
@@ -245,7 +253,7 @@ cudaError_t launch_pack(const void *src, int dtype, int64_t n, int n_waves, floa
 {
     if (n <= 0)
         return cudaSuccess;
-    if (n_waves < 1 || n_max < 1 || n_waves % n_max)
+    if (n_waves < 1 || n_waves > kPackMaxWaves || n_max < 1 || n_waves % n_max)
         return cudaErrorInvalidValue;
     return dtype == PWA_C64
                ? pack<float2>(src, n, n_waves, planes, pitch, amax, n_max, num_sms, s)

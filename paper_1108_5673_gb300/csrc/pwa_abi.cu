@@ -58,6 +58,7 @@ struct pwa_ctx {
         cudaGraphExec_t exec;
     };
     std::vector<EvalGraph> graphs;
+    bool captured = false;      // an asynchronous call went into a caller's graph
     unsigned epoch = 0;
     bool graphs_off = false;
     int tune_res_cps = 1;       // free-resonance kernel: blocks per SM
@@ -137,7 +138,7 @@ int dev_alloc(pwa_ctx *ctx, void **p, size_t bytes, const char *what)
     *p = nullptr;
     if (injected_alloc_failure())
         return fail(ctx, PWA_ENOMEM, "injected allocation failure (%s, %zu bytes)", what, bytes);
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = pool_alloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -147,11 +148,45 @@ int dev_alloc(pwa_ctx *ctx, void **p, size_t bytes, const char *what)
     return PWA_OK;
 }
 
+// Whether the last wait of this thread before returning memory succeeded: it is
+// kept for another context only then (else cudaFree and the like decide).
+thread_local bool t_quiet = true;
+
+// Before the memory of a context is returned: the work that may use it has
+// finished. All of it was enqueued on the context's stream, unless an
+// asynchronous call was captured into a caller's graph, whose launches may be
+// anywhere on the device.
+void quiet(pwa_ctx *c)
+{
+    t_quiet = (!c->stream || cudaStreamSynchronize(c->stream) == cudaSuccess) &&
+              (!c->captured || cudaDeviceSynchronize() == cudaSuccess);
+    if (!t_quiet)
+        cudaGetLastError();
+}
+
+// Notes that the context's work is being captured by the caller.
+void note_capture(pwa_ctx *c)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess)
+        cudaGetLastError();
+    if (st != cudaStreamCaptureStatusNone)
+        c->captured = true;
+}
+
+// Returns memory to the pool: no work in flight may still use it (the callers
+// have synchronised the stream or the device that did).
 template <typename T>
 void dev_free(T *&p)
 {
-    if (p)
-        cudaFree(p);
+    pool_free(p, t_quiet);
+    p = nullptr;
+}
+
+template <typename T>
+void host_free(T *&p)
+{
+    pool_host_free(p, t_quiet);
     p = nullptr;
 }
 
@@ -213,19 +248,21 @@ size_t io_doubles(int N, int max_k) { return io_flags_at(N, max_k) + max_k; }
 
 void free_res(pwa_ctx *c)
 {
+    if (c->res_data || c->res_mc || c->d_res || c->res_amax || c->h_res)
+        quiet(c);
     dev_free(c->res_data);
     dev_free(c->res_mc);
     dev_free(c->d_res);
     dev_free(c->res_amax);
-    if (c->h_res)
-        cudaFreeHost(c->h_res);
-    c->h_res = nullptr;
+    host_free(c->h_res);
     c->res_loaded = false;
     c->res_tma = false;
 }
 
 void free_sample(pwa_ctx *c)
 {
+    if (c->data.ptr || c->mc.ptr || c->table || c->tmax || c->xbf)
+        quiet(c);
     dev_free(c->data.ptr);
     dev_free(c->mc.ptr);
     dev_free(c->table);
@@ -268,13 +305,13 @@ int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *
                             c->stream);
         if (e != cudaSuccess) {
             cudaStreamSynchronize(c->stream);
-            cudaFree(staging);
+            dev_free(staging);
             cudaGetLastError();
             return fail(c, PWA_ECUDA, "loading amplitudes: %s", cudaGetErrorString(e));
         }
     }
     cudaError_t e = cudaStreamSynchronize(c->stream);
-    cudaFree(staging);
+    dev_free(staging);
     if (e != cudaSuccess)
         return fail(c, PWA_ECUDA, "loading amplitudes: %s", cudaGetErrorString(e));
     return PWA_OK;
@@ -328,7 +365,7 @@ int load_floats(pwa_ctx *c, const double *src, int64_t n, float *dst)
             e = launch_to_float(staging, m, dst + s, c->stream);
     }
     const cudaError_t e2 = cudaStreamSynchronize(c->stream);
-    cudaFree(staging);
+    dev_free(staging);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         cudaGetLastError();
         return fail(c, PWA_ECUDA, "loading masses: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
@@ -709,7 +746,7 @@ int pwa_load_resonance_events(pwa_ctx *c, int n_free, const double *m_data, cons
         rc = dev_alloc(c, (void **)&c->d_res, (npart + 1 + nio) * sizeof(double), "resonance io");
     if (!rc && cudaMemsetAsync(c->d_res, 0, (npart + 1 + nio) * sizeof(double), c->stream) != cudaSuccess)
         rc = fail(c, PWA_ECUDA, "memset");
-    if (!rc && cudaMallocHost((void **)&c->h_res, nio * sizeof(double)) != cudaSuccess) {
+    if (!rc && pool_host_alloc((void **)&c->h_res, nio * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         c->h_res = nullptr;
         rc = fail(c, PWA_ENOMEM, "pinned host buffer");
@@ -738,6 +775,7 @@ int pwa_load_resonance_events(pwa_ctx *c, int n_free, const double *m_data, cons
     c->res_n_mc = n_mc_acc;
     c->res_ngen = n_mc_gen;
     c->res_loaded = true;
+    pool_loaded();
     return PWA_OK;
 }
 
@@ -787,6 +825,7 @@ int pwa_nll_grad_res_async(pwa_ctx *c, const double *d_V, const double *d_mass,
     if (!c->res_loaded)
         return fail(c, PWA_ESTATE, "pwa_load_resonance_events must come first");
     DeviceGuard g(c->device);
+    note_capture(c);
     return enqueue_res(c, d_V, d_mass, d_width, d_out, c->async_status, nullptr);
 }
 
@@ -843,15 +882,15 @@ static int fx_alloc(pwa_ctx *c)
                                   hess_tc_partials_doubles(N, c->num_sms));
     const size_t bytes = (nio + npart) * sizeof(double);
     if (c->fx_bytes < bytes) {
+        if (c->d_fx || c->h_fx)
+            quiet(c);
         dev_free(c->d_fx);
-        if (c->h_fx)
-            cudaFreeHost(c->h_fx);
-        c->h_fx = nullptr;
+        host_free(c->h_fx);
         c->fx_bytes = 0;
         int rc = dev_alloc(c, (void **)&c->d_fx, bytes, "Hessian scratch");
         if (rc)
             return rc;
-        if (cudaMallocHost((void **)&c->h_fx, nio * sizeof(double)) != cudaSuccess) {
+        if (pool_host_alloc((void **)&c->h_fx, nio * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             c->h_fx = nullptr;
             dev_free(c->d_fx);
@@ -941,6 +980,7 @@ int pwa_hessian_async(pwa_ctx *c, const double *d_V, double *d_H)
     if (c->n_lambda > 1)
         return fail(c, PWA_ENOTSUP, "the Hessian takes coherent samples only");
     DeviceGuard g(c->device);
+    note_capture(c);
     int rc = fx_alloc(c);
     if (rc)
         return rc;
@@ -1071,17 +1111,17 @@ int pwa_create(pwa_ctx **out, int device, const pwa_config *cfg)
     }
     if ((forms & PWA_FORM_TABLE) && c->N > table_max_waves())
         return bail(fail(c, PWA_ENOTSUP, "the table form supports up to %d waves", table_max_waves()));
-    cudaError_t e = amp_configure();
+    cudaError_t e = configure_once(kConfigAmp, amp_configure);
     if (e == cudaSuccess && (forms & PWA_FORM_TABLE))
-        e = table_configure();
+        e = configure_once(kConfigTable, table_configure);
     if (e == cudaSuccess && (forms & PWA_FORM_TC))
-        e = batched_configure();
+        e = configure_once(kConfigBatched, batched_configure);
     if (e != cudaSuccess)
         return bail(fail(c, PWA_ECUDA, "kernel configuration: %s", cudaGetErrorString(e)));
     const size_t nio = io_doubles(c->N, cfg->max_k);
     if ((rc = dev_alloc(c, (void **)&c->d_io, nio * sizeof(double), "io")))
         return bail(rc);
-    if (cudaHostAlloc((void **)&c->h_io, nio * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
+    if (pool_host_alloc((void **)&c->h_io, nio * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         c->h_io = nullptr;
         return bail(fail(c, PWA_ENOMEM, "pinned host buffer"));
@@ -1125,6 +1165,7 @@ int pwa_destroy(pwa_ctx *c)
     DeviceGuard g(c->device);
     if (c->stream)
         cudaStreamSynchronize(c->stream);
+    quiet(c);
     for (auto &g : c->graphs)
         cudaGraphExecDestroy(g.exec);
     c->graphs.clear();
@@ -1136,11 +1177,9 @@ int pwa_destroy(pwa_ctx *c)
     dev_free(c->d_io);
     dev_free(c->d_fx);
     dev_free(c->d_w);
-    if (c->h_fx)
-        cudaFreeHost(c->h_fx);
+    host_free(c->h_fx);
     dev_free(c->d_work);
-    if (c->h_io)
-        cudaFreeHost(c->h_io);
+    host_free(c->h_io);
     if (c->own_stream && c->stream)
         cudaStreamDestroy(c->stream);
     delete c;
@@ -1242,6 +1281,7 @@ static int finish_load(pwa_ctx *c, int rc, int64_t n_data, int64_t n_mc_acc, dou
     c->n_gen = n_mc_gen;
     c->loaded = true;
     c->has_norm = false;
+    pool_loaded();
     return PWA_OK;
 }
 
@@ -1284,7 +1324,7 @@ static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_
                                         cudaMemcpyHostToDevice, c->stream);
         if (e != cudaSuccess) {
             cudaStreamSynchronize(c->stream);
-            cudaFree(staging);
+            dev_free(staging);
             return fail(c, PWA_ECUDA, "kinematics copy: %s", cudaGetErrorString(e));
         }
         dk = staging;
@@ -1293,8 +1333,7 @@ static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_
     cudaError_t e = launch_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, soa,
                                    pitch, c->num_sms, c->stream);
     cudaError_t e2 = cudaStreamSynchronize(c->stream);
-    if (staging)
-        cudaFree(staging);
+    dev_free(staging);
     if (e == cudaSuccess)
         e = e2;
     if (e != cudaSuccess) {
@@ -1416,7 +1455,7 @@ static int generate_cov(pwa_ctx *c, const CovTable &table, const double *p3, int
                                         cudaMemcpyHostToDevice, c->stream);
         if (e != cudaSuccess) {
             cudaStreamSynchronize(c->stream);
-            cudaFree(staging);
+            dev_free(staging);
             return fail(c, PWA_ECUDA, "momenta copy: %s", cudaGetErrorString(e));
         }
         dk = staging;
@@ -1425,8 +1464,7 @@ static int generate_cov(pwa_ctx *c, const CovTable &table, const double *p3, int
     cudaError_t e = launch_cov_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, mode,
                                        pitch, amax, c->num_sms, c->stream);
     cudaError_t e2 = cudaStreamSynchronize(c->stream);
-    if (staging)
-        cudaFree(staging);
+    dev_free(staging);
     if (e == cudaSuccess)
         e = e2;
     if (e != cudaSuccess) {
@@ -1556,6 +1594,7 @@ static int load_incoherent(pwa_ctx *c, int L, int64_t n_data, int64_t n_mc_acc, 
     c->n_gen = n_mc_gen;
     c->loaded = true;
     c->has_norm = false;
+    pool_loaded();
     return PWA_OK;
 }
 
@@ -1656,7 +1695,9 @@ int pwa_build_norm(pwa_ctx *c, double *M_out)
             e = cudaMemcpyAsync(&flags, dstat, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(c->stream);
-        cudaFree(scratch);
+        if (e != cudaSuccess)
+            quiet(c);
+        dev_free(scratch);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
@@ -1671,7 +1712,9 @@ int pwa_build_norm(pwa_ctx *c, double *M_out)
         cudaError_t e = launch_build_norm(c->mc, c->n_gen, c->M, scratch, c->num_sms, c->stream);
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(c->stream);
-        cudaFree(scratch);
+        if (e != cudaSuccess)
+            quiet(c);
+        dev_free(scratch);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
@@ -1729,6 +1772,7 @@ int pwa_nll_grad_async(pwa_ctx *c, const double *d_V, int K, double *d_nll, doub
     if (rc)
         return rc;
     DeviceGuard g(c->device);
+    note_capture(c);
     return enqueue_eval(c, d_V, K, d_nll, d_grad, c->async_status, nullptr);
 }
 

@@ -403,6 +403,19 @@ struct Planes {
 cudaError_t encode_planes_map(CUtensorMap *map, const float *base, int64_t n, int64_t pitch,
                               int rows, int box_x, int box_y);
 
+// pwa_pool.cu: device and mapped pinned memory, kept for the next context
+// within bounds. Free only what no work in flight on the device may use;
+// keep = false frees it (cudaFree) instead of keeping it. Null is accepted.
+cudaError_t pool_alloc(void **p, size_t bytes);  // on the current device
+void pool_free(void *p, bool keep);              // likewise
+cudaError_t pool_host_alloc(void **p, size_t bytes);
+void pool_host_free(void *p, bool keep);
+void pool_loaded();  // a sample was loaded: blocks that many loads did not take are freed
+unsigned long long cuda_context_id();  // of the current CUDA context; changes with a device reset
+// Runs one of the configure functions below once per CUDA context.
+enum { kConfigAmp = 0, kConfigTable = 1, kConfigBatched = 2, kConfigCount = 3 };
+cudaError_t configure_once(int which, cudaError_t (*configure)());
+
 // k_pack.cu
 // amax (may be null): amax[w mod n_max] = max of itself and |Re A_w| + |Im A_w|
 // over the events, so that several calls may share it (zeroed before the first)
