@@ -89,10 +89,23 @@ __host__ __device__ constexpr int s_cols(int xs) { return xs == 2 ? 256 : 192; }
 constexpr double kLn2 = 0.69314718055994530942;
 constexpr int kFixBits = 19;                // fixed-point resolution of log2 sums
 
+// v 2^e, exactly (ldexp): a product where 2^e is a normal double (ldexp itself
+// is tens of FP64 instructions, and FP64 is what the preparation waits for).
+__host__ __device__ inline double scale2(double v, int e)
+{
+    if (e < -1000 || e > 1000)
+        return ldexp(v, e);
+#ifdef __CUDA_ARCH__
+    return v * __hiloint2double((1023 + e) << 20, 0);
+#else
+    return ldexp(v, e);
+#endif
+}
+
 // Integer slices of v * 2^(8 - T): v ~ 2^(T-8) (w0 + w1 / 2^8 + w2 / 2^16).
 __host__ __device__ inline void split_slices(double v, int T, double (&w)[kWSlices])
 {
-    double x = ldexp(v, 8 - T);
+    double x = scale2(v, 8 - T);
     for (int p = 0; p < kWSlices; ++p) {
         w[p] = rint(x);
         x = (x - w[p]) * 256.0;
@@ -103,7 +116,7 @@ __host__ __device__ inline double round_slices(double v, int T)
 {
     double w[kWSlices];
     split_slices(v, T, w);
-    return ldexp(w[0] + (w[1] + w[2] / 256.0) / 256.0, T - 8);
+    return scale2(w[0] + (w[1] + w[2] / 256.0) / 256.0, T - 8);
 }
 
 struct BatchArgs {
@@ -198,57 +211,105 @@ struct BatchItem {
 };
 
 // ---- per-call preparation: W image and set exponents ------------------------
-// One block per (chunk, half, slice).
+// One warp per set, four sets per block: the lanes take the waves, find the
+// set's largest |Re V|, |Im V| (a maximum of bit patterns), form the slices of
+// Re V and Im V once and write them at their four places: row (k,re) holds
+// (vr, -vi) and row (k,im) holds (vi, vr) at features 2w, 2w + 1 (rounding to
+// nearest even commutes with the sign). A warp writes whole 128-byte rows.
+// Bound by the FP64 pipe, so spread over many SMs: 128 sets x 32 waves 8 us cold
+// (13.7 us with 32 sets per block, on four SMs; 26 us with a block per slice,
+// the slices formed anew at each of the four places and ldexp).
+constexpr int kPrepSets = 4;
+constexpr int kPrepThreads = kPrepSets * 32;
+constexpr int kPrepPerHalf = kHS / kPrepSets;
+
+// bit patterns of |V| of wave w; whether both are finite
+__device__ __forceinline__ bool abs_bits(const double *V, int w, unsigned long long &m)
+{
+    const unsigned long long r = __double_as_longlong(V[2 * w]) & 0x7fffffffffffffffull,
+                             i = __double_as_longlong(V[2 * w + 1]) & 0x7fffffffffffffffull;
+    m = max(m, max(r, i));
+    return r < 0x7ff0000000000000ull && i < 0x7ff0000000000000ull;
+}
+
+// blk = half chunk * kPrepPerHalf + its part; part 0 also writes the half's flags
 __device__ __forceinline__ void batched_prep_block(const BatchArgs &a, const int blk)
 {
-    const int p = blk % kWSlices, h = (blk / kWSlices) & 1, c = blk / (2 * kWSlices);
-    const int Nw = a.n_waves, KB = (a.F + 63) / 64;
-    __shared__ int s_T[kHS];
-    if (threadIdx.x < kHS) {
-        const int k = c * kKC + h * kHS + threadIdx.x;
-        int e = 0;
-        if (k < a.K) {
-            double m = 0.0;
+    const int Nw = a.n_waves, KB = (a.F + 63) / 64, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int half = blk / kPrepPerHalf, part = blk % kPrepPerHalf, sl = part * kPrepSets + warp;
+    const int k = half * kHS + sl;
+    if (part == 0) {
+        // sets with a V that is not finite: every intensity is undefined
+        __shared__ unsigned s_bad;
+        if (threadIdx.x == 0)
+            s_bad = 0u;
+        __syncthreads();
+        for (int i = warp; i < kHS && half * kHS + i < a.K; i += kPrepSets) {
+            unsigned long long m = 0ull;
             bool finite = true;
-            for (int w = 0; w < Nw; ++w) {
-                const double vr = a.V[2 * ((size_t)k * Nw + w)], vi = a.V[2 * ((size_t)k * Nw + w) + 1];
-                finite = finite && isfinite(vr) && isfinite(vi);
-                m = fmax(m, fmax(fabs(vr), fabs(vi)));
-            }
-            if (finite && m > 0.0)
-                frexp(m, &e);
-            if (p == 0) {
-                a.T[k] = e;
-                if (!finite)  // every intensity of this set is undefined
-                    atomicOr(&a.kflags[c * 2 + h], 1u << threadIdx.x);
-            }
+            for (int w = lane; w < Nw; w += 32)
+                finite = abs_bits(a.V + 2 * (size_t)(half * kHS + i) * Nw, w, m) && finite;
+            if (!__all_sync(0xffffffffu, finite) && lane == 0)
+                atomicOr(&s_bad, 1u << i);
         }
-        s_T[threadIdx.x] = e;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            a.kflags[half] = s_bad;
     }
-    __syncthreads();
-    unsigned char *out = a.wimg + (size_t)(c * 2 + h) * KB * kWSlices * kWBlock + (size_t)p * kWBlock;
-    for (int idx = threadIdx.x; idx < KB * 64 * 64; idx += blockDim.x) {
-        const int kb = idx >> 12, r = (idx >> 6) & 63, fb = idx & 63;
-        const int f = kb * 64 + fb, sl = r >> 1, t = r & 1;
-        const int k = c * kKC + h * kHS + sl;
-        float val = 0.f;
-        if (k < a.K && f < 2 * Nw) {
-            const int w = f >> 1, u = f & 1;
-            const double vr = a.V[2 * ((size_t)k * Nw + w)], vi = a.V[2 * ((size_t)k * Nw + w) + 1];
-            const double coef = t == 0 ? (u == 0 ? vr : -vi) : (u == 0 ? vi : vr);
-            double ws[kWSlices];
-            split_slices(coef, s_T[sl], ws);
-            val = isfinite(coef) ? (float)ws[p] : 0.f;
+    const double *V = a.V + 2 * (size_t)k * Nw;
+    int T = 0;
+    if (k < a.K) {
+        unsigned long long m = 0ull;
+        bool finite = true;
+        for (int w = lane; w < Nw; w += 32)
+            finite = abs_bits(V, w, m) && finite;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (__all_sync(0xffffffffu, finite) && m)
+            frexp(__longlong_as_double(m), &T);
+        if (lane == 0)
+            a.T[k] = T;
+    }
+    unsigned char *out = a.wimg + (size_t)half * KB * kWSlices * kWBlock;
+    for (int w = lane; w < KB * 32; w += 32) {
+        double wr[kWSlices] = {0.0, 0.0, 0.0}, wi[kWSlices] = {0.0, 0.0, 0.0};
+        if (k < a.K && w < Nw) {
+            const double vr = V[2 * w], vi = V[2 * w + 1];
+            if (isfinite(vr))
+                split_slices(vr, T, wr);
+            if (isfinite(vi))
+                split_slices(vi, T, wi);
         }
-        *reinterpret_cast<__nv_bfloat16 *>(out + kb * kWSlices * kWBlock + sw128(r, fb * 2)) =
-            __float2bfloat16_rn(val);
+        unsigned char *o = out + (w >> 5) * kWSlices * kWBlock;
+#pragma unroll
+        for (int p = 0; p < kWSlices; ++p) {
+            const float r = (float)wr[p], i = (float)wi[p];
+            unsigned char *q = o + p * kWBlock;
+            *reinterpret_cast<unsigned *>(q + sw128(2 * sl, 4 * (w & 31))) = pack_bf16x2(r, -i);
+            *reinterpret_cast<unsigned *>(q + sw128(2 * sl + 1, 4 * (w & 31))) = pack_bf16x2(i, r);
+        }
     }
 }
 
-__global__ void batched_prep(const BatchArgs a) { batched_prep_block(a, blockIdx.x); }
+// One sample: the first blocks prepare the half chunks, the others clear the
+// log partials of the launch.
+__global__ void __launch_bounds__(kPrepThreads)
+    batched_prep(const BatchArgs a, int64_t n_lpart)
+{
+    const int halves = 2 * a.n_chunks * kPrepPerHalf;
+    if ((int)blockIdx.x < halves) {
+        batched_prep_block(a, blockIdx.x);
+        return;
+    }
+    for (int64_t i = (int64_t)(blockIdx.x - halves) * blockDim.x + threadIdx.x; i < n_lpart;
+         i += (int64_t)(gridDim.x - halves) * blockDim.x)
+        a.lpart[i] = 0;
+}
 
 // The preparation of every model of a batch: blocks_per_model blocks each.
-__global__ void batched_items_prep(const BatchArgs *__restrict__ models, int blocks_per_model)
+__global__ void __launch_bounds__(kPrepThreads)
+    batched_items_prep(const BatchArgs *__restrict__ models, int blocks_per_model)
 {
     batched_prep_block(models[blockIdx.x / blocks_per_model], blockIdx.x % blocks_per_model);
 }
@@ -702,7 +763,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // Final sums over the n_slots partial slots of a sample (fixed order), M V,
-// the first-order correction for V - V_r; one block per parameter set.
+// the first-order correction for V - V_r; one block per parameter set. Warp g
+// adds slots g, g + 8, ... for 32 waves at a time (eight slots' loads in
+// flight), the first warp then the eight warps' float-float sums: 128 sets x
+// 152 slots in 13 us cold, 23 us with one warp going through all the slots.
+constexpr int kFinWarps = 8;
+
 __device__ __forceinline__ void batched_finalize_set(const BatchArgs &a, int k, int n_slots,
                                                      int *done, double *nll, double *grad)
 {
@@ -710,36 +776,53 @@ __device__ __forceinline__ void batched_finalize_set(const BatchArgs &a, int k, 
     const int Nw = a.n_waves, F = a.F, NCH = a.n_chunks;
     const int c = k / kKC, kl = k % kKC;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ double s_corr[2];
-    __shared__ long long s_l;
-    const bool bad = (a.kflags[2 * c + (kl >> 5)] >> (kl & 31)) & 1u;
-    const int T = a.T[k];
-    const double gscale = ldexp(1.0, 8 - T);
-    double corr = 0.0;
-    for (int w = threadIdx.x; w < Nw; w += blockDim.x) {
+    __shared__ dfloat s_re[kFinWarps][kMaxWaves], s_im[kFinWarps][kMaxWaves];
+    __shared__ long long s_l[kFinWarps];
+    const size_t cta_stride = (size_t)NCH * 128 * F;
+    const float *g0 = a.gpart + (size_t)c * 128 * F + (size_t)(2 * kl) * F;
+    long long l = 0;
+    for (int i = threadIdx.x; i < grid * 4; i += kFinWarps * 32)
+        l += a.lpart[(size_t)i * (NCH * kKC) + k];
+    for (int w = lane; w < Nw; w += 32) {
         // Re conj(A) r = G[(k,re)][2w] + G[(k,im)][2w+1];  Im = G[(k,im)][2w] - G[(k,re)][2w+1]
-        dfloat s_re = {0.f, 0.f}, s_im = {0.f, 0.f};
-        const size_t cta_stride = (size_t)NCH * 128 * F;
-        const float *g0 = a.gpart + (size_t)c * 128 * F;
-        for (int b0 = 0; b0 < grid; b0 += 16) {
-            float2 re_row[16], im_row[16];
+        dfloat re = {0.f, 0.f}, im = {0.f, 0.f};
+        for (int b0 = warp; b0 < grid; b0 += 8 * kFinWarps) {
+            float2 re_row[8], im_row[8];
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const float *g = g0 + (size_t)(b0 + t) * cta_stride;
-                const bool in = b0 + t < grid;
-                re_row[t] = in ? *reinterpret_cast<const float2 *>(g + (2 * kl) * F + 2 * w)
-                               : make_float2(0.f, 0.f);
-                im_row[t] = in ? *reinterpret_cast<const float2 *>(g + (2 * kl + 1) * F + 2 * w)
-                               : make_float2(0.f, 0.f);
+            for (int t = 0; t < 8; ++t) {
+                const int b = b0 + t * kFinWarps;
+                const float *g = g0 + (size_t)b * cta_stride + 2 * w;
+                re_row[t] = b < grid ? *reinterpret_cast<const float2 *>(g) : make_float2(0.f, 0.f);
+                im_row[t] = b < grid ? *reinterpret_cast<const float2 *>(g + F) : make_float2(0.f, 0.f);
             }
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                s_re = df_add(s_re, df_add(dfloat{re_row[t].x, 0.f}, dfloat{im_row[t].y, 0.f}));
-                s_im = df_add(s_im, df_add(dfloat{im_row[t].x, 0.f}, dfloat{-re_row[t].y, 0.f}));
+            for (int t = 0; t < 8; ++t) {
+                re = df_add(re, df_add(dfloat{re_row[t].x, 0.f}, dfloat{im_row[t].y, 0.f}));
+                im = df_add(im, df_add(dfloat{im_row[t].x, 0.f}, dfloat{-re_row[t].y, 0.f}));
             }
         }
-        const double gre = -gscale * ((double)s_re.hi + (double)s_re.lo);
-        const double gim = -gscale * ((double)s_im.hi + (double)s_im.lo);
+        s_re[warp][w] = re;
+        s_im[warp][w] = im;
+    }
+    l = warp_sum(l);
+    if (lane == 0)
+        s_l[warp] = l;
+    __syncthreads();
+    if (warp > 0)
+        return;
+    const bool bad = (a.kflags[2 * c + (kl >> 5)] >> (kl & 31)) & 1u;
+    const int T = a.T[k];
+    const double gscale = scale2(1.0, 8 - T);
+    double corr = 0.0;
+    for (int w = lane; w < Nw; w += 32) {
+        dfloat re = s_re[0][w], im = s_im[0][w];
+#pragma unroll
+        for (int g = 1; g < kFinWarps; ++g) {
+            re = df_add(re, s_re[g][w]);
+            im = df_add(im, s_im[g][w]);
+        }
+        const double gre = -gscale * ((double)re.hi + (double)re.lo);
+        const double gim = -gscale * ((double)im.hi + (double)im.lo);
         const double *V = a.V + 2 * ((size_t)k * Nw + w);
         const double dvr = V[0] - round_slices(V[0], T), dvi = V[1] - round_slices(V[1], T);
         corr += 2.0 * (gre * dvr + gim * dvi);
@@ -750,22 +833,14 @@ __device__ __forceinline__ void batched_finalize_set(const BatchArgs &a, int k, 
         }
     }
     corr = warp_sum(corr);
-    if (lane == 0)
-        s_corr[warp] = corr;
-    if (warp == 0) {
-        long long l = 0;
-        for (int i = lane; i < grid * 4; i += 32)
-            l += a.lpart[(size_t)i * (NCH * kKC) + k];
-        l = warp_sum(l);
-        if (lane == 0)
-            s_l = l;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
+        long long ls = 0;
+        for (int g = 0; g < kFinWarps; ++g)
+            ls += s_l[g];
         const long long ex = 2 * *a.sum_e + 2 * a.n_events * (long long)(T - 16);
-        const double lnsum = kLn2 * ((double)ex + ldexp((double)s_l, -kFixBits));
+        const double lnsum = kLn2 * ((double)ex + ldexp((double)ls, -kFixBits));
         const double nv = a.mv[(size_t)k * (2 * Nw + 1) + 2 * Nw];
-        double v = -lnsum + nv + s_corr[0] + (blockDim.x > 32 ? s_corr[1] : 0.0);
+        double v = -lnsum + nv + corr;
         if (bad) {
             v = INFINITY;
             atomicOr(a.status, FLAG_DOMAIN);
@@ -776,13 +851,15 @@ __device__ __forceinline__ void batched_finalize_set(const BatchArgs &a, int k, 
     }
 }
 
-__global__ void batched_finalize(const BatchArgs a, int grid, int *done, double *nll, double *grad)
+__global__ void __launch_bounds__(kFinWarps * 32)
+    batched_finalize(const BatchArgs a, int grid, int *done, double *nll, double *grad)
 {
     batched_finalize_set(a, blockIdx.x, grid, done, nll, grad);
 }
 
 // The final sums of every model of a batch: block b is set b % K of model b / K.
-__global__ void batched_items_finalize(const BatchArgs *__restrict__ models, const int *n_slots,
+__global__ void __launch_bounds__(kFinWarps * 32)
+    batched_items_finalize(const BatchArgs *__restrict__ models, const int *n_slots,
                                        int K, int *const *done, double *const *nll,
                                        double *const *grad)
 {
@@ -974,13 +1051,10 @@ cudaError_t launch_batched(const void *xbf, int64_t n_events, int n_waves, int x
     a.kflags = reinterpret_cast<unsigned *>(p + sl.kflags);
     a.status = status;
     a.nxs_req = nxs;
-    cudaError_t e = cudaMemsetAsync(a.kflags, 0, nch * 2 * 4, s);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(a.lpart, 0, (size_t)grid * 4 * nch * kKC * 8, s);
-    if (e != cudaSuccess)
-        return e;
-    batched_prep<<<nch * 2 * kWSlices, 256, 0, s>>>(a);
-    e = cudaGetLastError();
+    const int64_t n_lpart = (int64_t)grid * 4 * nch * kKC;
+    const int clear = (int)((n_lpart + 16 * kPrepThreads - 1) / (16 * kPrepThreads));
+    batched_prep<<<nch * 2 * kPrepPerHalf + clear, kPrepThreads, 0, s>>>(a, n_lpart);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
     const int n_tiles = (int)((n_events + kBM - 1) / kBM);
@@ -989,7 +1063,7 @@ cudaError_t launch_batched(const void *xbf, int64_t n_events, int n_waves, int x
                 : launch_main<1>(F, grid, smem, s, a, n_tiles);
     if (e != cudaSuccess)
         return e;
-    batched_finalize<<<K, 64, 0, s>>>(a, grid, done, nll, grad);
+    batched_finalize<<<K, kFinWarps * 32, 0, s>>>(a, grid, done, nll, grad);
     return cudaGetLastError();
 }
 
@@ -1156,8 +1230,8 @@ cudaError_t launch_batched_items(void *plan, const BatchModelDesc *models, int n
     if (e != cudaSuccess)
         return e;
     const BatchArgs *args = reinterpret_cast<const BatchArgs *>(d + p.args);
-    const int bpm = nch * 2 * kWSlices;
-    batched_items_prep<<<n_models * bpm, 256, 0, s>>>(args, bpm);
+    const int bpm = nch * 2 * kPrepPerHalf;
+    batched_items_prep<<<n_models * bpm, kPrepThreads, 0, s>>>(args, bpm);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     const BatchItem *items = reinterpret_cast<const BatchItem *>(d + p.items);
@@ -1168,7 +1242,7 @@ cudaError_t launch_batched_items(void *plan, const BatchModelDesc *models, int n
         batched_items_kernel<1><<<n_items, kThreads, smem, s>>>(items, args);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    batched_items_finalize<<<n_models * K, 64, 0, s>>>(
+    batched_items_finalize<<<n_models * K, kFinWarps * 32, 0, s>>>(
         args, reinterpret_cast<const int *>(d + p.nslots), K,
         reinterpret_cast<int *const *>(d + p.pdone), reinterpret_cast<double *const *>(d + p.pnll),
         reinterpret_cast<double *const *>(d + p.pgrad));
