@@ -10,8 +10,11 @@
 // One persistent CTA per SM streams tiles of 192 events x (1 + 2n) rows (m,
 // then Re/Im of Y_r for the free waves r < R and of A_a for the fixed waves)
 // from both samples, the data tiles first, into a ring of shared-memory
-// stages with TMA; two groups of three consumer warps take tiles in turn, each
-// thread two adjacent events packed in FP32x2 registers:
+// stages with TMA. Two groups take tiles in turn; a tile is three units of 64
+// events, two adjacent ones per lane packed in FP32x2 registers. A unit has two
+// gradient warps (even and odd waves), which keep the sums of its events over
+// all its tiles; twelve S warps, which take the units' S in turn, run ahead of
+// them and hand them w_i S_i through shared memory:
 //  * BW_r per event with the exact-pair denominator of the per-event kernel
 //    (M^2, M G, (M G)^2 as float pairs, m^2 and D^2 split by FMA, a Newton
 //    step of the reciprocal against the pair), then A_r = BW_r Y_r;
@@ -22,8 +25,17 @@
 //    for the free waves;
 //  * ln I = e ln 2 + ln f, e and round(2^23 ln f) summed as integers; the MC
 //    sum of I and all gradients in FP32 per thread, float-float per warp and
-//    block, FP64 across blocks in block order (the last CTA, atomic ticket).
+//    block, FP64 across blocks in a fixed order (the last CTA, atomic ticket).
 // Every wait is bounded (FLAG_TIMEOUT) so a stalled pipeline returns.
+//
+// Bound by the FP32 pipe's latency before HBM: with both passes in one warp per
+// unit (seven warps per SM at 255 registers) 36% of the issue slots were used.
+// Twelve S warps and twelve gradient warps (72 registers) keep every sum's
+// order. Per call at 2M + 5M events x 20 waves, 4 free: 303 us (3.8 TB/s), 373
+// before; six and six warps 330, nine and six 315, fifteen and twelve 303. At 12
+// waves, 3 free 229 (279), at 28 and 4, 1M + 2.5M events 252 (291). Splitting a
+// unit's waves over two warps in the S pass too changes the order of S's
+// remainders and with it the last digits of the gradients (3.6e-9).
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -34,21 +46,28 @@ constexpr int kMaxFreeT = 8;
 
 template <int NP, int RP>
 struct ResTmaCfg {
-    static constexpr int G = 2;                     // consumer groups
-    static constexpr int GW = 3;                    // warps per group (7 warps in all: the
-                                                    // register cap is then 255, not 168)
-    static constexpr int CW = G * GW;
+    static constexpr int G = 2;                     // groups (tiles in turn)
+    static constexpr int GW = 3;                    // units (64 events) per tile
+    static constexpr int UNITS = G * GW;
+    static constexpr int GH = 2;                    // gradient warps per unit: even and odd waves
+    static constexpr int NH = NP / GH, RH = RP / GH;
+    static constexpr int SR = 4;                    // S warps per unit of a tile: every SR-th tile each
+    static constexpr int SWARPS = SR * GW;
     static constexpr int TE = GW * 32 * 2;          // events per tile
     static constexpr int ROWS = 1 + 2 * NP;
     static constexpr uint32_t STAGE_BYTES = ROWS * TE * 4;
     static constexpr int SPG_RAW = (200 * 1024) / (STAGE_BYTES * G);
     static constexpr int SPG = SPG_RAW < 1 ? 1 : (SPG_RAW > 4 ? 4 : SPG_RAW);
     static constexpr int STAGES = G * SPG;
-    static constexpr int THREADS = (CW + 1) * 32;      // + the producer warp
-    static constexpr int NR = 4 + 2 * NP + 2 * RP;  // per-warp float partials
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 2 * STAGES * sizeof(uint64_t);
-    // dynamic shared memory must leave room for the static arrays (< 8 KB)
-    static constexpr bool FITS = SMEM <= 210 * 1024;
+    static constexpr int THREADS = (1 + SWARPS + GH * UNITS) * 32;  // + the producer warp
+    static constexpr int NR = 2 * NP + 2 * RP;      // per-unit float partials
+    // the ring, then the weights w S of a stage's events (16 bytes per lane)
+    static constexpr size_t RING_BYTES = (size_t)STAGES * STAGE_BYTES;
+    static constexpr size_t WS_BYTES = (size_t)STAGES * GW * 32 * 16;
+    static constexpr size_t SMEM =
+        RING_BYTES + WS_BYTES + (2 + GW) * STAGES * sizeof(uint64_t);
+    static constexpr size_t STATIC_BYTES = 32 * NP + 64 * RP + 8 * NR * UNITS + 32 * SWARPS + 256;
+    static constexpr bool FITS = SMEM + STATIC_BYTES <= 227 * 1024;
 };
 
 struct ResWave {
@@ -87,17 +106,20 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
                        const ResArgs a, const float *amax, int tiles_d, int tiles_m)
 {
     using C = ResTmaCfg<NP, RP>;
-    constexpr int TE = C::TE, ROWS = C::ROWS, STAGES = C::STAGES, GW = C::GW, CW = C::CW, NR = C::NR;
+    constexpr int TE = C::TE, ROWS = C::ROWS, STAGES = C::STAGES, GW = C::GW, NR = C::NR;
+    constexpr int UNITS = C::UNITS, SWARPS = C::SWARPS, GH = C::GH, NH = C::NH, RH = C::RH;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *tiles = reinterpret_cast<float *>(smem_raw);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + (size_t)STAGES * C::STAGE_BYTES);
-    uint64_t *empty = full + STAGES;
+    float4 *ws = reinterpret_cast<float4 *>(smem_raw + C::RING_BYTES);  // [STAGES][GW][32]
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + C::RING_BYTES + C::WS_BYTES);
+    uint64_t *empty = full + STAGES, *wfull = empty + STAGES;           // wfull [STAGES][GW]
 
     __shared__ ResWave Vc[NP];
     __shared__ ResFree Fr[RP];
     __shared__ float s_sigma, s_unit;
-    __shared__ long long red_i[CW][2];
-    __shared__ float red_f[2][CW][NR];
+    __shared__ long long red_i[SWARPS][2];   // data: sums of round(2^23 ln f) and exponents
+    __shared__ float red_s[2][SWARPS][2];    // remainders of 2^23 ln f (data), I (MC)
+    __shared__ float red_f[2][UNITS][NR];    // gradients
     __shared__ int s_flags, s_last;
 
     const int N = a.n_waves, R = a.n_free;
@@ -120,7 +142,9 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], GW);
+            mbar_init(&empty[s], (1 + C::GH) * GW);
+            for (int k = 0; k < GW; ++k)
+                mbar_init(&wfull[s * GW + k], 1);
         }
         fence_barrier_init();
         s_flags = 0;
@@ -199,207 +223,248 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
                 if (!mbar_wait(&full[stage_of(q)], use_of(q) & 1))
                     flags |= FLAG_TIMEOUT;
         }
-    } else if (warp <= CW) {
-        // ---- consumers: group grp takes tiles j = grp, grp + G, ... ----------
-        const int cw = warp - 1;
-        const int grp = cw / GW;
-        const int ct = (cw % GW) * 32 + lane;
-        const float sigma = s_sigma, unit = s_unit;
-        const f2 SG = pk2(sigma, sigma), Z = 0ull, ONE = pk2(1.f, 1.f);
-        const unsigned im_offset = 2u * (unsigned)NP * __float_as_uint(sigma);
-        float gs[2 * NP];
-        f2 gm[RP], gw[RP];
-        long long l_int = 0;
-        int eacc = 0;
-        dfloat acc = {0.f, 0.f};  // data: remainders of 2^23 ln f; MC: sum of I
-        int bad = 0;
-        auto reset = [&]() {
-#pragma unroll
-            for (int c = 0; c < 2 * NP; ++c)
-                gs[c] = 0.f;
-#pragma unroll
-            for (int r = 0; r < RP; ++r)
-                gm[r] = gw[r] = Z;
-            l_int = 0;
-            eacc = 0;
-            acc = dfloat{0.f, 0.f};
+    } else {
+        // ---- S warps, then the gradient warps: unit u is 64 events, ug = u % GW, of
+        // the tiles of group u / GW, its warp gh takes waves gh, gh + GH, ... ----------
+        const bool s_warp = warp <= SWARPS;
+        const int sw = warp - 1, gi = warp - 1 - SWARPS, u = gi / GH, gh = gi % GH;
+        const int ug = (s_warp ? sw : u) % GW, ct = ug * 32 + lane;
+        const f2 Z = 0ull, ONE = pk2(1.f, 1.f);
+        // BW_r(m) of the two events, formed by either warp for itself
+        auto bw = [&](int r, f2 mm, f2 me, f2 &br, f2 &bi) {
+            const ResFree &f = Fr[r];
+            const f2 D = add2(sub2(f.m2h, mm), sub2(f.m2l, me));
+            // den = D^2 + (M G)^2 as the pair dh + dl (see the per-event kernel)
+            const f2 p = mul2(D, D), pe = fma2(D, D, neg2(p));
+            const f2 dh = add2(f.g2h, p), bb = sub2(dh, f.g2h);
+            const f2 dl = add2(add2(add2(sub2(f.g2h, sub2(dh, bb)), sub2(p, bb)), pe), f.g2l);
+            const f2 q0 = rcp2(dh);
+            const f2 q = fma2(q0, fma2(neg2(dl), q0, fma2(neg2(dh), q0, ONE)), q0);
+            br = mul2(D, q);
+            bi = fma2(f.gh, q, mul2(f.gl, q));
         };
-        // per-warp sums of this thread's accumulators for a phase (fixed order)
-        auto flush = [&](int ph) {
-            const dfloat aw = warp_sum(acc);
-            const long long li = warp_sum(l_int), ei = warp_sum((long long)eacc);
-            if (lane == 0) {
-                red_f[ph][cw][0] = aw.hi;
-                red_f[ph][cw][1] = aw.lo;
-                if (ph == 0) {
-                    red_i[cw][0] = li;
-                    red_i[cw][1] = ei;
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 2 * NP; ++c) {
-                const float v = warp_sum(gs[c]);
-                if (lane == 0)
-                    red_f[ph][cw][4 + c] = v;
-            }
-#pragma unroll
-            for (int r = 0; r < RP; ++r) {
-                float m0, m1, w0, w1;
-                upk2(gm[r], m0, m1);
-                upk2(gw[r], w0, w1);
-                const float vm = warp_sum(m0 + m1), vw = warp_sum(w0 + w1);
-                if (lane == 0) {
-                    red_f[ph][cw][4 + 2 * NP + r] = vm;
-                    red_f[ph][cw][4 + 2 * NP + RP + r] = vw;
-                }
+        // amplitude pair of wave w: A_w from the tile, or BW_w Y_w for a free wave
+        // (free waves are among the first RP: `maybe_free` is known at compile time)
+        auto amp = [&](const float *T, f2 mm, f2 me, int w, bool maybe_free, f2 &ar, f2 &ai, f2 &br,
+                       f2 &bi) {
+            ar = lds2r(T + (1 + 2 * w) * TE);
+            ai = lds2r(T + (2 + 2 * w) * TE);
+            if (maybe_free && w < R) {
+                bw(w, mm, me, br, bi);
+                const f2 yr = ar, yi = ai;
+                ar = fma2(br, yr, neg2(mul2(bi, yi)));
+                ai = fma2(br, yi, mul2(bi, yr));
             }
         };
-        reset();
         int phase = 0;
-        for (int j = grp; j < n_my; j += C::G) {
-            const int t = (int)blockIdx.x + j * (int)gridDim.x;
-            const int ph = t < tiles_d ? 0 : 1;
-            if (ph != phase) {  // every data tile of this CTA precedes its MC tiles
-                flush(0);
-                reset();
-                phase = 1;
-            }
-            const int s = stage_of(j);
-            if (!mbar_wait(&full[s], use_of(j) & 1)) {
-                flags |= FLAG_TIMEOUT;
-                break;
-            }
-            const float *T = tiles + (size_t)s * ROWS * TE + 2 * ct;
-            const int64_t ev0 = (int64_t)(ph ? t - tiles_d : t) * TE + 2 * ct;
-            const int64_t n_ph = ph ? a.n_mc : a.n_data;
-
-            // free waves: BW_r(m) for the two events, computed where needed (in
-            // the S pass and again in the gradient pass) rather than held in
-            // registers across the pass over the waves
-            const f2 m = lds2r(T);
-            const f2 mm = mul2(m, m), me = fma2(m, m, neg2(mm));  // m^2 = mm + me exactly
-            auto bw = [&](int r, f2 &br, f2 &bi) {
-                const ResFree &f = Fr[r];
-                const f2 D = add2(sub2(f.m2h, mm), sub2(f.m2l, me));
-                // den = D^2 + (M G)^2 as the pair dh + dl (see the per-event kernel)
-                const f2 p = mul2(D, D), pe = fma2(D, D, neg2(p));
-                const f2 dh = add2(f.g2h, p), bb = sub2(dh, f.g2h);
-                const f2 dl = add2(add2(add2(sub2(f.g2h, sub2(dh, bb)), sub2(p, bb)), pe), f.g2l);
-                const f2 q0 = rcp2(dh);
-                const f2 q = fma2(q0, fma2(neg2(dl), q0, fma2(neg2(dh), q0, ONE)), q0);
-                br = mul2(D, q);
-                bi = fma2(f.gh, q, mul2(f.gl, q));
-            };
-            // amplitude pair of wave w: A_w from the tile, or BW_w Y_w for a free wave
-            auto amp = [&](int w, f2 &ar, f2 &ai, f2 &br, f2 &bi) {
-                ar = lds2r(T + (1 + 2 * w) * TE);
-                ai = lds2r(T + (2 + 2 * w) * TE);
-                if (w < RP && w < R) {
-                    bw(w, br, bi);
-                    const f2 yr = ar, yi = ai;
-                    ar = fma2(br, yr, neg2(mul2(bi, yi)));
-                    ai = fma2(br, yi, mul2(bi, yr));
-                }
-            };
-            // S, exact product split (Re S = vr ar - vi ai, Im S = vr ai + vi ar)
-            unsigned hR0 = 0, hR1 = 0, hI0 = 0, hI1 = 0;
-            f2 lR = Z, lRm = Z, lI = Z;
-#pragma unroll
-            for (int w = 0; w < NP; ++w) {
-                f2 ar, ai, br, bi;
-                amp(w, ar, ai, br, bi);
-                const ResWave cf = Vc[w];
-                unsigned x0, x1;
-                lR = add2(lR, extract2(cf.vr, ar, SG, x0, x1));
-                hR0 += x0;
-                hR1 += x1;
-                lRm = add2(lRm, extract2(cf.vi, ai, SG, x0, x1));
-                hR0 -= x0;
-                hR1 -= x1;
-                lI = add2(lI, extract2(cf.vr, ai, SG, x0, x1));
-                hI0 += x0;
-                hI1 += x1;
-                lI = add2(lI, extract2(cf.vi, ar, SG, x0, x1));
-                hI0 += x0;
-                hI1 += x1;
-                lR = fma2(cf.lr, ar, lR);
-                lRm = fma2(cf.li, ai, lRm);
-                lI = fma2(cf.lr, ai, fma2(cf.li, ar, lI));
-            }
-            float Sr[2], Si[2], wr[2], wi[2];
-            {
-                const f2 hR = pk2((float)(int)hR0 * unit, (float)(int)hR1 * unit);
-                const f2 hI = pk2((float)(int)(hI0 - im_offset) * unit,
-                                  (float)(int)(hI1 - im_offset) * unit);
-                upk2(add2(hR, sub2(lR, lRm)), Sr[0], Sr[1]);
-                upk2(add2(hI, lI), Si[0], Si[1]);
-            }
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                wr[e] = wi[e] = 0.f;
-                if (ev0 + e < n_ph) {
-                    const float I = fmaf(Sr[e], Sr[e], Si[e] * Si[e]);
+        if (s_warp) {
+            // ---- S, ln I or I, and w S of the events ug of tiles j = sw / GW mod SR.
+            // Each warp waits for every tile's copy, its own or not, so that its parity
+            // waits follow the stages' uses one by one.
+            const float sigma = s_sigma, unit = s_unit;
+            const f2 SG = pk2(sigma, sigma);
+            const unsigned im_offset = 2u * (unsigned)NP * __float_as_uint(sigma);
+            long long l_int = 0;
+            int eacc = 0;
+            dfloat acc = {0.f, 0.f};  // data: remainders of 2^23 ln f; MC: sum of I
+            int bad = 0;
+            auto flush = [&](int ph) {
+                const dfloat aw = warp_sum(acc);
+                const long long li = warp_sum(l_int), ei = warp_sum((long long)eacc);
+                if (lane == 0) {
+                    red_s[ph][sw][0] = aw.hi;
+                    red_s[ph][sw][1] = aw.lo;
                     if (ph == 0) {
-                        if (I > 0.f && I < INFINITY) {
-                            int ex;
-                            const float f = split_exponent(I, ex);
-                            const float y = logf(f) * 8388608.0f;
-                            const float tt = y + 12582912.0f;
-                            l_int += __float_as_int(tt) - 0x4B400000;
-                            acc = df_add(acc, dfloat{y - (tt - 12582912.0f), 0.f});
-                            eacc += ex;
-                            const float rI = -__frcp_rn(I);
-                            wr[e] = Sr[e] * rI;
-                            wi[e] = Si[e] * rI;
-                        } else {
-                            bad = 1;
-                        }
-                    } else {
-                        acc = df_add(acc, dfloat{I, 0.f});
-                        wr[e] = Sr[e];
-                        wi[e] = Si[e];
+                        red_i[sw][0] = li;
+                        red_i[sw][1] = ei;
                     }
                 }
-            }
-            const f2 WR = pk2(wr[0], wr[1]), WI = pk2(wi[0], wi[1]);
+                l_int = 0;
+                eacc = 0;
+                acc = dfloat{0.f, 0.f};
+            };
+            for (int j = 0; j < n_my; ++j) {
+                const int s = stage_of(j);
+                if (!mbar_wait(&full[s], use_of(j) & 1)) {
+                    flags |= FLAG_TIMEOUT;
+                    break;
+                }
+                if (j % C::SR != sw / GW)
+                    continue;
+                const int t = (int)blockIdx.x + j * (int)gridDim.x;
+                const int ph = t < tiles_d ? 0 : 1;
+                if (ph != phase) {  // every data tile of this CTA precedes its MC tiles
+                    flush(0);
+                    phase = 1;
+                }
+                const float *T = tiles + (size_t)s * ROWS * TE + 2 * ct;
+                const int64_t ev0 = (int64_t)(ph ? t - tiles_d : t) * TE + 2 * ct;
+                const int64_t n_ph = ph ? a.n_mc : a.n_data;
+                const f2 m = lds2r(T);
+                const f2 mm = mul2(m, m), me = fma2(m, m, neg2(mm));  // m^2 = mm + me exactly
+                // S, exact product split (Re S = vr ar - vi ai, Im S = vr ai + vi ar)
+                unsigned hR0 = 0, hR1 = 0, hI0 = 0, hI1 = 0;
+                f2 lR = Z, lRm = Z, lI = Z;
 #pragma unroll
-            for (int w = 0; w < NP; ++w) {
-                f2 ar, ai, br, bi;
-                amp(w, ar, ai, br, bi);
-                // gradient in V: conj(A) (wr + i wi) = (ar wr + ai wi) + i (ar wi - ai wr)
-                float a0, a1, b0, b1;
-                upk2(ar, a0, a1);
-                upk2(ai, b0, b1);
-                gs[2 * w] = fmaf(a0, wr[0], fmaf(b0, wi[0], gs[2 * w]));
-                gs[2 * w] = fmaf(a1, wr[1], fmaf(b1, wi[1], gs[2 * w]));
-                gs[2 * w + 1] = fmaf(a0, wi[0], fmaf(-b0, wr[0], gs[2 * w + 1]));
-                gs[2 * w + 1] = fmaf(a1, wi[1], fmaf(-b1, wr[1], gs[2 * w + 1]));
-                // masses and widths: c = conj(w S) (V_r A_r BW_r) per event, then
-                // dM += -4 M Re c - 2 G Im c, dG += -2 M Im c
-                if (w < RP && w < R) {
+                for (int w = 0; w < NP; ++w) {
+                    f2 ar, ai, br, bi;
+                    amp(T, mm, me, w, w < RP, ar, ai, br, bi);
                     const ResWave cf = Vc[w];
-                    const f2 tr = fma2(cf.vr, ar, neg2(mul2(cf.vi, ai)));
-                    const f2 ti = fma2(cf.vr, ai, mul2(cf.vi, ar));
-                    const f2 ur = fma2(tr, br, neg2(mul2(ti, bi)));
-                    const f2 ui = fma2(tr, bi, mul2(ti, br));
-                    const f2 cr = fma2(WR, ur, mul2(WI, ui)), ci = fma2(WR, ui, neg2(mul2(WI, ur)));
-                    const float Mf = Fr[w].mf, Gf = Fr[w].wf;
-                    gm[w] = fma2(pk2(-4.f * Mf, -4.f * Mf), cr,
-                                 fma2(pk2(-2.f * Gf, -2.f * Gf), ci, gm[w]));
-                    gw[w] = fma2(pk2(-2.f * Mf, -2.f * Mf), ci, gw[w]);
+                    unsigned x0, x1;
+                    lR = add2(lR, extract2(cf.vr, ar, SG, x0, x1));
+                    hR0 += x0;
+                    hR1 += x1;
+                    lRm = add2(lRm, extract2(cf.vi, ai, SG, x0, x1));
+                    hR0 -= x0;
+                    hR1 -= x1;
+                    lI = add2(lI, extract2(cf.vr, ai, SG, x0, x1));
+                    hI0 += x0;
+                    hI1 += x1;
+                    lI = add2(lI, extract2(cf.vi, ar, SG, x0, x1));
+                    hI0 += x0;
+                    hI1 += x1;
+                    lR = fma2(cf.lr, ar, lR);
+                    lRm = fma2(cf.li, ai, lRm);
+                    lI = fma2(cf.lr, ai, fma2(cf.li, ar, lI));
+                }
+                float Sr[2], Si[2], wr[2], wi[2];
+                {
+                    const f2 hR = pk2((float)(int)hR0 * unit, (float)(int)hR1 * unit);
+                    const f2 hI = pk2((float)(int)(hI0 - im_offset) * unit,
+                                      (float)(int)(hI1 - im_offset) * unit);
+                    upk2(add2(hR, sub2(lR, lRm)), Sr[0], Sr[1]);
+                    upk2(add2(hI, lI), Si[0], Si[1]);
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    wr[e] = wi[e] = 0.f;
+                    if (ev0 + e < n_ph) {
+                        const float I = fmaf(Sr[e], Sr[e], Si[e] * Si[e]);
+                        if (ph == 0) {
+                            if (I > 0.f && I < INFINITY) {
+                                int ex;
+                                const float f = split_exponent(I, ex);
+                                const float y = logf(f) * 8388608.0f;
+                                const float tt = y + 12582912.0f;
+                                l_int += __float_as_int(tt) - 0x4B400000;
+                                acc = df_add(acc, dfloat{y - (tt - 12582912.0f), 0.f});
+                                eacc += ex;
+                                const float rI = -__frcp_rn(I);
+                                wr[e] = Sr[e] * rI;
+                                wi[e] = Si[e] * rI;
+                            } else {
+                                bad = 1;
+                            }
+                        } else {
+                            acc = df_add(acc, dfloat{I, 0.f});
+                            wr[e] = Sr[e];
+                            wi[e] = Si[e];
+                        }
+                    }
+                }
+                ws[(s * GW + ug) * 32 + lane] = make_float4(wr[0], wr[1], wi[0], wi[1]);
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&wfull[s * GW + ug]);
+                    mbar_arrive(&empty[s]);
                 }
             }
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&empty[s]);
-        }
-        if (bad)
-            flags |= FLAG_DOMAIN;
-        if (phase == 0) {  // this group saw no MC tile: its MC sums are zero
-            flush(0);
+            if (bad)
+                flags |= FLAG_DOMAIN;
+            if (phase == 0)  // no MC tile of its own: its MC sums are zero
+                flush(0);
+            flush(1);
+        } else {
+            // ---- gradients: each thread adds up its two events of every tile for its
+            // half of the waves
+            float gs[2 * NH];
+            f2 gm[RH], gw[RH];
+            auto reset = [&]() {
+#pragma unroll
+                for (int c = 0; c < 2 * NH; ++c)
+                    gs[c] = 0.f;
+#pragma unroll
+                for (int r = 0; r < RH; ++r)
+                    gm[r] = gw[r] = Z;
+            };
+            // per-warp sums of this thread's accumulators for a phase (fixed order)
+            auto flush = [&](int ph) {
+#pragma unroll
+                for (int c = 0; c < 2 * NH; ++c) {
+                    const float v = warp_sum(gs[c]);
+                    if (lane == 0)
+                        red_f[ph][u][2 * (GH * (c / 2) + gh) + (c & 1)] = v;
+                }
+#pragma unroll
+                for (int r = 0; r < RH; ++r) {
+                    float m0, m1, w0, w1;
+                    upk2(gm[r], m0, m1);
+                    upk2(gw[r], w0, w1);
+                    const float vm = warp_sum(m0 + m1), vw = warp_sum(w0 + w1);
+                    if (lane == 0) {
+                        red_f[ph][u][2 * NP + GH * r + gh] = vm;
+                        red_f[ph][u][2 * NP + RP + GH * r + gh] = vw;
+                    }
+                }
+            };
             reset();
+            for (int j = u / GW; j < n_my; j += C::G) {
+                const int s = stage_of(j);
+                const int ph = (int)blockIdx.x + j * (int)gridDim.x < tiles_d ? 0 : 1;
+                if (ph != phase) {
+                    flush(0);
+                    reset();
+                    phase = 1;
+                }
+                if (!mbar_wait(&full[s], use_of(j) & 1) ||
+                    !mbar_wait(&wfull[s * GW + ug], use_of(j) & 1)) {
+                    flags |= FLAG_TIMEOUT;
+                    break;
+                }
+                const float *T = tiles + (size_t)s * ROWS * TE + 2 * ct;
+                const f2 m = lds2r(T);
+                const f2 mm = mul2(m, m), me = fma2(m, m, neg2(mm));
+                const float4 w4 = ws[(s * GW + ug) * 32 + lane];
+                const float wr[2] = {w4.x, w4.y}, wi[2] = {w4.z, w4.w};
+                const f2 WR = pk2(wr[0], wr[1]), WI = pk2(wi[0], wi[1]);
+#pragma unroll
+                for (int i = 0; i < NH; ++i) {
+                    const int w = GH * i + gh;
+                    f2 ar, ai, br, bi;
+                    amp(T, mm, me, w, i < RH, ar, ai, br, bi);
+                    // gradient in V: conj(A) (wr + i wi) = (ar wr + ai wi) + i (ar wi - ai wr)
+                    float a0, a1, b0, b1;
+                    upk2(ar, a0, a1);
+                    upk2(ai, b0, b1);
+                    gs[2 * i] = fmaf(a0, wr[0], fmaf(b0, wi[0], gs[2 * i]));
+                    gs[2 * i] = fmaf(a1, wr[1], fmaf(b1, wi[1], gs[2 * i]));
+                    gs[2 * i + 1] = fmaf(a0, wi[0], fmaf(-b0, wr[0], gs[2 * i + 1]));
+                    gs[2 * i + 1] = fmaf(a1, wi[1], fmaf(-b1, wr[1], gs[2 * i + 1]));
+                    // masses and widths: c = conj(w S) (V_r A_r BW_r) per event, then
+                    // dM += -4 M Re c - 2 G Im c, dG += -2 M Im c
+                    if (i < RH && w < R) {
+                        const ResWave cf = Vc[w];
+                        const f2 tr = fma2(cf.vr, ar, neg2(mul2(cf.vi, ai)));
+                        const f2 ti = fma2(cf.vr, ai, mul2(cf.vi, ar));
+                        const f2 ur = fma2(tr, br, neg2(mul2(ti, bi)));
+                        const f2 ui = fma2(tr, bi, mul2(ti, br));
+                        const f2 cr = fma2(WR, ur, mul2(WI, ui)), ci = fma2(WR, ui, neg2(mul2(WI, ur)));
+                        const float Mf = Fr[w].mf, Gf = Fr[w].wf;
+                        gm[i < RH ? i : 0] = fma2(pk2(-4.f * Mf, -4.f * Mf), cr,
+                                     fma2(pk2(-2.f * Gf, -2.f * Gf), ci, gm[i < RH ? i : 0]));
+                        gw[i < RH ? i : 0] = fma2(pk2(-2.f * Mf, -2.f * Mf), ci, gw[i < RH ? i : 0]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&empty[s]);
+            }
+            if (phase == 0) {  // this group saw no MC tile: its MC sums are zero
+                flush(0);
+                reset();
+            }
+            flush(1);
         }
-        flush(1);
     }
     if (flags)
         atomicOr(&s_flags, flags);
@@ -411,29 +476,30 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
         const int ph = item / P, c = item % P;
         double v = 0.0;
         if (c == 0) {
-            for (int w = 0; w < CW; ++w)
-                v += (double)red_f[ph][w][0] + (double)red_f[ph][w][1];
+            for (int w = 0; w < SWARPS; ++w)
+                v += (double)red_s[ph][w][0] + (double)red_s[ph][w][1];
             if (ph == 0) {
                 long long li = 0;
-                for (int w = 0; w < CW; ++w)
+                for (int w = 0; w < SWARPS; ++w)
                     li += red_i[w][0];
                 v = ((double)li + v) * 0x1p-23;   // sum of ln f
             }
         } else if (c == 1) {
             if (ph == 0) {
                 long long ei = 0;
-                for (int w = 0; w < CW; ++w)
+                for (int w = 0; w < SWARPS; ++w)
                     ei += red_i[w][1];
                 v = (double)ei;                    // sum of exponents
             }
         } else {
             const int k = c - 2;  // gradient V (2N), then dM (R), dG (R)
-            const int col = k < 2 * N ? 4 + k : (k < 2 * N + R ? 4 + 2 * NP + (k - 2 * N)
-                                                               : 4 + 2 * NP + RP + (k - 2 * N - R));
-            for (int w = 0; w < CW; ++w)
+            const int col = k < 2 * N ? k
+                            : k < 2 * N + R ? 2 * NP + (k - 2 * N)
+                                            : 2 * NP + RP + (k - 2 * N - R);
+            for (int w = 0; w < UNITS; ++w)
                 v += (double)red_f[ph][w][col];
         }
-        a.partials[((size_t)blockIdx.x * 2 + ph) * P + c] = v;
+        a.partials[(size_t)item * gridDim.x + blockIdx.x] = v;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -446,15 +512,17 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     __syncthreads();
     if (!s_last)
         return;
-    // ---- last CTA: sums over CTAs in block order, FP64 -----------------------
+    // ---- last CTA: sums over CTAs in FP64, a warp per value (lane k adds CTAs
+    // k, k + 32, ..., then a fixed shuffle tree) ---------------------------------
     __threadfence();
     double *fin = reinterpret_cast<double *>(tiles);   // the ring is idle now
-    for (int item = threadIdx.x; item < 2 * P; item += blockDim.x) {
-        const int ph = item / P, c = item % P;
+    for (int item = warp; item < 2 * P; item += blockDim.x / 32) {
         double v = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b)
-            v += __ldcg(a.partials + ((size_t)b * 2 + ph) * P + c);
-        fin[item] = v;
+        for (int b = lane; b < (int)gridDim.x; b += 32)
+            v += __ldcg(a.partials + (size_t)item * gridDim.x + b);
+        v = warp_sum(v);
+        if (lane == 0)
+            fin[item] = v;
     }
     __syncthreads();
     const int st = *(volatile int *)a.status;
