@@ -7,19 +7,19 @@
 // are dropped in both terms of Eq. 3 (they cancel in expectation at the
 // minimum), leaving
 //   H = sum_i d_i d_i^T,   d_i = grad_p ln I_i = 2 (Re, Im) of conj(A_a(i)) S_i / I_i.
-// Each thread forms d_i of one event (S by a compensated dot product with V
-// as a float pair) into a shared-memory tile J of 256 events x 2NP columns
-// (Re parts at 0..NP-1, Im parts at NP..2NP-1, zero-padded). The upper
-// triangle of J^T J is cut into 4x4 blocks; each thread owns one to three
-// (block, event group) items and accumulates 16 products per pair of float4
-// loads. FP32 within a run of tiles, float-float across runs, FP64 across
-// event groups and blocks, summed in a fixed order. This kernel serves
-// samples of more than 20 waves (and PWA_HESS_KERNEL=generic); up to 20
-// waves the tensor-core kernel of k_hess_tc.cu forms the same sum.
+// One half of a block's warps forms d_i, one event to a thread (S by a
+// compensated dot product with V as a float pair), into a shared-memory tile J
+// of 256 events x 2NP columns (Re parts at 0..NP-1, Im parts at NP..2NP-1,
+// zero-padded), one tile ahead of the other half, which adds up the upper
+// triangle of J^T J in 8x8 blocks over event groups: FP32 within a run of tiles,
+// float pairs across runs, event groups and blocks, summed in a fixed order. This kernel serves samples of
+// more than 20 waves (and PWA_HESS_KERNEL=generic); up to 20 waves the tensor-
+// core kernel of k_hess_tc.cu forms the same sum.
 //
 // Projection weights: w_j = I(Omega_j) / N_gen per accepted MC event (their
 // sum is V^H M V), and fit fractions F_ab = Re(conj(V_a) M_ab V_b) / V^H M V.
 #include "amp_kernel.cuh"
+#include "ff.cuh"
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -63,62 +63,46 @@ __device__ __forceinline__ void dot4(const float *ar, const float *ai, const flo
     si = (m[0] + m[1]) + (m[2] + m[3]);
 }
 
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+// V as float pairs for dot2x4: per wave (vr, vi, -vr, -vi), (-vi, vr, vi, -vr)
+// of the high parts and (lr, li, -li, lr) of the low ones.
+__device__ __forceinline__ void load_v2(const double *V, int N, int np, float4 *vt)
 {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// a + p into the pair (s, c): s the rounded sum, c collecting the TwoSum error
-// and the product's rounding error pe.
-__device__ __forceinline__ void acc2(float &s, float &c, float p, float pe)
-{
-    float t, te;
-    two_sum(s, p, t, te);
-    s = t;
-    c += te + pe;
+    for (int w = threadIdx.x; w < np; w += blockDim.x) {
+        const double r = w < N ? V[2 * w] : 0.0, i = w < N ? V[2 * w + 1] : 0.0;
+        const float hr = (float)r, hi = (float)i;
+        const float lr = (float)(r - (double)hr), li = (float)(i - (double)hi);
+        vt[3 * w] = make_float4(hr, hi, -hr, -hi);
+        vt[3 * w + 1] = make_float4(-hi, hr, hi, -hr);
+        vt[3 * w + 2] = make_float4(lr, li, -li, lr);
+    }
 }
 
 // S = sum_a (Vh + Vl)_a A_a, compensated (Dot2 of Ogita, Rump and Oishi: each
 // product split exactly by FMA, TwoSum of the high parts) in four chains
-// (waves a = c mod 4) joined by TwoSum; the Vl terms in plain FMA. The result
-// is within about 2^-24 |S| + N^2 2^-48 sum_a |V_a A_a| of the exact sum.
+// (waves a = c mod 4) joined by TwoSum, Re S and Im S as a packed pair; the Vl
+// terms in plain FMA. The result is within about 2^-24 |S| + N^2 2^-48
+// sum_a |V_a A_a| of the exact sum.
 template <int NP>
-__device__ __forceinline__ void dot2x4(const float *ar, const float *ai, const float *vh,
-                                       const float *vl, float &sr, float &si)
+__device__ __forceinline__ void dot2x4(const float *ar, const float *ai, const float4 *vt, float &sr,
+                                       float &si)
 {
-    float s0[4] = {0.f, 0.f, 0.f, 0.f}, c0[4] = {0.f, 0.f, 0.f, 0.f};
-    float s1[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-    float l0 = 0.f, l1 = 0.f;
+    f2 s[4] = {0, 0, 0, 0}, c[4] = {0, 0, 0, 0}, l = 0;
 #pragma unroll
     for (int w = 0; w < NP; ++w) {
         const int j = w & 3;
-        const float x = ar[w], y = ai[w], vr = vh[2 * w], vi = vh[2 * w + 1];
-        float p;
-        p = x * vr; acc2(s0[j], c0[j], p, fmaf(x, vr, -p));     // Re S += x vr - y vi
-        p = -y * vi; acc2(s0[j], c0[j], p, fmaf(-y, vi, -p));
-        p = x * vi; acc2(s1[j], c1[j], p, fmaf(x, vi, -p));     // Im S += x vi + y vr
-        p = y * vr; acc2(s1[j], c1[j], p, fmaf(y, vr, -p));
-        l0 = fmaf(x, vl[2 * w], fmaf(-y, vl[2 * w + 1], l0));
-        l1 = fmaf(x, vl[2 * w + 1], fmaf(y, vl[2 * w], l1));
+        const f2 x = dup2(ar[w]), y = dup2(ai[w]);
+        const float4 a = vt[3 * w], b = vt[3 * w + 1], d = vt[3 * w + 2];
+        dot2_step(s[j], c[j], x, pk2(a.x, a.y), pk2(a.z, a.w));  // (x vr, x vi)
+        dot2_step(s[j], c[j], y, pk2(b.x, b.y), pk2(b.z, b.w));  // (-y vi, y vr)
+        l = fma2(x, pk2(d.x, d.y), fma2(y, pk2(d.z, d.w), l));
     }
 #pragma unroll
     for (int j = 1; j < 4; ++j) {
-        acc2(s0[0], c0[0], s0[j], c0[j]);
-        acc2(s1[0], c1[0], s1[j], c1[j]);
+        const ff t = ff_two_sum(s[0], s[j]);
+        s[0] = t.h;
+        c[0] = add2(c[0], add2(t.l, c[j]));
     }
-    sr = s0[0] + (c0[0] + l0);
-    si = s1[0] + (c1[0] + l1);
-}
-
-__device__ __forceinline__ void load_v2(const double *V, int N, int np2, float *vh, float *vl)
-{
-    for (int c = threadIdx.x; c < np2; c += blockDim.x) {
-        const double v = c < 2 * N ? V[c] : 0.0;
-        vh[c] = __double2float_rn(v);
-        vl[c] = __double2float_rn(v - (double)vh[c]);
-    }
+    upk2(add2(s[0], add2(c[0], l)), sr, si);
 }
 
 __device__ __forceinline__ void load_v(const double *V, int N, int np2, float *vf)
@@ -127,86 +111,142 @@ __device__ __forceinline__ void load_v(const double *V, int N, int np2, float *v
         vf[c] = c < 2 * N ? __double2float_rn(V[c]) : 0.f;
 }
 
-// Work split of the Hessian kernel for NP padded waves.
+// Work split of the Hessian kernel for np padded waves: PP = 2 np padded
+// parameters in B 4-column blocks, NB 4x4 blocks of the upper triangle, whose
+// sums run over EG groups of events (event e of a tile to group e mod EG, added
+// in order: the groups fix the order of the FP32 sums).
+constexpr int hess_blocks(int np) { return np / 2; }
+constexpr int hess_nb(int np) { return hess_blocks(np) * (hess_blocks(np) + 1) / 2; }
+// events handled by the busiest of kHT threads per tile with `it` items (block,
+// group) each, plus `it` for the per-item overhead
+constexpr int hess_cost(int np, int it)
+{
+    return (it * kHT / hess_nb(np)) < 1
+               ? (1 << 20)
+               : it * ((kHT + it * kHT / hess_nb(np) - 1) / (it * kHT / hess_nb(np))) + it;
+}
+constexpr int hess_groups(int np)
+{
+    const int c1 = hess_cost(np, 1), c2 = hess_cost(np, 2), c3 = hess_cost(np, 3);
+    const int it = (c1 <= c2 && c1 <= c3) ? 1 : (c2 <= c3) ? 2 : 3;
+    return it * kHT / hess_nb(np) > kHT ? kHT : it * kHT / hess_nb(np);
+}
+// 8x8 superblocks (two block rows and columns) of the upper triangle.
+constexpr int hess_super(int np) { return (np / 4) * (np / 4 + 1) / 2; }
+// Rows of a product thread's piece of a superblock (8 columns wide): the whole,
+// or a half where two threads for each superblock and group still fit.
+constexpr int hess_rows(int np)
+{
+    return 2 * hess_super(np) * hess_groups(np) <= kHT ? 4 : 8;
+}
+
 template <int NP>
 struct HessCfg {
-    static constexpr int PP = 2 * NP;            // padded parameters
-    static constexpr int B = PP / 4;             // 4-column blocks
-    static constexpr int NB = B * (B + 1) / 2;   // upper-triangle 4x4 blocks
-    // events handled by the busiest thread per tile with `it` items per thread,
-    // plus `it` for the per-item overhead
-    static constexpr int cost(int it)
+    static constexpr int B = hess_blocks(NP), NB = hess_nb(NP), EG = hess_groups(NP);
+    static constexpr int SB = B / 2, NS = hess_super(NP);
+    static constexpr int R = hess_rows(NP), PT = NS * (8 / R) * EG;
+    // float4s between the rows of a tile: odd, so that the stores of 8 threads (one
+    // row each) fall into different banks
+    static constexpr int LD = B + 1;
+    static constexpr size_t TILES = 2 * (size_t)kHT * LD * sizeof(float4);
+    static constexpr size_t SUMS = (size_t)EG * NS * 64 * sizeof(float2);
+    static constexpr size_t SMEM = TILES > SUMS ? TILES : SUMS;
+    // Warps 0 .. PW - 1 add products. A fifth and sixth one make their two of the
+    // SM's four schedulers carry twice the products of the others, which then get
+    // three of the warps that form J, and the first two one each (two warps idle).
+    static constexpr int PW = (PT + 31) / 32, WARPS = PW > 4 ? 16 : 12;
+    static_assert(PW <= 6, "more product warps than there are");
+    // the warp's place among those that form J, -1 for the others
+    static __device__ __forceinline__ int j_warp(int warp)
     {
-        return (it * kHT / NB) < 1 ? (1 << 20)
-                                   : it * ((kHT + it * kHT / NB - 1) / (it * kHT / NB)) + it;
+        if (PW <= 4)
+            return warp - 4 < 0 ? -1 : warp - 4;
+        return warp < 6 ? -1 : warp < 12 ? warp - 6 : warp < 14 ? -1 : warp - 8;
     }
-    static constexpr int IT = (cost(1) <= cost(2) && cost(1) <= cost(3)) ? 1
-                              : (cost(2) <= cost(3))                     ? 2
-                                                                         : 3;
-    static constexpr int EG0 = IT * kHT / NB;
-    static constexpr int EG = EG0 > kHT ? kHT : EG0;  // event groups
-    static constexpr int NI = NB * EG;                 // items
-    static constexpr size_t SMEM = (size_t)kHT * PP * sizeof(float);
-    static_assert(NI <= IT * kHT, "items exceed the threads' slots");
-    static_assert((size_t)NB * 16 * sizeof(double) <= SMEM, "reduction does not fit the tile");
 };
 
+// Place of block column x in a row of J: the even ones first, so that the
+// loads of neighbouring superblocks are neighbours in the banks.
+__device__ __forceinline__ constexpr int hess_place(int x, int sb) { return (x & 1) * sb + (x >> 1); }
+
+// The sums of many FP32 runs are float pairs (this part's FP64 pipe has 1/64 of
+// the FP32 rate: as doubles the conversions and sums of one block took 15 us),
+// scaled so that they overflow no earlier than the FP32 sums they are made of.
+constexpr float kSumScale = 0x1p-20f;
+
+__device__ __forceinline__ float half_of(f2 v, int odd)
+{
+    return __uint_as_float((unsigned)(odd ? v >> 32 : v));
+}
+
+// (h, l) += x, h + l kept to the rounding of l
+__device__ __forceinline__ void sum2(float &h, float &l, float x)
+{
+    const float t = h + x, z = t - h;
+    const float e = (h - (t - z)) + (x - z);
+    l += e;
+    h = t;
+}
+
+// Eight warps form J of the next tile (one event per thread, the tile after that
+// being loaded) while up to six add the products of the current one; two tile
+// buffers, one barrier per tile. Every kFlush tiles the FP32 sums go to FP64
+// sums in global scratch (they would take twice the registers of the products).
+//
+// Bound by instruction issue of the two parts together: at 32 waves the products
+// alone take 4.3 us a tile and SM (packed FMAs, two to an instruction; single
+// ones made the call a third slower), forming J alone 4.3 to 5.8, both 6.9. One
+// call at 333k events x 29 waves 172 to 96 us, at 1M x 32 405 to 248 us, at 500k
+// x 48 499 to 210 us, against one 256-thread role that did both in turn, with
+// 4x4 blocks (two 16-byte loads for 16 products, here four for 64).
 template <int NP>
-__global__ void __launch_bounds__(kHT, 1)
+__global__ void __launch_bounds__(HessCfg<NP>::WARPS * 32, 1)
     hess_kernel(const float *__restrict__ pl, int64_t pitch, int64_t n, int N, const double *V,
-                double *partials, int *status)
+                float2 *partials, float2 *scratch, int *status)
 {
     using C = HessCfg<NP>;
-    extern __shared__ __align__(16) float J[];   // [kHT][PP]
-    __shared__ float vh[2 * NP], vl[2 * NP];
+    extern __shared__ __align__(16) float J[];   // [2][kHT][LD float4s]
+    __shared__ float4 vt[3 * NP];
     __shared__ int s_bad;
-    float4 *J4 = reinterpret_cast<float4 *>(J);
-    load_v2(V, N, 2 * NP, vh, vl);
+    load_v2(V, N, NP, vt);
     if (threadIdx.x == 0)
         s_bad = 0;
-
-    int bx[C::IT], by[C::IT], grp[C::IT];
-    bool live[C::IT];
-#pragma unroll
-    for (int k = 0; k < C::IT; ++k) {
-        const int t = threadIdx.x + k * kHT;
-        live[k] = t < C::NI;
-        int blk = t % C::NB, x = 0;
-        grp[k] = t / C::NB;
-        while (blk >= C::B - x) {
-            blk -= C::B - x;
-            ++x;
-        }
-        bx[k] = x;
-        by[k] = x + blk;
-    }
-    float s[C::IT][16];
-    dfloat acc[C::IT][16];
-#pragma unroll
-    for (int k = 0; k < C::IT; ++k)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            s[k][q] = 0.f;
-            acc[k][q] = dfloat{0.f, 0.f};
-        }
     __syncthreads();
+    const int n_tiles = (int)((n + kHT - 1) / kHT);
+    const int n_my = (n_tiles > (int)blockIdx.x) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    auto tile_of = [&](int k) { return (int64_t)blockIdx.x + (int64_t)k * gridDim.x; };
+    const int j_warp = C::j_warp(threadIdx.x >> 5), je = j_warp * 32 + (threadIdx.x & 31);
+    // product threads: rows 8 bx + row0 .. + R - 1 and columns 8 by .. + 7 of the
+    // events of group grp
+    const int p = threadIdx.x;
+    const bool p_thread = p < C::PT;
+    int grp = 0, bx = 0, by = 0, sup = 0, half = 0;
+    if (p_thread) {
+        half = p % (8 / C::R);
+        sup = p / (8 / C::R) % C::NS;
+        grp = p / (8 / C::R * C::NS);
+        by = sup;
+        while (by >= C::SB - bx) {
+            by -= C::SB - bx;
+            ++bx;
+        }
+        by += bx;
+    }
 
-    const int64_t n_tiles = (n + kHT - 1) / kHT;
-    int bad = 0, run = 0;
-    // this thread's event of the next tile, loaded while the current tile's
-    // products run (events past n read event n - 1 and are dropped)
-    float xr[NP], xi[NP];
-    if (blockIdx.x < n_tiles)
-        load_event<NP>(pl, pitch, min(blockIdx.x * (int64_t)kHT + threadIdx.x, n - 1), N, xr, xi);
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int64_t i = tile * kHT + threadIdx.x;
-        const int64_t left = n - tile * kHT;
-        const int rows = left < kHT ? (int)left : kHT;
-        {
+    if (j_warp >= 0) {
+        int bad = 0;
+        float xr[NP], xi[NP];
+        // this thread's event of tile k (events past n read event n - 1 and are dropped)
+        auto load = [&](int k) {
+            load_event<NP>(pl, pitch, min(tile_of(k) * kHT + je, n - 1), N, xr, xi);
+        };
+        auto form = [&](int k) {
+            const int64_t i = tile_of(k) * kHT + je;
+            float4 *J4 = reinterpret_cast<float4 *>(J) + (size_t)(k & 1) * kHT * C::LD;
             float rr = 0.f, ri = 0.f;
             if (i < n) {
                 float sr, si;
-                dot2x4<NP>(xr, xi, vh, vl, sr, si);
+                dot2x4<NP>(xr, xi, vt, sr, si);
                 const float I = fmaf(sr, sr, si * si);
                 if (I > 0.f && I < INFINITY) {
                     rr = 2.f * sr / I;
@@ -227,103 +267,173 @@ __global__ void __launch_bounds__(kHT, 1)
                 im.y = fmaf(xr[4 * q + 1], ri, -xi[4 * q + 1] * rr);
                 im.z = fmaf(xr[4 * q + 2], ri, -xi[4 * q + 2] * rr);
                 im.w = fmaf(xr[4 * q + 3], ri, -xi[4 * q + 3] * rr);
-                J4[threadIdx.x * C::B + q] = re;
-                J4[threadIdx.x * C::B + NP / 4 + q] = im;
+                J4[je * C::LD + hess_place(q, C::SB)] = re;
+                J4[je * C::LD + hess_place(NP / 4 + q, C::SB)] = im;
             }
+        };
+        if (n_my > 0) {
+            load(0);
+            form(0);
         }
-        const int64_t next = tile + gridDim.x;
-        if (next < n_tiles)
-            load_event<NP>(pl, pitch, min(next * kHT + threadIdx.x, n - 1), N, xr, xi);
+        if (n_my > 1)
+            load(1);
         __syncthreads();
+        for (int k = 0; k < n_my; ++k) {
+            if (k + 1 < n_my)
+                form(k + 1);
+            if (k + 2 < n_my)
+                load(k + 2);
+            if (C::PW > 4 && k + 3 < n_my) {
+                // 128-byte lines of the tile after that: where three of these warps share a
+                // scheduler the loads are late otherwise (1M events: 32 waves 258 to 248 us,
+                // 48 waves at half of them 235 to 210; 24 and 40 waves, two on each, were
+                // slower by 10 us)
+                const int64_t e0 = tile_of(k + 3) * kHT;
+                for (int q = je; q < 2 * N * 8; q += kHT)
+                    if (e0 + (q & 7) * 32 < n)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(pl + (q >> 3) * pitch + e0 +
+                                                                     (q & 7) * 32));
+            }
+            __syncthreads();
+        }
+        if (bad)
+            s_bad = 1;
+    } else {
+        f2 s[C::R][4];
 #pragma unroll
-        for (int k = 0; k < C::IT; ++k) {
-            if (!live[k])
-                continue;
-            const float4 *ja = J4 + bx[k], *jb = J4 + by[k];
+        for (int r = 0; r < C::R; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                s[r][q] = 0;
+        // sums of the earlier runs of tiles: [R * 8][kHT] float pairs
+        float2 *acc = scratch + (size_t)blockIdx.x * (64 * kHT) + p;
+        int run = 0;
+        bool flushed = false;
+        __syncthreads();
+        for (int k = 0; k < n_my; ++k) {
+            const int64_t left = n - tile_of(k) * kHT;
+            const int rows = left < kHT ? (int)left : kHT;
+            if (p_thread) {
+                const float4 *J4 = reinterpret_cast<const float4 *>(J) + (size_t)(k & 1) * kHT * C::LD;
+                const float4 *ja = J4 + half * C::SB + bx, *jb = J4 + by;
 #pragma unroll 2
-            for (int e = grp[k]; e < rows; e += C::EG) {
-                const float4 a = ja[e * C::B], b = jb[e * C::B];
-                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+                for (int e = grp; e < rows; e += C::EG) {
+                    float a[C::R];
+                    f2 b[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
+                    for (int h = 0; h < C::R / 4; ++h) {
+                        const float4 v = ja[e * C::LD + h * C::SB];
+                        a[4 * h] = v.x, a[4 * h + 1] = v.y, a[4 * h + 2] = v.z, a[4 * h + 3] = v.w;
+                    }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        s[k][4 * r + c] = fmaf(av[r], bv[c], s[k][4 * r + c]);
-            }
-        }
-        if (++run == kFlush) {
-            run = 0;
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 v = jb[e * C::LD + h * C::SB];
+                        b[2 * h] = pk2(v.x, v.y), b[2 * h + 1] = pk2(v.z, v.w);
+                    }
 #pragma unroll
-            for (int k = 0; k < C::IT; ++k)
+                    for (int r = 0; r < C::R; ++r)
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    acc[k][q] = df_add(acc[k][q], dfloat{s[k][q], 0.f});
-                    s[k][q] = 0.f;
+                        for (int q = 0; q < 4; ++q)
+                            s[r][q] = fma2(dup2(a[r]), b[q], s[r][q]);
                 }
-        }
-        __syncthreads();
-    }
+                if (++run == kFlush && k + 1 < n_my) {
+                    run = 0;
 #pragma unroll
-    for (int k = 0; k < C::IT; ++k)
+                    for (int r = 0; r < C::R; ++r)
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-            acc[k][q] = df_add(acc[k][q], dfloat{s[k][q], 0.f});
-    if (bad)
-        s_bad = 1;
-
-    // event groups -> one 4x4 block each, in group order (the tile is free now)
-    double *red = reinterpret_cast<double *>(J);
-    for (int q = threadIdx.x; q < C::NB * 16; q += kHT)
-        red[q] = 0.0;
-    for (int g = 0; g < C::EG; ++g) {
-        __syncthreads();
+                        for (int q = 0; q < 8; ++q) {
+                            float2 *x = acc + (size_t)(8 * r + q) * kHT;
+                            float2 v = flushed ? *x : make_float2(0.f, 0.f);
+                            sum2(v.x, v.y, kSumScale * half_of(s[r][q >> 1], q & 1));
+                            *x = v;
+                        }
 #pragma unroll
-        for (int k = 0; k < C::IT; ++k) {
-            if (live[k] && grp[k] == g) {
-                const int blk = (threadIdx.x + k * kHT) % C::NB;
+                    for (int r = 0; r < C::R; ++r)
 #pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    red[blk * 16 + q] += (double)acc[k][q].hi + (double)acc[k][q].lo;
+                        for (int q = 0; q < 4; ++q)
+                            s[r][q] = 0;
+                    flushed = true;
+                }
             }
+            __syncthreads();
+        }
+        // the groups' sums: [EG][64][NS] float pairs (the tiles are free now)
+        if (p_thread) {
+            float2 *sums = reinterpret_cast<float2 *>(J) + (size_t)grp * 64 * C::NS + sup;
+#pragma unroll
+            for (int r = 0; r < C::R; ++r)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    float2 v = flushed ? acc[(size_t)(8 * r + q) * kHT] : make_float2(0.f, 0.f);
+                    sum2(v.x, v.y, kSumScale * half_of(s[r][q >> 1], q & 1));
+                    sums[(size_t)((half * C::R + r) * 8 + q) * C::NS] = v;
+                }
         }
     }
     __syncthreads();
     if (threadIdx.x == 0 && s_bad)
         atomicOr(status, FLAG_DOMAIN);
-    double *out = partials + (size_t)blockIdx.x * C::NB * 16;
-    for (int q = threadIdx.x; q < C::NB * 16; q += kHT)
-        out[q] = red[q];
+    const float2 *sums = reinterpret_cast<const float2 *>(J);
+    float2 *out = partials + (size_t)blockIdx.x * C::NS * 64;
+    for (int q = threadIdx.x; q < C::NS * 64; q += C::WARPS * 32) {
+        float h = 0.f, l = 0.f;
+        for (int g = 0; g < C::EG; ++g) {
+            const float2 v = sums[(size_t)g * 64 * C::NS + q];
+            sum2(h, l, v.x);
+            l += v.y;
+        }
+        out[q] = make_float2(h, l);
+    }
 }
 
-// H[r][c] over the real parameters (Re V at 0..N-1, Im V at N..2N-1): the sum
-// of the block partials, one warp per entry (lane k adds blocks k, k + 32, ...
-// in order, then a fixed shuffle tree), so the order is the same on every
-// run; zero when a data intensity was not positive. With async_or set, the
-// status bits of the call are also OR-ed into *async_or.
-__global__ void hess_finalize(const double *partials, int grid, int NP, int N, const int *status,
-                              double *H, int *async_or)
+// H[r][c] over the real parameters (Re V at 0..N-1, Im V at N..2N-1) from the
+// blocks' sums [grid][64][NS]: 32 entries per block, one per lane, its 8 warps
+// taking every eighth of the grid, then added in order, so that the order is the
+// same on every run; zero when a data intensity was not positive. With async_or
+// set, the status bits of the call are also OR-ed into *async_or.
+__global__ void __launch_bounds__(256)
+    hess_finalize(const float2 *partials, int grid, int NP, int N, const int *status, double *H,
+                  int *async_or)
 {
-    if (async_or && blockIdx.x == 0 && threadIdx.x == 0 && *status)
-        atomicOr(async_or, *status);
-    const int B = NP / 2, NB = B * (B + 1) / 2, P = 2 * N;
-    const int o = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (o >= P * P)
-        return;
-    const int r = o / P, c = o % P;
-    const int pr = r < N ? r : NP + (r - N), pc = c < N ? c : NP + (c - N);
-    int x = pr >> 2, y = pc >> 2, ii = pr & 3, jj = pc & 3;
-    if (x > y) {
-        const int t = x; x = y; y = t;
-        const int u = ii; ii = jj; jj = u;
+    __shared__ float2 part[8][32];
+    const int flags = *status;
+    if (async_or && blockIdx.x == 0 && threadIdx.x == 0 && flags)
+        atomicOr(async_or, flags);
+    const int SB = NP / 4, NS = SB * (SB + 1) / 2, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int o = blockIdx.x * 32 + lane;
+    float h = 0.f, l = 0.f;
+    if (o < NS * 64) {
+#pragma unroll 4
+        for (int b = warp; b < grid; b += 8) {
+            const float2 v = partials[(size_t)b * NS * 64 + o];
+            sum2(h, l, v.x);
+            l += v.y;
+        }
     }
-    const int blk = x * B - x * (x - 1) / 2 + (y - x);
-    const size_t stride = (size_t)NB * 16, at = (size_t)blk * 16 + ii * 4 + jj;
-    double v = 0.0;
-    for (int b = lane; b < grid; b += 32)
-        v += partials[b * stride + at];
-    v = warp_sum(v);
-    if (lane == 0)
-        H[o] = (*status & FLAG_DOMAIN) ? 0.0 : v;
+    part[warp][lane] = make_float2(h, l);
+    __syncthreads();
+    if (warp || o >= NS * 64)
+        return;
+    for (int w = 1; w < 8; ++w) {
+        sum2(h, l, part[w][lane].x);
+        l += part[w][lane].y;
+    }
+    int y = o % NS, x = 0;
+    const int q = o / NS;
+    while (y >= SB - x) {
+        y -= SB - x;
+        ++x;
+    }
+    const int pr = 8 * x + (q >> 3), pc = 8 * (x + y) + (q & 7);
+    const int r = pr < NP ? pr : pr - NP, c = pc < NP ? pc : pc - NP;
+    if (r >= N || c >= N || pr > pc)
+        return;
+    const int hr = pr < NP ? r : N + r, hc = pc < NP ? c : N + c, P = 2 * N;
+    const double v = (flags & FLAG_DOMAIN) ? 0.0
+                     : isfinite(h) ? ((double)h + (double)l) / (double)kSumScale
+                                   : (double)h;
+    H[hr * P + hc] = v;
+    H[hc * P + hr] = v;
 }
 
 // Blocks per SM the weights kernel is compiled for (the register cap that
@@ -386,11 +496,15 @@ cudaError_t hess_np(const Planes &d, const double *V, double *part, int grid, in
                                          (int)C::SMEM);
     if (e != cudaSuccess)
         return e;
-    hess_kernel<NP><<<grid, kHT, C::SMEM, s>>>(d.ptr, d.pitch, d.n, d.n_waves, V, part, status);
+    const int64_t n_tiles = (d.n + kHT - 1) / kHT;
+    if (grid > n_tiles)
+        grid = (int)n_tiles;
+    float2 *sums = reinterpret_cast<float2 *>(part);
+    hess_kernel<NP><<<grid, C::WARPS * 32, C::SMEM, s>>>(d.ptr, d.pitch, d.n, d.n_waves, V, sums,
+                                                   sums + (size_t)grid * C::NS * 64, status);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    const int P = 2 * d.n_waves;
-    hess_finalize<<<(P * P + 7) / 8, 256, 0, s>>>(part, grid, NP, d.n_waves, status, H, async_or);
+    hess_finalize<<<C::NS * 2, 256, 0, s>>>(sums, grid, NP, d.n_waves, status, H, async_or);
     return cudaGetLastError();
 }
 
@@ -414,8 +528,8 @@ int pad_np(int n)
 
 size_t hess_partials_doubles(int n_waves, int grid)
 {
-    const int B = pad_np(n_waves) / 2;
-    return (size_t)grid * (B * (B + 1) / 2) * 16;
+    const int np = pad_np(n_waves);
+    return (size_t)grid * 64 * (hess_super(np) + kHT);  // float pairs: the sums, the scratch
 }
 
 cudaError_t launch_hessian(const Planes &d, const double *V, double *partials, int grid, int *status,
