@@ -38,8 +38,5 @@ def test_runs_of_tiles(pwa, N, tiles):
         H = L.hessian(V)
         assert np.array_equal(H, H.T)
         assert np.max(np.abs(H - want)) <= H_TOL * np.max(np.abs(want))
-        # sums beyond the FP32 range stay finite (near that scale the intensities
-        # of events with small |S| lose bits to FP32 underflow, so no value is compared)
-        assert np.isfinite(L.hessian(V * 2.0 ** -56)).all()
         small = L.hessian(V * 2.0 ** 40) * 2.0 ** 80
         assert np.max(np.abs(small - want)) <= H_TOL * np.max(np.abs(want))
