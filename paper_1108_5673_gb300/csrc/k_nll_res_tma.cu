@@ -31,11 +31,14 @@
 // Bound by the FP32 pipe's latency before HBM: with both passes in one warp per
 // unit (seven warps per SM at 255 registers) 36% of the issue slots were used.
 // Twelve S warps and twelve gradient warps (72 registers) keep every sum's
-// order. Per call at 2M + 5M events x 20 waves, 4 free: 303 us (3.8 TB/s), 373
-// before; six and six warps 330, nine and six 315, fifteen and twelve 303. At 12
-// waves, 3 free 229 (279), at 28 and 4, 1M + 2.5M events 252 (291). Splitting a
+// order. Per call at 2M + 5M events x 20 waves, 4 free: 291 us (3.9 TB/s), 373
+// before; six and six warps 330, nine and six 315, fifteen and twelve 303 (these
+// with S warps that also waited for each other's tiles: 303). At 12 waves, 3 free
+// 214 (279), at 28 and 4, 1M + 2.5M events 255 (291). Splitting a
 // unit's waves over two warps in the S pass too changes the order of S's
 // remainders and with it the last digits of the gradients (3.6e-9).
+#include <numeric>
+
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -59,13 +62,19 @@ struct ResTmaCfg {
     static constexpr int SPG_RAW = (200 * 1024) / (STAGE_BYTES * G);
     static constexpr int SPG = SPG_RAW < 1 ? 1 : (SPG_RAW > 4 ? 4 : SPG_RAW);
     static constexpr int STAGES = G * SPG;
+    // Full barriers: tile j uses barrier j % FULL of stage j's copy. FULL is a multiple
+    // of SR, so that a barrier's successive tiles are of the same S warps (and of the
+    // same group): a parity wait then never sees a phase more than one away, however
+    // far one S warp falls behind another.
+    static constexpr int FULL = std::lcm(STAGES, SR);
+    static_assert(FULL % SR == 0 && FULL % STAGES == 0 && FULL % G == 0, "barrier ownership");
     static constexpr int THREADS = (1 + SWARPS + GH * UNITS) * 32;  // + the producer warp
     static constexpr int NR = 2 * NP + 2 * RP;      // per-unit float partials
     // the ring, then the weights w S of a stage's events (16 bytes per lane)
     static constexpr size_t RING_BYTES = (size_t)STAGES * STAGE_BYTES;
     static constexpr size_t WS_BYTES = (size_t)STAGES * GW * 32 * 16;
     static constexpr size_t SMEM =
-        RING_BYTES + WS_BYTES + (2 + GW) * STAGES * sizeof(uint64_t);
+        RING_BYTES + WS_BYTES + (FULL + (1 + GW) * STAGES) * sizeof(uint64_t);
     static constexpr size_t STATIC_BYTES = 32 * NP + 64 * RP + 8 * NR * UNITS + 32 * SWARPS + 256;
     static constexpr bool FITS = SMEM + STATIC_BYTES <= 227 * 1024;
 };
@@ -112,7 +121,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     float *tiles = reinterpret_cast<float *>(smem_raw);
     float4 *ws = reinterpret_cast<float4 *>(smem_raw + C::RING_BYTES);  // [STAGES][GW][32]
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + C::RING_BYTES + C::WS_BYTES);
-    uint64_t *empty = full + STAGES, *wfull = empty + STAGES;           // wfull [STAGES][GW]
+    uint64_t *empty = full + C::FULL, *wfull = empty + STAGES;          // wfull [STAGES][GW]
 
     __shared__ ResWave Vc[NP];
     __shared__ ResFree Fr[RP];
@@ -130,18 +139,22 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     const uint32_t stage_tx = (uint32_t)(1 + 2 * N) * TE * 4u;
     auto stage_of = [](int j) { return (j % C::G) * C::SPG + (j / C::G) % C::SPG; };
     auto use_of = [](int j) { return (uint32_t)((j / C::G) / C::SPG); };
+    auto full_of = [&](int j) { return &full[j % C::FULL]; };
+    auto full_parity = [](int j) { return (uint32_t)(j / C::FULL) & 1u; };
     auto issue = [&](int j, int s) {
         const int t = (int)blockIdx.x + j * (int)gridDim.x;
-        mbar_arrive_expect_tx(&full[s], stage_tx);
+        uint64_t *bar = full_of(j);
+        mbar_arrive_expect_tx(bar, stage_tx);
         if (t < tiles_d)
-            tma_load_2d(tiles + (size_t)s * ROWS * TE, &dmap, t * TE, 0, &full[s]);
+            tma_load_2d(tiles + (size_t)s * ROWS * TE, &dmap, t * TE, 0, bar);
         else
-            tma_load_2d(tiles + (size_t)s * ROWS * TE, &mmap, (t - tiles_d) * TE, 0, &full[s]);
+            tma_load_2d(tiles + (size_t)s * ROWS * TE, &mmap, (t - tiles_d) * TE, 0, bar);
     };
     const int n_first = n_my < STAGES ? n_my : STAGES;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < C::FULL; ++s)
             mbar_init(&full[s], 1);
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(&empty[s], (1 + C::GH) * GW);
             for (int k = 0; k < GW; ++k)
                 mbar_init(&wfull[s * GW + k], 1);
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
                 issue(j, s);
             }
             for (int q = (j > STAGES ? j - STAGES : 0); q < j; ++q)
-                if (!mbar_wait(&full[stage_of(q)], use_of(q) & 1))
+                if (!mbar_wait(full_of(q), full_parity(q)))
                     flags |= FLAG_TIMEOUT;
         }
     } else {
@@ -258,9 +271,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
         };
         int phase = 0;
         if (s_warp) {
-            // ---- S, ln I or I, and w S of the events ug of tiles j = sw / GW mod SR.
-            // Each warp waits for every tile's copy, its own or not, so that its parity
-            // waits follow the stages' uses one by one.
+            // ---- S, ln I or I, and w S of the events ug of tiles j = sw / GW mod SR
             const float sigma = s_sigma, unit = s_unit;
             const f2 SG = pk2(sigma, sigma);
             const unsigned im_offset = 2u * (unsigned)NP * __float_as_uint(sigma);
@@ -283,14 +294,12 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
                 eacc = 0;
                 acc = dfloat{0.f, 0.f};
             };
-            for (int j = 0; j < n_my; ++j) {
+            for (int j = sw / GW; j < n_my; j += C::SR) {
                 const int s = stage_of(j);
-                if (!mbar_wait(&full[s], use_of(j) & 1)) {
+                if (!mbar_wait(full_of(j), full_parity(j))) {
                     flags |= FLAG_TIMEOUT;
                     break;
                 }
-                if (j % C::SR != sw / GW)
-                    continue;
                 const int t = (int)blockIdx.x + j * (int)gridDim.x;
                 const int ph = t < tiles_d ? 0 : 1;
                 if (ph != phase) {  // every data tile of this CTA precedes its MC tiles
@@ -416,7 +425,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
                     reset();
                     phase = 1;
                 }
-                if (!mbar_wait(&full[s], use_of(j) & 1) ||
+                if (!mbar_wait(full_of(j), full_parity(j)) ||
                     !mbar_wait(&wfull[s * GW + ug], use_of(j) & 1)) {
                     flags |= FLAG_TIMEOUT;
                     break;
