@@ -1,8 +1,4 @@
-// Fused data-term kernel of the direct form (see k_nll_amp.cu for the
-// method): the kernel template, shared by the coherent launcher (k_nll_amp.cu,
-// one component per event) and the incoherent one (k_nll_incoh.cu, L
-// components per event: tiles of 2 L n rows, S^l of every component, I the
-// sum of their squared moduli, the gradient summed over components).
+// Fused data-term kernel of the direct form (see k_nll_amp.cu for the method).
 #pragma once
 
 #include "pwa_internal.cuh"
@@ -13,32 +9,29 @@ namespace {
 
 constexpr double kLn2 = 0.69314718055994530942;
 
-// N padded waves, G consumer groups, L components per event (1: the coherent
-// sum of Eq. 1; L > 1: an incoherent sum over L components, rows 2 (l n + a)
-// of a tile holding component l of wave a for n loaded waves).
-template <int N, int G, int L = 1>
+// N padded waves, G consumer groups.
+template <int N, int G>
 struct AmpCfg {
     static constexpr int GROUPS = G;                   // consumer groups (tiles in turn)
-    // warps per group: 4; 3 with several components or from 40 waves on, so
-    // that a CTA of two groups keeps to eight warps and the register cap of
-    // 255 (a larger CTA is allocated as twelve warps: 168 registers; the
-    // per-component state, or at 40 and 48 waves the per-wave state, does
-    // not fit). Measured on 1 GB samples: four-warp groups at 32 waves
+    // warps per group: 4; 3 from 40 waves on, so that a CTA of two groups
+    // keeps to eight warps and the register cap of 255 (a larger CTA is
+    // allocated as twelve warps: 168 registers; the per-wave state does not
+    // fit). Measured on 1 GB samples: four-warp groups at 32 waves
     // (with the re-read of the amplitudes below) 14% faster than three, and
     // at 40 and 48 waves three-warp groups 1.7 and 1.6 times faster than four.
-    static constexpr int GW = (L > 1 || N >= 40) ? 3 : 4;
+    static constexpr int GW = N >= 40 ? 3 : 4;
     static constexpr int CW = GROUPS * GW;             // consumer warps
     static constexpr int TE = GW * 32 * 2;             // events per tile (2 per thread)
-    static constexpr int ROWS = 2 * N * L;
+    static constexpr int ROWS = 2 * N;
     static constexpr uint32_t STAGE_BYTES = ROWS * TE * 4;
     // The ring. When two or more stages per group fit in 200 KB, each group
     // owns SPG of them (at most four): tile j goes to group j % G and to that
     // group's stage (j / G) % SPG, so a stage's successive uses belong to one
     // group and a waiter is never a whole phase behind. Otherwise (one stage
     // per group would fit), as many stages as fit are shared by the groups:
-    // tile j sits in stage j % STAGES (a third stage at 32 waves, or for two
-    // components of 20 waves, measured 8% and 21% faster than two; a fifth
-    // shared 40 KB stage at 20 waves was slower than four owned ones). A
+    // tile j sits in stage j % STAGES (a third stage at 32 waves measured 8%
+    // faster than two; a fifth shared 40 KB stage at 20 waves was slower than
+    // four owned ones). A
     // shared stage has two full barriers, for its even and its odd uses.
     // A group waiting for use u of a stage (tile j) waits on the barrier
     // whose previous phase was use u - 2 (tile j - 2 STAGES); with 2 STAGES a
@@ -226,14 +219,13 @@ __device__ __forceinline__ void exact_scale(const double *V, const float *amax, 
 }
 
 // WEIGHTS: instead of the NLL, write I / N_gen of every event to a.weights
-// (the projection weights of the accepted MC events; L = 1), with no sums.
-template <int N, int G, int L = 1, bool WEIGHTS = false>
-__global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
+// (the projection weights of the accepted MC events), with no sums.
+template <int N, int G, bool WEIGHTS = false>
+__global__ void __launch_bounds__(AmpCfg<N, G>::THREADS, 1)
     nll_amp_kernel(const __grid_constant__ CUtensorMap map, const EvalArgs a, const int n_tiles,
                    int *work_flags)
 {
-    static_assert(!WEIGHTS || L == 1, "projection weights of a coherent sample");
-    using C = AmpCfg<N, G, L>;
+    using C = AmpCfg<N, G>;
     constexpr int TE = C::TE, ROWS = C::ROWS, STAGES = C::STAGES, CW = C::CW;
     constexpr int GROUPS = C::GROUPS, GW = C::GW;
     constexpr int NF = C::NF;
@@ -258,7 +250,7 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
     // to group j % GROUPS and to stage stage_of(j) (see AmpCfg)
     const int n_my =
         (n_tiles > (int)blockIdx.x) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const uint32_t stage_tx = 2u * (uint32_t)a.n_waves * L * TE * 4u;
+    const uint32_t stage_tx = 2u * (uint32_t)a.n_waves * TE * 4u;
     auto stage_of = [](int j) {
         return C::SHARED ? j % STAGES : (j % GROUPS) * C::SPG + (j / GROUPS) % C::SPG;
     };
@@ -291,7 +283,7 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
     // Rows of padded waves (n_waves < N) are never written by TMA: zero them
     // once so that they contribute nothing (their V is zero as well).
     for (int s = 0; s < STAGES; ++s)
-        for (int i = 2 * a.n_waves * L * TE + threadIdx.x; i < ROWS * TE; i += blockDim.x)
+        for (int i = 2 * a.n_waves * TE + threadIdx.x; i < ROWS * TE; i += blockDim.x)
             tiles[(size_t)s * ROWS * TE + i] = 0.f;
     // V may sit in host memory: these reads and those of the helper warp are
     // its only ones (one round trip each, concurrent with the first tiles)
@@ -351,55 +343,17 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
             const float *T = tiles + (size_t)s * ROWS * TE + 2 * ct;
             const int64_t ev0 = (int64_t)((int)blockIdx.x + j * (int)gridDim.x) * TE + 2 * ct;
 
-            // component l of wave w sits at rows 2 (l n + w), 2 (l n + w) + 1
             // (padded waves w >= n carry V = 0: their products are exactly 0)
-            const int comp_rows = 2 * a.n_waves * TE;
-            // S of the two events of this thread for the component at Tl
-            auto component_sum = [&](const float *Tl, float (&sr)[2], float (&si)[2]) {
-                exact_sum2<N>(
-                    [&](int w, f2 &ar, f2 &ai) {
-                        ar = lds2(Tl + (2 * w) * TE);
-                        ai = lds2(Tl + (2 * w + 1) * TE);
-                    },
-                    Vc, SG, unit, im_offset, sr, si);
-            };
-            // gs += conj(A) r for the component at Tl, r = S / I of the two events
-            auto component_grad = [&](const float *Tl, float r0, float r1, float i0, float i1) {
-#pragma unroll
-                for (int w = 0; w < N; ++w) {
-                    float a0, a1, b0, b1;
-                    upk2(lds2(Tl + (2 * w) * TE), a0, a1);
-                    upk2(lds2(Tl + (2 * w + 1) * TE), b0, b1);
-                    // conj(A) r = (ar rr + ai ri) + i (ar ri - ai rr)
-                    gs[2 * w] = fmaf(a0, r0, fmaf(b0, i0, gs[2 * w]));
-                    gs[2 * w] = fmaf(a1, r1, fmaf(b1, i1, gs[2 * w]));
-                    gs[2 * w + 1] = fmaf(a0, i0, fmaf(-b0, r0, gs[2 * w + 1]));
-                    gs[2 * w + 1] = fmaf(a1, i1, fmaf(-b1, r1, gs[2 * w + 1]));
-                }
-            };
-            float Sr[L][2], Si[L][2], rr[L][2], ri[L][2];
-            if constexpr (L == 1) {
-                component_sum(T, Sr[0], Si[0]);
-            } else {
-                // not unrolled: unrolled, the compiler holds every wave's V
-                // coefficients across the components and spills
-#pragma unroll 1
-                for (int l = 0; l < L; ++l) {
-                    float sr[2], si[2];
-                    component_sum(T + l * comp_rows, sr, si);
-#pragma unroll
-                    for (int k = 0; k < L; ++k)
-                        if (k == l) {
-                            Sr[k][0] = sr[0];
-                            Sr[k][1] = sr[1];
-                            Si[k][0] = si[0];
-                            Si[k][1] = si[1];
-                        }
-                }
-            }
+            float Sr[2], Si[2], rr[2], ri[2];
+            exact_sum2<N>(
+                [&](int w, f2 &ar, f2 &ai) {
+                    ar = lds2(T + (2 * w) * TE);
+                    ai = lds2(T + (2 * w + 1) * TE);
+                },
+                Vc, SG, unit, im_offset, Sr, Si);
             if constexpr (WEIGHTS) {
-                const float w0 = fmaf(Sr[0][0], Sr[0][0], Si[0][0] * Si[0][0]) * a.inv_ngen;
-                const float w1 = fmaf(Sr[0][1], Sr[0][1], Si[0][1] * Si[0][1]) * a.inv_ngen;
+                const float w0 = fmaf(Sr[0], Sr[0], Si[0] * Si[0]) * a.inv_ngen;
+                const float w1 = fmaf(Sr[1], Sr[1], Si[1] * Si[1]) * a.inv_ngen;
                 if (ev0 + 1 < a.n_events)
                     *reinterpret_cast<float2 *>(a.weights + ev0) = make_float2(w0, w1);
                 else if (ev0 < a.n_events)
@@ -411,17 +365,11 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                float I = fmaf(Sr[0][e], Sr[0][e], Si[0][e] * Si[0][e]);
-#pragma unroll
-                for (int l = 1; l < L; ++l)
-                    I = I + fmaf(Sr[l][e], Sr[l][e], Si[l][e] * Si[l][e]);
+                const float I = fmaf(Sr[e], Sr[e], Si[e] * Si[e]);
                 const bool in = (ev0 + e) < a.n_events;
                 const bool ok = (I > 0.f) && (I < INFINITY);
-#pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    rr[l][e] = 0.f;
-                    ri[l][e] = 0.f;
-                }
+                rr[e] = 0.f;
+                ri[e] = 0.f;
                 if (in) {
                     if (ok) {
                         int ex;
@@ -433,39 +381,31 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
                         l_frac += y - (t - 12582912.0f);
                         eacc += ex;
                         const float rI = __frcp_rn(I);
-#pragma unroll
-                        for (int l = 0; l < L; ++l) {
-                            rr[l][e] = Sr[l][e] * rI;
-                            ri[l][e] = Si[l][e] * rI;
-                        }
+                        rr[e] = Sr[e] * rI;
+                        ri[e] = Si[e] * rI;
                     } else {
                         bad = 1;
                     }
                 }
             }
-            if constexpr (L == 1) {
-                // from 32 waves on, the amplitudes are read again from shared
-                // memory rather than held from the pass for S (4N registers,
-                // which spilled: 0.5 KB per thread at 32 waves with four-warp
-                // groups, 1.4 KB at 48); below, holding them is faster (24
-                // waves: 3% slower with the re-read)
-                if constexpr (N >= 32)
-                    asm volatile("" ::: "memory");
-                component_grad(T, rr[0][0], rr[0][1], ri[0][0], ri[0][1]);
-            } else {
-#pragma unroll 1
-                for (int l = 0; l < L; ++l) {
-                    float r0 = rr[0][0], r1 = rr[0][1], i0 = ri[0][0], i1 = ri[0][1];
+            // from 32 waves on, the amplitudes are read again from shared
+            // memory rather than held from the pass for S (4N registers,
+            // which spilled: 0.5 KB per thread at 32 waves with four-warp
+            // groups, 1.4 KB at 48); below, holding them is faster (24
+            // waves: 3% slower with the re-read)
+            if constexpr (N >= 32)
+                asm volatile("" ::: "memory");
+            // gs += conj(A) r, r = S / I of the two events
 #pragma unroll
-                    for (int k = 1; k < L; ++k)
-                        if (k == l) {
-                            r0 = rr[k][0];
-                            r1 = rr[k][1];
-                            i0 = ri[k][0];
-                            i1 = ri[k][1];
-                        }
-                    component_grad(T + l * comp_rows, r0, r1, i0, i1);
-                }
+            for (int w = 0; w < N; ++w) {
+                float a0, a1, b0, b1;
+                upk2(lds2(T + (2 * w) * TE), a0, a1);
+                upk2(lds2(T + (2 * w + 1) * TE), b0, b1);
+                // conj(A) r = (ar rr + ai ri) + i (ar ri - ai rr)
+                gs[2 * w] = fmaf(a0, rr[0], fmaf(b0, ri[0], gs[2 * w]));
+                gs[2 * w] = fmaf(a1, rr[1], fmaf(b1, ri[1], gs[2 * w]));
+                gs[2 * w + 1] = fmaf(a0, ri[0], fmaf(-b0, rr[0], gs[2 * w + 1]));
+                gs[2 * w + 1] = fmaf(a1, ri[1], fmaf(-b1, rr[1], gs[2 * w + 1]));
             }
             __syncwarp();
             if (lane == 0)
@@ -537,135 +477,16 @@ __global__ void __launch_bounds__(AmpCfg<N, G, L>::THREADS, 1)
             v = df_add(v, dfloat{red_f[w][c], 0.f});
         sc.pf[(size_t)c * gridDim.x + blockIdx.x] = make_float2(v.hi, v.lo);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (s_flags)
-            atomicOr(work_flags, s_flags);
-        __threadfence();
-        const unsigned t = atomicAdd(a.ticket, 1u);
-        s_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_last)
-        return;
-
-    // ---- last CTA: deterministic final sum + normalisation term ---------
-    // One warp per component (2N+1 float-float ones, then the 2 integer
-    // ones): lane l adds CTAs l, l + 32, ... (coalesced loads, all issued
-    // before the adds, with M V and the launch's flags: one L2 round trip),
-    // then a fixed shuffle tree. (The partials are read with L2 loads after
-    // the ticket, so no further fence is needed.)
-    const int Nw = a.n_waves;
-    const int G_ = gridDim.x;
-    constexpr int NWARPS = C::THREADS / 32;
-    constexpr int CPW = (NF + 2 + NWARPS - 1) / NWARPS;  // components per warp
-    constexpr int QB = 5;                                 // loads per lane and component in flight
-    dfloat *tot_f = reinterpret_cast<dfloat *>(tiles);                  // [NF]
-    long long *tot_i = reinterpret_cast<long long *>(tot_f + NF);       // [2]
-    double *smv = reinterpret_cast<double *>(tot_i + 2);                // [2N] M V, V^H M V
-    const double mv_i = threadIdx.x < 2 * Nw ? __ldcg(&sc.mv[threadIdx.x])
-                                             : threadIdx.x == 2 * Nw ? __ldcg(&sc.mv[2 * kMaxWaves])
-                                                                      : 0.0;
-    const int wf = __ldcg(work_flags);
-    {
-        // a partial is 8 bytes either way: a float pair (hi in the low word)
-        // or an integer
-        const unsigned long long *pf64 = reinterpret_cast<const unsigned long long *>(sc.pf);
-        const unsigned long long *pi64 = reinterpret_cast<const unsigned long long *>(sc.pi);
-        dfloat acc[CPW];
-        long long iacc[CPW];
-#pragma unroll
-        for (int k = 0; k < CPW; ++k) {
-            acc[k] = dfloat{0.f, 0.f};
-            iacc[k] = 0;
-        }
-        for (int b0 = 0; b0 < G_; b0 += 32 * QB) {
-            unsigned long long r[CPW][QB];
-#pragma unroll
-            for (int k = 0; k < CPW; ++k) {
-                const int comp = warp + k * NWARPS;
-                const unsigned long long *src =
-                    comp < NF ? pf64 + (size_t)comp * G_ : pi64 + (size_t)(comp - NF) * G_;
-#pragma unroll
-                for (int q = 0; q < QB; ++q) {
-                    const int b = b0 + lane + 32 * q;
-                    r[k][q] = (b < G_ && comp < NF + 2) ? __ldcg(src + b) : 0ull;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < CPW; ++k) {
-                if (warp + k * NWARPS < NF) {
-#pragma unroll
-                    for (int q = 0; q < QB; ++q)
-                        acc[k] = df_add(acc[k], dfloat{__uint_as_float((unsigned)r[k][q]),
-                                                       __uint_as_float((unsigned)(r[k][q] >> 32))});
-                } else {
-#pragma unroll
-                    for (int q = 0; q < QB; ++q)
-                        iacc[k] += (long long)r[k][q];
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < CPW; ++k) {
-            const int comp = warp + k * NWARPS;
-            if (comp < NF) {
-                const dfloat v = warp_sum(acc[k]);
-                if (lane == 0)
-                    tot_f[comp] = v;
-            } else if (comp < NF + 2) {
-                const long long v = warp_sum(iacc[k]);
-                if (lane == 0)
-                    tot_i[comp - NF] = v;
-            }
-        }
-    }
-    if (threadIdx.x <= 2 * Nw)
-        smv[threadIdx.x] = mv_i;
-    __syncthreads();
-    const bool invalid = (wf & (FLAG_DOMAIN | FLAG_TIMEOUT)) != 0;
-    for (int c = threadIdx.x; c < 2 * Nw + 1; c += blockDim.x) {  // padded waves excluded
-        const dfloat v = tot_f[c];
-        if (c > 0) {
-            // gradient: - sum_i conj(A) S / I + (M V)
-            if (a.grad)
-                a.grad[c - 1] = invalid ? 0.0 : (smv[c - 1] - (double)v.hi) - (double)v.lo;
-        } else {
-            // ln sum: integer part and exponents are exact; the rest is small
-            const long long li = tot_i[0], ei = tot_i[1];
-            const double lnsum =
-                fma((double)ei, kLn2, ((double)li + ((double)v.hi + (double)v.lo)) * 0x1p-23);
-            double nll = smv[2 * Nw] - lnsum;
-            if (wf & FLAG_DOMAIN)
-                nll = INFINITY;
-            if (wf & FLAG_TIMEOUT)
-                nll = NAN;
-            a.nll[0] = nll;
-            if (wf)
-                atomicOr(a.status, wf);
-            if (a.done)
-                atomicAdd(a.done, 1);
-        }
-    }
-    if (a.host_flag)
-        __threadfence_system();  // this thread's results reach the host before the flag
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        *work_flags = 0;
-        *a.ticket = 0u;
-        if (a.host_flag)
-            *reinterpret_cast<volatile unsigned long long *>(a.host_flag) =
-                ((unsigned long long)a.seq << 32) | (unsigned)wf;
-    }
+#include "direct_finish.cuh"
 }
 
 // The last CTA keeps its sub-sums in its (then idle) stage buffers.
-template <int N, int G, int L = 1>
+template <int N, int G>
 constexpr bool finalize_fits(int grid)
 {
     (void)grid;
-    return (size_t)(2 * N + 3) * 8 + 8 * (2 * N + 1) <= AmpCfg<N, G, L>::SMEM &&
-           AmpCfg<N, G, L>::THREADS > 2 * N;
+    return (size_t)(2 * N + 3) * 8 + 8 * (2 * N + 1) <= AmpCfg<N, G>::SMEM &&
+           AmpCfg<N, G>::THREADS > 2 * N;
 }
 
 }  // namespace

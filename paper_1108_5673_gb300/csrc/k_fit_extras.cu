@@ -586,12 +586,12 @@ template <int N>
 cudaError_t weights_tma_n(const CUtensorMap *map, const EvalArgs &a, int grid, cudaStream_t s)
 {
     using C = AmpCfg<N, 2>;
-    cudaError_t e = cudaFuncSetAttribute(nll_amp_kernel<N, 2, 1, true>,
+    cudaError_t e = cudaFuncSetAttribute(nll_amp_kernel<N, 2, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess)
         return e;
     const int n_tiles = (int)((a.n_events + C::TE - 1) / C::TE);
-    nll_amp_kernel<N, 2, 1, true><<<grid, C::THREADS, C::SMEM, s>>>(*map, a, n_tiles, nullptr);
+    nll_amp_kernel<N, 2, true><<<grid, C::THREADS, C::SMEM, s>>>(*map, a, n_tiles, nullptr);
     return cudaGetLastError();
 }
 }  // namespace

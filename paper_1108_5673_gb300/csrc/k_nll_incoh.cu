@@ -20,7 +20,7 @@
 // FP64 across warps and blocks. The last block (atomic ticket) adds the
 // block partials in block order and the normalisation term in FP64, so the
 // results are bitwise reproducible.
-#include "amp_kernel.cuh"
+#include "split_kernel.cuh"
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -304,30 +304,24 @@ int pad_np(int n)
     return 1 << 20;
 }
 
-// ---- TMA-fed path: the direct-form kernel with L components per event ------
-// (amp_kernel.cuh): tiles of 192 events x 2 L n rows streamed by TMA, the
-// products split exactly against sigma (bounded over all components) and
-// their high parts summed as integers, two events per thread in FP32x2, two
-// groups of three consumer warps. It serves N_pad * L <= 48 (stages of
-// 2 L N_pad x 192 floats in the 200 KB ring, owned by a group where two or
-// more per group fit, shared by both groups otherwise).
+// ---- TMA-fed path (split_kernel.cuh): units of 64 events x 2 L n rows streamed
+// by TMA, the products split exactly against sigma (bounded over all
+// components) and their high parts summed as integers, two events per lane in
+// FP32x2, S and the gradient in warps of their own. It serves N_pad * L <= 48.
 template <int N, int L>
 cudaError_t launch_tma_nl(const CUtensorMap *map, const EvalArgs &a, int grid, cudaStream_t s)
 {
     if constexpr (N * L > kMaxLanes || L < 2) {
         return cudaErrorInvalidValue;
     } else {
-        using C = AmpCfg<N, 2, L>;
-        static_assert(C::FITS, "one stage per consumer group must fit");
-        if (!finalize_fits<N, 2, L>(grid))
-            return cudaErrorInvalidConfiguration;
-        cudaError_t e = cudaFuncSetAttribute(nll_amp_kernel<N, 2, L>,
+        using C = SplitCfg<N, L>;
+        cudaError_t e = cudaFuncSetAttribute(nll_split_kernel<N, L>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess)
             return e;
-        const int n_tiles = (int)((a.n_events + C::TE - 1) / C::TE);
+        const int n_tiles = (int)((a.n_events + C::GW * C::UE - 1) / (C::GW * C::UE));
         int *work_flags = amp_scratch(a.partials, grid).flags;
-        nll_amp_kernel<N, 2, L><<<grid, C::THREADS, C::SMEM, s>>>(*map, a, n_tiles, work_flags);
+        nll_split_kernel<N, L><<<grid, C::THREADS, C::SMEM, s>>>(*map, a, n_tiles, work_flags);
         return cudaGetLastError();
     }
 }
@@ -351,7 +345,7 @@ bool incoh_tma_available(int n_waves, int n_lambda)
     return n_lambda >= 2 && n_lambda <= kMaxLambda && pad_np(n_waves) * n_lambda <= kMaxLanes;
 }
 
-int incoh_tma_box_events() { return AmpCfg<4, 2, 2>::TE; }
+int incoh_tma_box_events() { return SplitCfg<4, 2>::UE; }
 
 cudaError_t launch_nll_incoh_tma(const CUtensorMap *map, int n_lambda, const EvalArgs &a, int grid,
                                  cudaStream_t s)

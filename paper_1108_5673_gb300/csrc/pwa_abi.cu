@@ -552,15 +552,16 @@ cudaGraphExec_t eval_graph(pwa_ctx *c, int K, bool with_grad)
 // The direct form's host call without copies: the kernels read V from the
 // pinned buffer and write nll, grad and a flag (sequence number, status
 // bits) straight back into it, and the host spins on the flags instead of
-// synchronising the stream. Used for coherent samples in the direct form
-// unless PWA_ZERO_COPY=0.
+// synchronising the stream (whose return comes in steps of some 12 us here).
+// Used in the direct form, coherent or TMA-fed incoherent, unless
+// PWA_ZERO_COPY=0.
 bool zero_copy_ok(const pwa_ctx *c)
 {
     static const bool off = [] {
         const char *v = getenv("PWA_ZERO_COPY");
         return v && strcmp(v, "0") == 0;
     }();
-    return !off && c->h_io_dev && c->form == PWA_FORM_AMP && c->n_lambda == 1;
+    return !off && c->h_io_dev && c->form == PWA_FORM_AMP && (c->n_lambda == 1 || c->incoh_tma);
 }
 
 int eval_host_zc(pwa_ctx *c, const double *V, int K, double *nll, double *grad)
@@ -590,7 +591,10 @@ int eval_host_zc(pwa_ctx *c, const double *V, int K, double *nll, double *grad)
         a.host_flag = reinterpret_cast<unsigned long long *>(dev(flags + k));
         a.seq = seq;
         a.stall_ns = test_stall_ns();
-        const cudaError_t e = launch_nll_amp(c->data, &c->data_map, a, c->num_sms, c->stream,
+        const cudaError_t e =
+            c->n_lambda > 1 ? launch_nll_incoh_tma(&c->data_map, c->n_lambda, a,
+                                                   amp_grid(N, c->num_sms), c->stream)
+                            : launch_nll_amp(c->data, &c->data_map, a, c->num_sms, c->stream,
                                              c->tune_groups);
         if (e != cudaSuccess) {
             cudaGetLastError();
