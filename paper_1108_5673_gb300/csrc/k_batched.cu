@@ -41,10 +41,10 @@
 // R' = Q / |Q|^2, rounded to BF16, by both slices (N = XS F columns).
 //
 // Layout in shared memory (128-byte swizzled, 1 KB aligned):
-//  W   [chunk][half][F/64 blocks][slice w0,w1,w2][64 rows][128 B]: K-major B
-//      operands of GEMM 1 (the three slices of a block are adjacent, so one
-//      product covers w0|w1|w2 as 192 columns), copied once per launch from an
-//      image the prep kernel builds.
+//  W   [step][F/64 blocks][slice w0,w1,w2][64 or 32 rows][128 B]: K-major B
+//      operands of GEMM 1 for a step's 32 or 16 sets (the three slices of a block
+//      are adjacent, so one product covers w0|w1|w2 as 192 or 96 columns), copied
+//      once per launch from an image the prep kernel builds.
 //  X   [stage][2 blocks of 64 events][XS F rows (x0 then x1)][128 B]: MN-major
 //      A operand of GEMM 1 (events contiguous) and K-major B operand of GEMM 2
 //      (K = events) -- the same bytes serve both products. The data store in
@@ -53,13 +53,24 @@
 //      events x XS F rows reads XS F separate 128-byte pieces, far apart).
 //  R'  [2 blocks of 64 rows (k,re/im)][128 events][128 B]: MN-major A operand
 //      of GEMM 2, written by the epilogue (each thread stores its event's row).
-// Tensor memory (512 columns): acc0..acc3 of one half chunk (32 sets, 64
-// columns each), then the G^T accumulators of every chunk (XS F columns each)
-// for the whole launch.
+// Tensor memory (512 columns): acc0..acc3 of one step of 32 sets (64 columns
+// each) or of two of 16 (32 each), then the G^T accumulators of every chunk (XS F
+// columns each) for the whole launch.
 //
-// Warps: 0-15 epilogue (warp w reads TMEM lane quarter w%4 and the 8 sets
-// w/4 of each half chunk), 16 producer (TMA), 17 MMA issuer (one thread),
-// 18 helper (M V and V^H M V in FP64). Every wait is bounded.
+// Warps: 0-15 epilogue (warp w reads TMEM lane quarter w%4 and 8 sets of a step),
+// 16 producer (TMA), 17 MMA issuer, 18 helper (M V and V^H M V in FP64). Every
+// wait is bounded.
+//
+// Bound by the epilogue's instructions and the chain of a step (GEMM 1 958 cycles,
+// its completion ~250, the read of the accumulators ~430, the way back to the
+// issuer; GEMM 2 257 a step, which fills the gaps): 32 waves in 16-bit slices take
+// 2250 cycles a step of 32 sets x 128 events where the products alone take 1215.
+// The issuer was on that chain: as one lane of a divergent branch it took its
+// descriptors through vector registers and divided for its indices; as a warp that
+// the compiler knows to be converged, counting instead, it brought 1M events x 32
+// waves x 256 sets from 614 to 521 us a call and 16 models x 16 sets from 1101 to
+// 936 (890 in steps of 16). Polling instead of suspended waits in the epilogue,
+// GEMM 1 before GEMM 2 when both can go, no fence: no difference or slower.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -75,13 +86,18 @@ namespace {
 
 constexpr int kBM = 128;        // events per tile
 constexpr int kKC = 64;         // parameter sets per chunk (GEMM 2: M = 2 kKC = 128)
-constexpr int kHS = 32;         // parameter sets per half chunk (one GEMM 1 / epilogue step)
+constexpr int kHS = 32;         // parameter sets per half chunk (one block of R', one flag word)
+// Parameter sets per GEMM 1 / epilogue step: 32 (a half chunk), whose epilogue takes
+// all 16 warps; 16 for up to 16 sets, where two groups of eight warps take the tiles
+// in turn, each with accumulators of its own. 16 models of up to 1M events x 16
+// sets: 895 us a call with steps of 16, 936 with steps of 32 (half of whose products
+// and warps are padding then); 1M events x 32 waves x 256 sets 568 and 521 us.
+__host__ __device__ constexpr int step_sets(int K) { return K <= 16 ? 16 : 32; }
 constexpr int kXSMax = 6;       // X stages at most (as many as shared memory takes, at least 2)
 constexpr int kMaxSmem = 226 * 1024;
 constexpr int kMaxChunks = 4;
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 3) * 32;
-constexpr uint32_t kWBlock = 64 * 128;      // 64 rows x 64 BF16 features
 constexpr uint32_t kRBytes = 2 * 128 * 128;
 constexpr int kWSlices = 3;                 // BF16 slices of V
 // tensor-memory columns: accumulators acc0..acc3 at 64 j, then G^T
@@ -141,22 +157,22 @@ struct Smem {
     int nxs;   // X stages
 };
 
-// Bytes of the W image of n_chunks chunks (both halves of each), as built in
+// Bytes of the W image of n_chunks chunks (all steps of each), as built in
 // global memory by the prep kernel.
 __host__ __device__ inline uint32_t w_image_bytes(int F, int n_chunks)
 {
-    return (uint32_t)n_chunks * 2 * kWSlices * ((F + 63) / 64) * kWBlock;
+    return (uint32_t)n_chunks * kKC * kWSlices * ((F + 63) / 64) * 2 * 128;
 }
 
-// Shared memory of a launch for K sets: the W image of the hpt half chunks
+// Shared memory of a launch for K sets: the W image of the steps
 // that hold sets (its first part), then as many X stages as fit (2..kXSMax),
 // then R'. Small K leave room for a deeper X pipeline, which their short
 // per-tile work needs to hide the loads.
-__host__ __device__ inline Smem batch_smem(int F, int xs, int hpt, int nxs_req = 0)
+__host__ __device__ inline Smem batch_smem(int F, int xs, int K, int nxs_req = 0)
 {
     const int kb = (F + 63) / 64;
     Smem s;
-    s.w_bytes = (uint32_t)hpt * kWSlices * kb * kWBlock;
+    s.w_bytes = (uint32_t)((K + step_sets(K) - 1) / step_sets(K) * step_sets(K)) * kWSlices * kb * 2 * 128;
     const uint32_t stage = 2u * xs * F * 128;
     const int64_t room = (int64_t)kMaxSmem - 1024 - kRBytes - (int64_t)s.w_bytes;
     const int fit = room > 0 ? (int)(room / stage) : 0;
@@ -169,8 +185,6 @@ __host__ __device__ inline Smem batch_smem(int F, int xs, int hpt, int nxs_req =
     s.bytes = s.r_off + kRBytes + 1024;  // + alignment slack
     return s;
 }
-
-__host__ __device__ inline int batch_hpt(int K) { return (K + kHS - 1) / kHS; }
 
 __host__ __device__ inline uint32_t sw128(int row, int byte_in_row)
 {
@@ -271,7 +285,9 @@ __device__ __forceinline__ void batched_prep_block(const BatchArgs &a, const int
         if (lane == 0)
             a.T[k] = T;
     }
-    unsigned char *out = a.wimg + (size_t)half * KB * kWSlices * kWBlock;
+    const int qs = step_sets(a.K), rl = 2 * (sl % qs);  // the set's rows in its step
+    const size_t wblock = 2 * qs * 128;
+    unsigned char *out = a.wimg + (half * (kHS / qs) + sl / qs) * KB * kWSlices * wblock;
     for (int w = lane; w < KB * 32; w += 32) {
         double wr[kWSlices] = {0.0, 0.0, 0.0}, wi[kWSlices] = {0.0, 0.0, 0.0};
         if (k < a.K && w < Nw) {
@@ -281,13 +297,13 @@ __device__ __forceinline__ void batched_prep_block(const BatchArgs &a, const int
             if (isfinite(vi))
                 split_slices(vi, T, wi);
         }
-        unsigned char *o = out + (w >> 5) * kWSlices * kWBlock;
+        unsigned char *o = out + (w >> 5) * kWSlices * wblock;
 #pragma unroll
         for (int p = 0; p < kWSlices; ++p) {
             const float r = (float)wr[p], i = (float)wi[p];
-            unsigned char *q = o + p * kWBlock;
-            *reinterpret_cast<unsigned *>(q + sw128(2 * sl, 4 * (w & 31))) = pack_bf16x2(r, -i);
-            *reinterpret_cast<unsigned *>(q + sw128(2 * sl + 1, 4 * (w & 31))) = pack_bf16x2(i, r);
+            unsigned char *q = o + p * wblock;
+            *reinterpret_cast<unsigned *>(q + sw128(rl, 4 * (w & 31))) = pack_bf16x2(r, -i);
+            *reinterpret_cast<unsigned *>(q + sw128(rl + 1, 4 * (w & 31))) = pack_bf16x2(i, r);
         }
     }
 }
@@ -326,40 +342,46 @@ struct TileRange {
 // The CTA's barriers and small state (declared once per kernel, so that the
 // several instantiations of the body in one kernel share them).
 struct BatchShared {
-    uint64_t w_full, x_full[kXSMax], x_empty[kXSMax], s_full, s_free, r_full, r_free, g_done;
+    uint64_t w_full, x_full[kXSMax], x_empty[kXSMax], s_full[2], s_free[2], r_full, r_free, g_done;
     uint32_t tmem_base;
     int s_flags;
     unsigned s_kflags[2 * kMaxChunks];
 };
 
-template <int F, int XS>
+// NB accumulator buffers (and groups of epilogue warps): 1 for steps of 32 sets; 2
+// for K <= 16, one step of 16 sets a tile.
+template <int F, int XS, int NB>
 __device__ __forceinline__ void batched_body(const BatchArgs &a,
                                              const TileRange &tr, unsigned char *smem_dyn,
                                              BatchShared &sh)
 {
     constexpr int KB = (F + 63) / 64;
-    constexpr int kGCol = s_cols(XS);
+    constexpr int QS = 32 / NB, SPC = kKC / 32;           // sets of a step, steps of a chunk
+    constexpr int AC = 2 * QS;                            // columns of one accumulator
+    constexpr int kGCol = s_cols(XS), kSCol = kGCol / NB; // G^T; one group's accumulators
+    constexpr uint32_t kWBlock = 2 * QS * 128;            // rows (k,re/im) x 64 BF16 features
     constexpr uint32_t kXBlk = XS * F * 128;    // one 64-event block: x0 (and x1) rows
     constexpr uint32_t kXBytes = 2 * kXBlk;     // one stage
-    uint64_t &w_full = sh.w_full, &s_full = sh.s_full, &s_free = sh.s_free, &r_full = sh.r_full,
-             &r_free = sh.r_free, &g_done = sh.g_done;
-    uint64_t *x_full = sh.x_full, *x_empty = sh.x_empty;
+    uint64_t &w_full = sh.w_full, &r_full = sh.r_full, &r_free = sh.r_free, &g_done = sh.g_done;
+    uint64_t *x_full = sh.x_full, *x_empty = sh.x_empty, *s_full = sh.s_full, *s_free = sh.s_free;
     uint32_t &tmem_base = sh.tmem_base;
     int &s_flags = sh.s_flags;
     unsigned *s_kflags = sh.s_kflags;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the warp's number as a value the compiler knows to be the same in every lane:
+    // what the issuer's branch computes can then stay in uniform registers
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int NCH = a.n_chunks;
-    // half chunks per tile that hold parameter sets (a last half past K is skipped)
-    const int HPT = batch_hpt(a.K);
-    const Smem L = batch_smem(F, XS, HPT, a.nxs_req);
+    // steps per tile that hold parameter sets (those past K are skipped)
+    const int SPT = (a.K + QS - 1) / QS;
+    const Smem L = batch_smem(F, XS, a.K, a.nxs_req);
     const int NXS = L.nxs;
     unsigned char *base = smem_dyn + ((1024 - (smem_u32(smem_dyn) & 1023)) & 1023);
     unsigned char *sW = base + L.w_off;
     unsigned char *sX = base + L.x_off;
     unsigned char *sR = base + L.r_off;
     const int n_my = tr.n_tiles;
-    const int steps = n_my * HPT;
+    const int steps = n_my * SPT;
 
     if (threadIdx.x == 0) {
         mbar_init(&w_full, 1);
@@ -367,9 +389,11 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
             mbar_init(&x_full[s], 1);
             mbar_init(&x_empty[s], 1);
         }
-        mbar_init(&s_full, 1);
-        mbar_init(&s_free, kEpiWarps);
-        mbar_init(&r_full, kEpiWarps);
+        for (int b = 0; b < NB; ++b) {
+            mbar_init(&s_full[b], 1);
+            mbar_init(&s_free[b], kEpiWarps / NB);
+        }
+        mbar_init(&r_full, kEpiWarps / NB);
         mbar_init(&r_free, 1);
         mbar_init(&g_done, 1);
         fence_barrier_init();
@@ -382,7 +406,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
     int flags = 0;
 
     if (warp == kEpiWarps) {
@@ -410,147 +434,177 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
                 flags |= FLAG_TIMEOUT;
         }
     } else if (warp == kEpiWarps + 1) {
-        // ---- MMA issuer ---------------------------------------------------
-        if (lane == 0) {
-            const uint32_t id64 = umma_idesc_bf16(128, 64, 1, 0);
-            const uint32_t id128 = umma_idesc_bf16(128, 128, 1, 0);
-            const uint32_t id192 = umma_idesc_bf16(128, 192, 1, 0);
-            const uint32_t id2 = umma_idesc_bf16(128, XS * F, 1, 0);
-            const uint32_t xbase = smem_u32(sX), wbase = smem_u32(sW), rbase = smem_u32(sR);
-            // descriptors without their start address (added as address / 16 below)
-            const uint64_t dA = umma_desc_sw128(0, kXBlk, 1024);      // X, MN-major
-            const uint64_t dR = umma_desc_sw128(0, 128 * 128, 1024);  // R', MN-major
-            const uint64_t dK = umma_desc_sw128(0, 16, 1024);         // K-major operands
-            // GEMM 2 of chunk step cq (its R' complete: r_full phase cq)
-            auto gemm2 = [&](int cq) {
-                const int j = cq / NCH, c = cq % NCH, s = j % NXS;
-                tc_fence_after();
-                const uint32_t xs = xbase + s * kXBytes;
+        // ---- MMA issuer: the warp runs as one, an elected lane issues ------
+        const bool lead = elect_one();
+        auto test = [&](uint64_t *bar, uint32_t parity) {
+            return (bool)__all_sync(0xffffffffu, mbar_test(bar, parity));
+        };
+        const uint32_t id_w1 = umma_idesc_bf16(128, AC, 1, 0);      // one, two, three slices of W
+        const uint32_t id_w2 = umma_idesc_bf16(128, 2 * AC, 1, 0);
+        const uint32_t id_w3 = umma_idesc_bf16(128, 3 * AC, 1, 0);
+        const uint32_t id2 = umma_idesc_bf16(128, XS * F, 1, 0);
+        const uint32_t xbase = smem_u32(sX), wbase = smem_u32(sW), rbase = smem_u32(sR);
+        // descriptors without their start address (added as address / 16 below)
+        const uint64_t dA = umma_desc_sw128(0, kXBlk, 1024);      // X, MN-major
+        const uint64_t dR = umma_desc_sw128(0, 128 * 128, 1024);  // R', MN-major
+        const uint64_t dK = umma_desc_sw128(0, 16, 1024);         // K-major operands
+        // GEMM 2 does not wait in line behind GEMM 1: while the warp waits for what a
+        // GEMM 1 needs, it issues the GEMM 2 of each chunk step whose R' is complete,
+        // in order. It polls without sleeping: a suspended thread was measured to
+        // resume up to ~1300 cycles after the phase completed, on the critical path of
+        // GEMM 1. GEMM 1 of the first step of chunk cq needs the GEMM 2 of
+        // cq - 2 issued: its completion, seen by the epilogue as s_full, then implies
+        // that r_free has passed phase cq - 2, so the epilogue's parity wait for phase
+        // cq - 1 cannot match an older phase. Bounded as mbar_wait. Everything in this
+        // loop is on the critical path (a step is ~2000 cycles), so tiles, chunks and
+        // stages are counted, not divided.
+        int g2 = 0, g2_ready = 0;       // next GEMM 2; chunk steps whose GEMM 1s are issued
+        int g2_c = 0, g2_s = 0;         // its chunk, its stage
+        uint32_t g2_acc = 0;            // 0 for the first tile
+        bool ok = __all_sync(0xffffffffu, mbar_wait(&w_full, 0));
+        int c0 = 0, ch = 0, s = 0;      // chunk steps before this tile, step of the tile, its stage
+        uint32_t xph = 0;               // parity of the stage's use
+        for (int q = 0; q <= steps && ok; ++q) {
+            const bool last = q == steps;           // only the GEMM 2s that are left
+            const int c = ch / SPC;
+            const int need = last ? g2_ready : ch % SPC == 0 ? c0 + c - 1 : 0;
+            bool wx = !last && ch == 0, ws = !last && q >= NB;
+            unsigned long long t0 = 0;
+            for (unsigned it = 1;; ++it) {
+                if (g2 < g2_ready && test(&r_full, g2 & 1)) {
+                    tc_fence_after();
+                    const uint32_t xs = xbase + g2_s * kXBytes;
+                    if (lead) {
 #pragma unroll
-                for (int ks = 0; ks < kBM / 16; ++ks) {
-                    const uint32_t ra = rbase + ks * 2048;
-                    const uint32_t xa = xs + (ks >> 2) * kXBlk + (ks & 3) * 32;
-                    umma_bf16(tmem + kGCol + c * XS * F, dR + (ra >> 4), dK + (xa >> 4), id2,
-                              (j > 0 || ks > 0) ? 1u : 0u);
-                }
-                umma_commit(&r_free);
-                if (c == NCH - 1)
-                    umma_commit(&x_empty[s]);
-            };
-            // GEMM 2 does not wait in line behind GEMM 1: while the thread
-            // waits for a barrier (bar, parity), it issues the GEMM 2 of each
-            // chunk step whose R' is complete, in order, and returns once the
-            // barrier's phase is complete and at least `need` GEMM 2s are
-            // issued (bar = null: the barrier part holds). It polls without
-            // sleeping: a suspended thread was measured to resume up to ~1300
-            // cycles after the phase completed, on the critical path of GEMM 1.
-            // GEMM 1 of the first half of
-            // chunk step cq needs the GEMM 2 of cq - 2 issued: its completion,
-            // seen by the epilogue as s_full, then implies that r_free has
-            // passed phase cq - 2, so the epilogue's parity wait for phase
-            // cq - 1 cannot match an older phase. Bounded as mbar_wait.
-            int g2 = 0, g2_ready = 0;   // next GEMM 2; chunk steps whose GEMM 1s are issued
-            auto serve = [&](uint64_t *bar, uint32_t parity, int need) -> bool {
-                const unsigned long long t0 = global_timer_ns();
-                for (unsigned it = 1;; ++it) {
-                    if (g2 < g2_ready && mbar_test(&r_full, g2 & 1)) {
-                        gemm2(g2++);
-                        continue;
+                        for (int ks = 0; ks < kBM / 16; ++ks) {
+                            const uint32_t ra = rbase + ks * 2048;
+                            const uint32_t xa = xs + (ks >> 2) * kXBlk + (ks & 3) * 32;
+                            umma_bf16(tmem + kGCol + g2_c * XS * F, dR + (ra >> 4), dK + (xa >> 4), id2,
+                                      ks > 0 ? 1u : g2_acc);
+                        }
+                        umma_commit(&r_free);
+                        if (g2_c == NCH - 1)
+                            umma_commit(&x_empty[g2_s]);
                     }
-                    if (g2 >= need && (!bar || mbar_test(bar, parity)))
-                        return true;
-                    if ((it & 255) == 0 && global_timer_ns() - t0 > kWaitLimitNs)
-                        return false;
+                    __syncwarp();
+                    ++g2;
+                    if (++g2_c == NCH) {
+                        g2_c = 0;
+                        g2_acc = 1;
+                        if (++g2_s == NXS)
+                            g2_s = 0;
+                    }
+                    continue;
                 }
-            };
-            bool ok = mbar_wait(&w_full, 0);
-            for (int q = 0; q < steps && ok; ++q) {
-                const int j = q / HPT, ch = q % HPT, c = ch >> 1, h = ch & 1, s = j % NXS;
-                const int need = h == 0 ? j * NCH + c - 1 : 0;
-                if (ch == 0 && !serve(&x_full[s], (j / NXS) & 1, need)) {
-                    ok = false;
-                    break;
+                if (g2 >= need) {
+                    if (wx)
+                        wx = !test(&x_full[s], xph);
+                    if (ws)
+                        ws = !test(&s_free[q % NB], (q / NB - 1) & 1);
+                    if (!wx && !ws)
+                        break;
                 }
-                if (q >= 1 && !serve(&s_free, (q - 1) & 1, need)) {
-                    ok = false;
-                    break;
+                if ((it & 255) == 0) {
+                    const unsigned long long t = global_timer_ns();
+                    if (it == 256)
+                        t0 = t;
+                    if (__any_sync(0xffffffffu, t - t0 > kWaitLimitNs)) {
+                        ok = false;
+                        break;
+                    }
                 }
-                tc_fence_after();
-                const uint32_t xs = xbase + s * kXBytes;
-                const uint32_t wb = wbase + (uint32_t)(c * 2 + h) * KB * kWSlices * kWBlock;
-                // accumulator j (64 columns at 64 j) collects the slice products x_i w_p, i + p = j
+            }
+            if (last || !ok)
+                break;
+            tc_fence_after();
+            const uint32_t xs = xbase + s * kXBytes;
+            const uint32_t wb = wbase + (uint32_t)ch * KB * kWSlices * kWBlock;
+            const uint32_t sb = tmem + (q % NB) * kSCol;
+            if (lead) {
+                // accumulator j (columns from AC j on) collects the slice products x_i w_p, i + p = j
 #pragma unroll
                 for (int ks = 0; ks < F / 16; ++ks) {
                     const uint32_t x0a = xs + ks * 2048;
                     const uint32_t wa = wb + (ks >> 2) * kWSlices * kWBlock + (ks & 3) * 32;
-                    const uint32_t acc = ks > 0 ? 1u : 0u;
+                    // x0 [w0|w1|w2] into acc0..2 and x1 [w0|w1|w2] into acc1..3: two
+                    // products of three slices per K step; in the first, acc3 is
+                    // started by x1 w2 alone (one accumulate flag per MMA)
+                    umma_bf16(sb, dA + (x0a >> 4), dK + (wa >> 4), id_w3, ks > 0 ? 1u : 0u);
                     if (XS == 2) {
-                        // x0 [w0|w1|w2] into acc0..2 and x1 [w0|w1|w2] into acc1..3:
-                        // two N = 192 products per K step; in the first, acc3
-                        // is started by x1 w2 alone (one accumulate flag per MMA)
                         const uint32_t x1a = x0a + F * 128;
-                        umma_bf16(tmem, dA + (x0a >> 4), dK + (wa >> 4), id192, acc);        // acc0..2 x0 [w0|w1|w2]
                         if (ks == 0) {
-                            umma_bf16(tmem + 192, dA + (x1a >> 4), dK + ((wa + 2 * kWBlock) >> 4), id64,
-                                      0u);                                                   // acc3    x1 w2
-                            umma_bf16(tmem + 64, dA + (x1a >> 4), dK + (wa >> 4), id128, 1u);  // acc1..2 x1 [w0|w1]
+                            umma_bf16(sb + 3 * AC, dA + (x1a >> 4), dK + ((wa + 2 * kWBlock) >> 4), id_w1, 0u);
+                            umma_bf16(sb + AC, dA + (x1a >> 4), dK + (wa >> 4), id_w2, 1u);
                         } else {
-                            umma_bf16(tmem + 64, dA + (x1a >> 4), dK + (wa >> 4), id192, 1u);  // acc1..3 x1 [w0|w1|w2]
+                            umma_bf16(sb + AC, dA + (x1a >> 4), dK + (wa >> 4), id_w3, 1u);
                         }
-                    } else {
-                        umma_bf16(tmem, dA + (x0a >> 4), dK + (wa >> 4), id192, acc);        // acc0..2 x0 [w0|w1|w2]
                     }
                 }
-                umma_commit(&s_full);
-                if (h == 1 || ch == HPT - 1)  // the chunk step's last GEMM 1
-                    g2_ready = j * NCH + c + 1;
+                umma_commit(&s_full[q % NB]);
             }
-            if (ok && !serve(nullptr, 0, g2_ready))
-                ok = false;
-            umma_commit(&g_done);
-            // tensor memory is released only after every product has finished
-            if (!mbar_wait(&g_done, 0))
-                ok = false;
-            if (!ok)
-                flags |= FLAG_TIMEOUT;
+            __syncwarp();
+            if (ch % SPC == SPC - 1 || ch == SPT - 1)  // the chunk step's last GEMM 1
+                g2_ready = c0 + c + 1;
+            if (++ch == SPT) {
+                ch = 0;
+                c0 += NCH;
+                if (++s == NXS) {
+                    s = 0;
+                    xph ^= 1;
+                }
+            }
         }
+        if (lead)
+            umma_commit(&g_done);
+        __syncwarp();
+        // tensor memory is released only after every product has finished
+        if (!mbar_wait(&g_done, 0))
+            ok = false;
+        if (!ok)
+            flags |= FLAG_TIMEOUT;
     } else if (warp < kEpiWarps) {
         // ---- epilogue -------------------------------------------------------
-        const int qq = warp & 3, sg = warp >> 2;
+        // NB groups take the steps in turn; a warp takes 8 sets of a step
+        const int qq = warp & 3, grp = NB == 2 ? warp >> 3 : 0, s8 = (warp >> 2) % (4 / NB);
         const int e = qq * 32 + lane;                  // event row of the tile = TMEM lane
         const uint32_t lane_addr = (uint32_t)(qq * 32) << 16;
-        // per-thread constants: R' store offsets, the atomic partials of this lane
-        const uint32_t st0 = sw128(e, 32 * sg), st1 = sw128(e, 32 * sg + 16);
+        const uint32_t s_addr = tmem + lane_addr + grp * kSCol + 16 * s8;
+        // R' store offsets, the atomic partials of this lane
+        const uint32_t st0 = sw128(e, 32 * s8), st1 = sw128(e, 32 * s8 + 16);
         unsigned long long *lp = reinterpret_cast<unsigned long long *>(
-            a.lpart + ((size_t)tr.slot * 4 + qq) * (NCH * kKC) + 8 * sg + lane);
+            a.lpart + ((size_t)tr.slot * 4 + qq) * (NCH * kKC) + 8 * s8 + lane);
         const f2 c8 = pk2(1.0f / 256.0f, 1.0f / 256.0f), one2 = pk2(1.0f, 1.0f);
         int64_t ev = (int64_t)tr.tile0 * kBM + e;          // this thread's event in tile j
         const int64_t ev_step = (int64_t)tr.stride * kBM;
         bool ok = true;
-        int j = 0, ch = 0;                                 // tile, half chunk (q = j HPT + ch)
-        for (int q = 0; q < steps && ok; ++q) {
-            const int h = ch & 1, cq = j * NCH + (ch >> 1);
-            const bool last_half = h == 1 || ch == HPT - 1;
-            if (!mbar_wait(&s_full, q & 1)) {
+        int j = 0, ch = grp;                               // tile, its step (q = j SPT + ch)
+        for (int q = grp; q < steps; q += NB, ch += NB) {
+            while (ch >= SPT) {
+                ch -= SPT;
+                ++j;
+                ev += ev_step;
+            }
+            const int cq = j * NCH + ch / SPC;
+            if (!mbar_wait(&s_full[grp], (q / NB) & 1)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            // a warp whose 8 sets all lie past K (padding of the last half
-            // chunk) keeps to the barriers and does no work: its rows of R'
+            // a warp whose 8 sets all lie past K (padding of the last
+            // step) keeps to the barriers and does no work: its rows of R'
             // feed only the G^T rows of those sets, which are never read
-            const int nvs = a.K - (ch >> 1) * kKC - h * kHS - 8 * sg;
+            const int nvs = a.K - ch * QS - 8 * s8;
             const bool idle = nvs <= 0;
             // Q = acc0 + (acc1 + (acc2 + acc3 / 2^8) / 2^8) / 2^8 of this warp's
             // 8 sets, as (re, im) pairs
             f2 qv[8];
             if (!idle) {
                 uint32_t v0[16], v1[16], v2[16], v3[16];
-                tmem_ld16(tmem + lane_addr + 16 * sg, v0);
-                tmem_ld16(tmem + lane_addr + 64 + 16 * sg, v1);
-                tmem_ld16(tmem + lane_addr + 128 + 16 * sg, v2);
+                tmem_ld16(s_addr, v0);
+                tmem_ld16(s_addr + AC, v1);
+                tmem_ld16(s_addr + 2 * AC, v2);
                 if (XS == 2)
-                    tmem_ld16(tmem + lane_addr + 192 + 16 * sg, v3);
+                    tmem_ld16(s_addr + 3 * AC, v3);
                 tmem_ld_wait();
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
@@ -564,7 +618,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
             tc_fence_before();
             __syncwarp();
             if (lane == 0)
-                mbar_arrive(&s_free);
+                mbar_arrive(&s_free[grp]);
             uint32_t rpk[8];
             int l[8];
             if (!idle && ev < a.n_events) {
@@ -601,7 +655,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
                         float qr, qi;
                         upk2(qv[t], qr, qi);
                         if (t < nvs && fmaf(qr, qr, qi * qi) == 0.f)
-                            atomicOr(&s_kflags[ch], 1u << (8 * sg + t));
+                            atomicOr(&s_kflags[ch], 1u << (8 * s8 + t));
                     }
                 }
             } else {
@@ -620,28 +674,23 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
                     mine = lane == t ? sum : mine;
                 }
                 if (lane < 8)  // no return value: a fire-and-forget reduction
-                    atomicAdd(lp + ch * kHS, (unsigned long long)(long long)mine);
+                    atomicAdd(lp + ch * QS, (unsigned long long)(long long)mine);
             }
             // R' may be overwritten once GEMM 2 of the previous chunk step is done
-            if (h == 0 && cq >= 1 && !mbar_wait(&r_free, (cq - 1) & 1)) {
+            if (ch % SPC == 0 && cq >= 1 && !mbar_wait(&r_free, (cq - 1) & 1)) {
                 ok = false;
                 break;
             }
-            unsigned char *rrow = sR + h * (128 * 128);
             if (!idle) {
+                unsigned char *rrow = sR + ch % SPC * (128 * 128);
                 *reinterpret_cast<uint4 *>(rrow + st0) = make_uint4(rpk[0], rpk[1], rpk[2], rpk[3]);
                 *reinterpret_cast<uint4 *>(rrow + st1) = make_uint4(rpk[4], rpk[5], rpk[6], rpk[7]);
             }
-            if (last_half) {
+            if (ch % SPC == SPC - 1 || ch == SPT - 1) {  // the chunk's last step
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(&r_full);
-            }
-            if (++ch == HPT) {
-                ch = 0;
-                ++j;
-                ev += ev_step;
             }
         }
         if (!ok)
@@ -650,7 +699,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
         if (ok && mbar_wait(&g_done, 0)) {
             tc_fence_after();
             for (int c = 0; c < NCH; ++c) {
-                for (int c0 = 8 * sg; c0 < F; c0 += 32) {
+                for (int c0 = 8 * (warp >> 2); c0 < F; c0 += 32) {
                     uint32_t g[8], g1[8];
                     if (n_my > 0) {
                         tmem_ld8(tmem + lane_addr + kGCol + c * XS * F + c0, g);
@@ -713,7 +762,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
 }
 
 // One sample, a persistent grid: CTA b takes tiles b, b + grid, ...
-template <int F, int XS>
+template <int F, int XS, int NB>
 __global__ void __launch_bounds__(kThreads, 1)
     batched_kernel(const BatchArgs a, const int n_tiles)
 {
@@ -726,7 +775,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tr.slot = blockIdx.x;
     tr.mv_k0 = blockIdx.x;
     tr.mv_kstride = gridDim.x;
-    batched_body<F, XS>(a, tr, smem_dyn, sh);
+    batched_body<F, XS, NB>(a, tr, smem_dyn, sh);
 }
 
 // Many samples (the uneven model batch) in one launch: CTA b is the work item
@@ -736,7 +785,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // in which the final kernel adds their partials are fixed, so the results
 // do not depend on that schedule. The body is instantiated per feature
 // count F (the tile shape of each wave-count bucket).
-template <int XS>
+template <int XS, int NB>
 __global__ void __launch_bounds__(kThreads, 1)
     batched_items_kernel(const BatchItem *__restrict__ items, const BatchArgs *__restrict__ models)
 {
@@ -752,12 +801,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     tr.mv_k0 = it.slot == 0 ? 0 : a.K;    // the model's first item forms M V
     tr.mv_kstride = 1;
     switch (a.F) {
-    case 16: batched_body<16, XS>(a, tr, smem_dyn, sh); break;
-    case 32: batched_body<32, XS>(a, tr, smem_dyn, sh); break;
-    case 48: batched_body<48, XS>(a, tr, smem_dyn, sh); break;
-    case 64: batched_body<64, XS>(a, tr, smem_dyn, sh); break;
-    case 80: batched_body<80, XS>(a, tr, smem_dyn, sh); break;
-    case 96: batched_body<96, XS>(a, tr, smem_dyn, sh); break;
+    case 16: batched_body<16, XS, NB>(a, tr, smem_dyn, sh); break;
+    case 32: batched_body<32, XS, NB>(a, tr, smem_dyn, sh); break;
+    case 48: batched_body<48, XS, NB>(a, tr, smem_dyn, sh); break;
+    case 64: batched_body<64, XS, NB>(a, tr, smem_dyn, sh); break;
+    case 80: batched_body<80, XS, NB>(a, tr, smem_dyn, sh); break;
+    case 96: batched_body<96, XS, NB>(a, tr, smem_dyn, sh); break;
     default: break;
     }
 }
@@ -919,38 +968,37 @@ __global__ void batched_encode_kernel(const float *__restrict__ planes, int64_t 
     }
 }
 
-template <int F, int XS>
-cudaError_t configure_f()
+template <class Kernel>
+cudaError_t configure_kernel(Kernel *k)
 {
-    return cudaFuncSetAttribute(batched_kernel<F, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kMaxSmem);
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
 }
 
-template <int XS>
-cudaError_t configure_xs()
+template <int XS, int NB>
+cudaError_t configure()
 {
     cudaError_t e = cudaSuccess;
-    for (cudaError_t r : {configure_f<16, XS>(), configure_f<32, XS>(), configure_f<48, XS>(),
-                          configure_f<64, XS>(), configure_f<80, XS>(), configure_f<96, XS>(),
-                          cudaFuncSetAttribute(batched_items_kernel<XS>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               kMaxSmem)})
+    for (cudaError_t r :
+         {configure_kernel(batched_kernel<16, XS, NB>), configure_kernel(batched_kernel<32, XS, NB>),
+          configure_kernel(batched_kernel<48, XS, NB>), configure_kernel(batched_kernel<64, XS, NB>),
+          configure_kernel(batched_kernel<80, XS, NB>), configure_kernel(batched_kernel<96, XS, NB>),
+          configure_kernel(batched_items_kernel<XS, NB>)})
         if (r != cudaSuccess)
             e = r;
     return e;
 }
 
-template <int XS>
+template <int XS, int NB>
 cudaError_t launch_main(int F, int grid, uint32_t smem, cudaStream_t s, const BatchArgs &a,
                         int n_tiles)
 {
     switch (F) {
-    case 16: batched_kernel<16, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
-    case 32: batched_kernel<32, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
-    case 48: batched_kernel<48, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
-    case 64: batched_kernel<64, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
-    case 80: batched_kernel<80, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
-    case 96: batched_kernel<96, XS><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 16: batched_kernel<16, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 32: batched_kernel<32, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 48: batched_kernel<48, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 64: batched_kernel<64, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 80: batched_kernel<80, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
+    case 96: batched_kernel<96, XS, NB><<<grid, kThreads, smem, s>>>(a, n_tiles); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -985,14 +1033,14 @@ int batched_max_k(int n_waves, int xs)
     int nch = kMaxChunks;
     while (nch > 0 &&
            (s_cols(xs) + nch * xs * F > 512 ||
-            (int)batch_smem(F, xs, batch_hpt(nch * kKC)).bytes > kMaxSmem))
+            (int)batch_smem(F, xs, nch * kKC).bytes > kMaxSmem))
         --nch;
     return nch * kKC;
 }
 
 int batched_max_x_stages(int n_waves, int xs, int K)
 {
-    return batch_smem(batched_features(n_waves), xs, batch_hpt(K)).nxs;
+    return batch_smem(batched_features(n_waves), xs, K).nxs;
 }
 
 size_t batched_scratch_bytes(int n_waves, int xs, int K, int grid)
@@ -1002,8 +1050,10 @@ size_t batched_scratch_bytes(int n_waves, int xs, int K, int grid)
 
 cudaError_t batched_configure()
 {
-    const cudaError_t e1 = configure_xs<1>(), e2 = configure_xs<2>();
-    return e1 != cudaSuccess ? e1 : e2;
+    for (cudaError_t e : {configure<1, 1>(), configure<1, 2>(), configure<2, 1>(), configure<2, 2>()})
+        if (e != cudaSuccess)
+            return e;
+    return cudaSuccess;
 }
 
 cudaError_t launch_batched_encode(const float *planes, int64_t pitch, int64_t n, int n_waves, int xs,
@@ -1058,9 +1108,10 @@ cudaError_t launch_batched(const void *xbf, int64_t n_events, int n_waves, int x
     if (e != cudaSuccess)
         return e;
     const int n_tiles = (int)((n_events + kBM - 1) / kBM);
-    const uint32_t smem = batch_smem(F, xs, batch_hpt(K), nxs).bytes;
-    e = xs == 2 ? launch_main<2>(F, grid, smem, s, a, n_tiles)
-                : launch_main<1>(F, grid, smem, s, a, n_tiles);
+    const uint32_t smem = batch_smem(F, xs, K, nxs).bytes;
+    const auto launch = step_sets(K) == 16 ? (xs == 2 ? launch_main<2, 2> : launch_main<1, 2>)
+                                           : (xs == 2 ? launch_main<2, 1> : launch_main<1, 1>);
+    e = launch(F, grid, smem, s, a, n_tiles);
     if (e != cudaSuccess)
         return e;
     batched_finalize<<<K, kFinWarps * 32, 0, s>>>(a, grid, done, nll, grad);
@@ -1225,7 +1276,7 @@ cudaError_t launch_batched_items(void *plan, const BatchModelDesc *models, int n
     uint32_t smem = 0;
     for (int i = 0; i < n_models; ++i)
         smem = std::max(smem,
-                        batch_smem(batched_features(models[i].n_waves), xs, batch_hpt(K), nxs).bytes);
+                        batch_smem(batched_features(models[i].n_waves), xs, K, nxs).bytes);
     cudaError_t e = cudaMemsetAsync(d + p.zero, 0, p.zero_bytes, s);
     if (e != cudaSuccess)
         return e;
@@ -1236,10 +1287,10 @@ cudaError_t launch_batched_items(void *plan, const BatchModelDesc *models, int n
         return e;
     const BatchItem *items = reinterpret_cast<const BatchItem *>(d + p.items);
     const int n_items = (int)p.items_h.size();
-    if (xs == 2)
-        batched_items_kernel<2><<<n_items, kThreads, smem, s>>>(items, args);
-    else
-        batched_items_kernel<1><<<n_items, kThreads, smem, s>>>(items, args);
+    const auto kernel = step_sets(K) == 16
+                            ? (xs == 2 ? batched_items_kernel<2, 2> : batched_items_kernel<1, 2>)
+                            : (xs == 2 ? batched_items_kernel<2, 1> : batched_items_kernel<1, 1>);
+    kernel<<<n_items, kThreads, smem, s>>>(items, args);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     batched_items_finalize<<<n_models * K, kFinWarps * 32, 0, s>>>(
