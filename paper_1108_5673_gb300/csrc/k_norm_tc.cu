@@ -63,11 +63,15 @@
 //
 // Bound: the digit split (30 packed FP32 operations per two rows and four
 // events, on six warps) and the MMAs, about 1300 and 1024 cycles per tile at
-// 32 waves, overlapping in part. Per call of pwa_build_norm: 10M x 32 in 0.94
-// ms (2.7 TB/s of amplitudes), 5M x 20 in 0.35 ms, 10M x 12 in 0.41 ms, 4M x
-// 48 in 1.18 ms; before, with one-warp consumers per tile, 0.49 ms at 5M x 20
-// and 0.63 at 10M x 12, and on the FP64 pipe beyond 20 waves 81 ms at 10M x
-// 32 and 69 ms at 4M x 48.
+// 32 waves, overlapping in part; at few waves the fixed cost of a tile, ~600 cycles
+// (a copy 430, a step of the issuer). Producer and issuer run as converged warps
+// with one elected lane issuing, so that their addresses and descriptors stay in
+// uniform registers: as single lanes they took 5M x 4 from 183 to 207 us a call, 5M
+// x 16 from 305 to 340, 10M x 12 from 381 to 404, 5M x 20 from 334 to 352. Per call
+// of pwa_build_norm: 10M x 32 in 0.92 ms (2.8 TB/s of amplitudes), 5M x 20 in 0.33
+// ms, 10M x 12 in 0.38 ms, 4M x 48 in 1.16 ms; before, with one-warp consumers per
+// tile, 0.49 ms at 5M x 20 and 0.63 at 10M x 12, and on the FP64 pipe beyond 20
+// waves 81 ms at 10M x 32 and 69 ms at 4M x 48.
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -231,7 +235,9 @@ __global__ void __launch_bounds__(kNThreads, 1)
     __shared__ uint32_t tmem_base;
     __shared__ int s_flags;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the warp's number as a value the compiler knows to be the same in every lane:
+    // what the producer and the issuer compute can then stay in uniform registers
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     // tiles of this CTA: blockIdx.x + j gridDim.x, j < n_my; tile j goes to
     // consumer group j % GROUPS, TMA stage j % STAGES, digit buffer j % NBUF
     const int n_my =
@@ -286,50 +292,52 @@ __global__ void __launch_bounds__(kNThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
     int flags = 0;
 
     if (warp == 0) {
-        // ---- producer: one thread issues the TMA copies --------------------
-        if (lane == 0) {
-            int j = n_first;
-            for (; j < n_my; ++j) {
-                if (!mbar_wait(&empty[j % STAGES], (uint32_t)(j / STAGES - 1) & 1)) {
-                    flags |= FLAG_TIMEOUT;
-                    break;
-                }
-                issue(j);
+        // ---- producer: the warp runs as one, an elected lane issues the copies ----
+        const bool lead = elect_one();
+        int j = n_first;
+        for (; j < n_my; ++j) {
+            if (!warp_wait(&empty[j % STAGES], (uint32_t)(j / STAGES - 1) & 1)) {
+                flags |= FLAG_TIMEOUT;
+                break;
             }
-            // no copy may still be landing in shared memory when the CTA exits
-            for (int q = (j > STAGES ? j - STAGES : 0); q < j; ++q)
-                if (!mbar_wait(&full[q % STAGES], (uint32_t)(q / STAGES) & 1))
-                    flags |= FLAG_TIMEOUT;
+            if (lead)
+                issue(j);
+            __syncwarp();
         }
+        // no copy may still be landing in shared memory when the CTA exits
+        for (int q = (j > STAGES ? j - STAGES : 0); q < j; ++q)
+            if (!mbar_wait(&full[q % STAGES], (uint32_t)(q / STAGES) & 1))
+                flags |= FLAG_TIMEOUT;
     } else if (warp == 1) {
-        // ---- MMA issuer ----------------------------------------------------
-        if (lane == 0) {
-            const uint32_t id1 = umma_idesc_bf16(128, C::NI1, 0, 0);
-            const uint32_t id2 = umma_idesc_bf16(128, C::N2, 0, 0);
-            const uint64_t dK = umma_desc_sw128(0, 16, 1024);
-            const uint32_t row2 = (uint32_t)(S1 * R) * 128u;  // byte offset of digit S1 + 1's rows
-            bool ok = true;
-            for (int j = 0; j < n_my; ++j) {
-                const int b = j % NBUF;
-                if (!mbar_wait(&jfull[b], (uint32_t)(j / NBUF) & 1)) {
-                    ok = false;
-                    break;
-                }
-                const int P = j / kNPeriod, set = P % NACC;
-                const bool first = (j % kNPeriod) == 0;
-                const bool last = (j % kNPeriod) == kNPeriod - 1 || j == n_my - 1;
-                const uint32_t jb = jbase + (uint32_t)b * C::JBYTES;
-                const uint32_t acc1 = tmem + (uint32_t)set * (C::N1 + C::N2), acc2 = acc1 + C::N1;
-                // an accumulator is free once the period NACC before has been drained
-                if (first && P >= NACC && !mbar_wait(&accempty[2 * set], (uint32_t)(P / NACC - 1) & 1)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
+        // ---- MMA issuer: as the producer -----------------------------------
+        const bool lead = elect_one();
+        const uint32_t id1 = umma_idesc_bf16(128, C::NI1, 0, 0);
+        const uint32_t id2 = umma_idesc_bf16(128, C::N2, 0, 0);
+        const uint64_t dK = umma_desc_sw128(0, 16, 1024);
+        const uint32_t row2 = (uint32_t)(S1 * R) * 128u;  // byte offset of digit S1 + 1's rows
+        bool ok = true;
+        for (int j = 0; j < n_my; ++j) {
+            const int b = j % NBUF;
+            if (!warp_wait(&jfull[b], (uint32_t)(j / NBUF) & 1)) {
+                ok = false;
+                break;
+            }
+            const int P = j / kNPeriod, set = P % NACC;
+            const bool first = (j % kNPeriod) == 0;
+            const bool last = (j % kNPeriod) == kNPeriod - 1 || j == n_my - 1;
+            const uint32_t jb = jbase + (uint32_t)b * C::JBYTES;
+            const uint32_t acc1 = tmem + (uint32_t)set * (C::N1 + C::N2), acc2 = acc1 + C::N1;
+            // an accumulator is free once the period NACC before has been drained
+            if (first && P >= NACC && !warp_wait(&accempty[2 * set], (uint32_t)(P / NACC - 1) & 1)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            if (lead) {
 #pragma unroll
                 for (int ks = 0; ks < kNTE / 16; ++ks) {
                     const uint32_t a = jb + (uint32_t)ks * 32;  // 16 events = 32 bytes of a row
@@ -341,31 +349,40 @@ __global__ void __launch_bounds__(kNThreads, 1)
                 }
                 if (last)
                     umma_commit(&accfull[2 * set]);
-                if constexpr (C::B2 > 0) {
-                    if (first && P >= NACC &&
-                        !mbar_wait(&accempty[2 * set + 1], (uint32_t)(P / NACC - 1) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-    #pragma unroll
+            }
+            __syncwarp();
+            if constexpr (C::B2 > 0) {
+                if (first && P >= NACC &&
+                    !warp_wait(&accempty[2 * set + 1], (uint32_t)(P / NACC - 1) & 1)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                if (lead) {
+#pragma unroll
                     for (int ks = 0; ks < kNTE / 16; ++ks) {
                         const uint32_t a = jb + row2 + (uint32_t)ks * 32;
                         umma_bf16(acc2, dK + (a >> 4), dK + (a >> 4), id2, (first && ks == 0) ? 0u : 1u);
                     }
                 }
+                __syncwarp();
+            }
+            if (lead) {
                 // on completion the digit buffer is free again
                 umma_commit(&jempty[b]);
                 if (C::B2 > 0 && last)
                     umma_commit(&accfull[2 * set + 1]);
             }
-            umma_commit(&g_done);
-            // tensor memory is released only after every product has finished
-            if (!mbar_wait(&g_done, 0))
-                ok = false;
-            if (!ok)
-                flags |= FLAG_TIMEOUT;
+            __syncwarp();
         }
+        if (lead)
+            umma_commit(&g_done);
+        __syncwarp();
+        // tensor memory is released only after every product has finished
+        if (!mbar_wait(&g_done, 0))
+            ok = false;
+        if (!ok)
+            flags |= FLAG_TIMEOUT;
     } else if (warp < kNFirstCons) {
         // ---- drain: lane quarter q, rows m = 32 q + lane, columns half h ----
         // Row m holds row p = m % R of digit m / R of each MMA's A operand;

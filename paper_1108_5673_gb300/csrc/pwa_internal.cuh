@@ -110,6 +110,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
     }
 }
 
+// The same by a converged warp, with a result the compiler knows to be uniform.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity,
+                                          unsigned long long limit_ns = kWaitLimitNs)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
+
 // 2D tiled TMA load global -> shared, completion signalled on `bar`.
 // x is the innermost coordinate (elements); x * sizeof(elem) must be a
 // multiple of 16 bytes.
