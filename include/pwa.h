@@ -125,7 +125,7 @@ int pwa_load_events(pwa_ctx *ctx, const void *data_amp, int64_t n_data,
  *   A_a(Omega) = BW(m; M_a, G_a) Y_{l_a}^{m_a}(theta, phi),
  *   BW(m; M, G) = 1 / (M^2 - m^2 - i M G)   (fixed-width Breit-Wigner),
  *   Y_l^m the orthonormal spherical harmonic with the Condon-Shortley phase,
- * in double precision, each amplitude rounded once to float. */
+ * each component the float nearest to its double-precision value. */
 typedef struct pwa_wave {
     double mass;   /* M > 0 (GeV) */
     double width;  /* G > 0 (GeV) */
@@ -196,7 +196,7 @@ int pwa_load_events_incoherent(pwa_ctx *ctx, int n_lambda, const void *data_amp,
  *     with Q^2 = p.p/4 - mK^2, B2(Q) = sqrt(13 / (Q^4 + 3 Q^2 Q0^2 + 9 Q0^4)),
  *     Q0 = 0.197327 GeV (the spin-2 Blatt-Weisskopf barrier);
  *   BW(s) = 1 / (M^2 - s - i M G).
- * Evaluated in double precision, each amplitude rounded once to float. */
+ * Each component is the float nearest to its double-precision value. */
 typedef struct pwa_cov_wave {
     double mass;   /* M > 0 (GeV) */
     double width;  /* G > 0 (GeV) */

@@ -219,9 +219,9 @@ __device__ __forceinline__ f2 log2_fixed2(f2 z)
 }
 
 // A work item of the model batch: tiles [tile0, tile0 + n_tiles) of a model,
-// partial sums at `slot` among that model's.
+// partial sums at `slot` among that model's n_slots.
 struct BatchItem {
-    int model, tile0, n_tiles, slot;
+    int model, tile0, n_tiles, slot, n_slots;
 };
 
 // ---- per-call preparation: W image and set exponents ------------------------
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Many samples (the uneven model batch) in one launch: CTA b is the work item
 // items[b], a contiguous range of one model's tiles; its partials go to the
-// item's slot among the model's, and the model's first item forms M V. The
+// item's slot among the model's, and the model's items share M V. The
 // hardware starts an item's CTA as an SM frees up; the items and the order
 // in which the final kernel adds their partials are fixed, so the results
 // do not depend on that schedule. The body is instantiated per feature
@@ -798,8 +798,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     tr.n_tiles = it.n_tiles;
     tr.stride = 1;
     tr.slot = it.slot;
-    tr.mv_k0 = it.slot == 0 ? 0 : a.K;    // the model's first item forms M V
-    tr.mv_kstride = 1;
+    // M V of the sets shared out over the model's items: in FP64 a set of a large model
+    // takes tens of microseconds, and the first item held its SM for all of them
+    tr.mv_k0 = it.slot;
+    tr.mv_kstride = it.n_slots;
     switch (a.F) {
     case 16: batched_body<16, XS, NB>(a, tr, smem_dyn, sh); break;
     case 32: batched_body<32, XS, NB>(a, tr, smem_dyn, sh); break;
@@ -1159,7 +1161,7 @@ PlanLayout plan_layout(const BatchModelDesc *m, int n_models, int xs, int K, int
         p.slots[i] = n_it;
         for (int k = 0; k < n_it; ++k) {
             const int t0 = (int)((int64_t)tiles * k / n_it), t1 = (int)((int64_t)tiles * (k + 1) / n_it);
-            p.items_h.push_back({i, t0, t1 - t0, k});
+            p.items_h.push_back({i, t0, t1 - t0, k, n_it});
         }
     }
     // largest items first: the hardware hands out CTAs in block order
