@@ -109,6 +109,19 @@ __device__ __forceinline__ f2 rcp2(f2 a)
     return pk2(rcp_approx(x0), rcp_approx(x1));
 }
 
+// A CTA's sum of value `item` of [2][P] (data, MC) for the last CTA, in a.partials
+// [grid][2 P]: the ln I, exponent and intensity sums (the first two of each P) as they
+// are, the gradients, which come from FP32 sums, as float pairs, since the FP64 pipe
+// (1/64 of the FP32 rate) was what the final sums took their time for.
+__device__ __forceinline__ void res_partial(const ResArgs &a, int item, int P, double v)
+{
+    if (item % P >= 2) {
+        const float h = (float)v, l = (float)(v - (double)h);
+        v = __hiloint2double(__float_as_int(l), __float_as_int(h));
+    }
+    a.partials[(size_t)blockIdx.x * 2 * P + item] = v;
+}
+
 template <int NP, int RP>
 __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     nll_res_tma_kernel(const __grid_constant__ CUtensorMap dmap, const __grid_constant__ CUtensorMap mmap,
@@ -508,7 +521,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
             for (int w = 0; w < UNITS; ++w)
                 v += (double)red_f[ph][w][col];
         }
-        a.partials[(size_t)item * gridDim.x + blockIdx.x] = v;
+        res_partial(a, item, P, v);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -521,18 +534,44 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
     __syncthreads();
     if (!s_last)
         return;
-    // ---- last CTA: sums over CTAs in FP64, a warp per value (lane k adds CTAs
-    // k, k + 32, ..., then a fixed shuffle tree) ---------------------------------
+    // ---- last CTA: thread (item, slice) adds every slices-th CTA's value, eight loads
+    // in flight, then the slices in order (a warp per value, its lanes over the CTAs
+    // and FP64 throughout, held up every call by ~8 us: 20 waves, 4 free at 60k + 150k
+    // events 65 us a call, 54 now; 32 waves, 8 free at 20k + 50k 76 and 55) -----------
     __threadfence();
     double *fin = reinterpret_cast<double *>(tiles);   // the ring is idle now
-    for (int item = warp; item < 2 * P; item += blockDim.x / 32) {
+    const int n = 2 * P, slices = max(1, min(8, (int)blockDim.x / n));
+    const int n_cta = gridDim.x;
+    for (int t = threadIdx.x; t < slices * n; t += blockDim.x) {
+        const int item = t % n, sl = t / n;
         double v = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32)
-            v += __ldcg(a.partials + (size_t)item * gridDim.x + b);
-        v = warp_sum(v);
-        if (lane == 0)
-            fin[item] = v;
+        dfloat f = {0.f, 0.f};
+        for (int b0 = sl; b0 < n_cta; b0 += 8 * slices) {
+            double r[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int b = b0 + q * slices;
+                r[q] = b < n_cta ? __ldcg(a.partials + (size_t)b * n + item) : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (item % P < 2)
+                    v += r[q];
+                else
+                    f = df_add(f, dfloat{__int_as_float(__double2loint(r[q])),
+                                         __int_as_float(__double2hiint(r[q]))});
+            }
+        }
+        fin[t] = item % P < 2 ? v : (double)f.hi + (double)f.lo;
     }
+    __syncthreads();
+    double tot = 0.0;
+    if (threadIdx.x < n)
+        for (int sl = 0; sl < slices; ++sl)
+            tot += fin[sl * n + threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x < n)
+        fin[threadIdx.x] = tot;
     __syncthreads();
     const int st = *(volatile int *)a.status;
     const bool dom = (st & FLAG_DOMAIN) != 0, tmo = (st & FLAG_TIMEOUT) != 0;
@@ -554,7 +593,7 @@ cudaError_t launch_nr(const CUtensorMap *dmap, const CUtensorMap *mmap, const Re
 {
     using C = ResTmaCfg<NP, RP>;
     static_assert(C::FITS, "the ring must fit");
-    static_assert((size_t)2 * (2 + 2 * NP + 2 * RP) * 8 <= C::SMEM, "final sums must fit the ring");
+    static_assert((size_t)16 * (2 + 2 * NP + 2 * RP) * 8 <= C::RING_BYTES, "final sums must fit the ring");
     cudaError_t e = cudaFuncSetAttribute(nll_res_tma_kernel<NP, RP>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess)

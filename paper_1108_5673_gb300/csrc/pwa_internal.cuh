@@ -506,7 +506,7 @@ struct ResArgs {
     int64_t mc_pitch, n_mc;
     double inv_ngen;
     const double *V, *mass, *width;  // device
-    double *partials;    // [grid][2][pstride]
+    double *partials;    // 2 pstride grid (the order is the kernel's)
     unsigned *ticket;    // zero on entry, left at zero
     int *status;         // status bits OR-ed here
     int *done;           // incremented once (may be null)
