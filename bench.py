@@ -23,7 +23,7 @@ Other workloads (one JSON line each, same keys):
   incoh_table  the same sample in the table form (table bytes independent of
           the number of components)
   ampgen  amplitudes BW x Y_l^m of 5M events x 20 waves generated on the
-          device from their kinematics (FP64, rounded to complex64)
+          device from their kinematics (as rounded from FP64 to complex64)
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
                   [--workload direct|table|tc|res|models|hessian|weights|incoh|incoh_table|ampgen]
@@ -67,22 +67,21 @@ WORKLOAD = "1M data events x 20 waves (FP32 amplitudes, direct form), M from 5M 
 TRAFFIC = {"direct": 160.139776e6 + 3.347968e6,
            "table": 1600.119e6 + 3.221760e6,
            "tc": 2 * (1024.872e6 + 3.708160e6),        # a step is two launches of 128 sets
-           "res": 1148.176e6 + 3.313920e6,
+           "res": 1148.176e6 + 3.313920e6,             # the same bytes since its S warps
            "models": None,
            "hessian": 160.091648e6 + 3.346944e6,
            "weights": 800.125184e6 + 21.052672e6,
-           "incoh": 320.158464e6 + 3.042048e6,
+           "incoh": None,          # kernel changed since its capture
            "incoh_table": None,   # the table kernel's capture is of the coherent sample
-           "ampgen": 278.9e6 + 962.9e6,   # FP64-bound; DRAM bytes for reference
+           "ampgen": None,         # kernel changed since its capture
            "direct_4M_32": None,   # kernel changed since its capture (four-warp groups, amplitudes re-read)
-           "cov_ampgen": 1233.902e6 + 2723.644e6}   # FP64-bound; DRAM bytes for reference
+           "cov_ampgen": None}     # kernel changed since its capture
 KERNELS = {"direct": "nll_amp_kernel<20, 2>", "table": "nll_table_kernel<20>",
-           "tc": "batched_kernel<64, 2>", "res": "nll_res_tma_kernel<20, 4>",
-           "models": "batched_items_kernel<2> (all models, one launch)", "hessian": "hess_tc_kernel<20>",
-           "weights": "nll_amp_kernel<20, 2, 1, true> (weights mode)", "incoh": "nll_amp_kernel<20, 2, 2>",
+           "tc": "batched_kernel<64, 2, 1>", "res": "nll_res_tma_kernel<20, 4>",
+           "models": "batched_items_kernel<2, 2> (all models, one launch)", "hessian": "hess_tc_kernel<20>",
+           "weights": "nll_amp_kernel<20, 2, true> (weights mode)", "incoh": "nll_split_kernel<20, 2>",
            "incoh_table": "nll_table_kernel<20>", "ampgen": "amp_gen_kernel",
            "direct_4M_32": "nll_amp_kernel<32, 2>", "cov_ampgen": "cov_amp_kernel"}
-FP64_NOMINAL_TFLOPS = 1.25   # GB300 dense FP64 (nominal)
 HBM_NOMINAL_GBS = 7900.0     # GB300 HBM3e (nominal), beside the measured copy peak
 BF16_NOMINAL_TFLOPS = 2250.0  # GB300 dense bf16 (nominal)
 DEFAULT_STEPS = {"direct": 3000, "table": 1000, "tc": 300, "res": 1000, "models": 100,
@@ -492,7 +491,7 @@ def job_incoh(pwa, torch, stream, local, rank, form="amp"):
 
 
 def ampgen_flops(waves):
-    """FP64 operations per event of the generator as written: 6 per power of
+    """Real operations per event of the generator's formulas: 6 per power of
     e^{i phi} up to max |m|, and per wave 4 per step of P_m^m, 7 per step of
     the recurrence in l, 20 for the normalisation, Breit-Wigner and complex
     product (divisions and the one sincos counted as one operation each)."""
@@ -523,18 +522,18 @@ def job_ampgen(pwa, torch, stream, local, rank):
         name="ampgen", lib=L, step=lambda: L.amplitudes(waves, kin, out),
         host_step=lambda: L.amplitudes(waves, kin_h), sync=lambda: L.last_status,
         evals_per_step=1, launches_per_step=1, flush=False,
-        metric="amplitude-generation passes/s (5M events x 20 waves, BW x Y_l^m); % FP64 peak",
+        metric="amplitude-generation passes/s (5M events x 20 waves, BW x Y_l^m); % HBM",
         unit="passes/s",
         workload="amplitudes BW x Y_l^m of 5M events x 20 waves from device-resident "
-                 "kinematics (FP64 arithmetic, complex64 out to a device buffer)",
+                 "kinematics (as rounded from FP64 to complex64, out to a device buffer)",
         config={"n_waves": N_WAVES, "n_events": n, "flops_per_event": ampgen_flops(waves)},
-        roof={"bound": "alu", "flops": float(ampgen_flops(waves)) * n},
+        roof={"bound": "hbm", "bytes": (24.0 + 8.0 * N_WAVES) * n},
         dtype="f64", h2d=24 * n, d2h=8 * N_WAVES * n, cpu_baseline=cpu_baseline,
         note="e2e passes host kinematics in (120 MB) and takes the amplitudes back (800 MB)")
 
 
 def cov_ampgen_flops(n_waves):
-    """FP64 operations per event of the covariant generator as written, each
+    """Real operations per event of the covariant generator's formulas, each
     +, -, x, fma, division and square root counted as one: ~357 for the
     four-vectors, r~, the barrier factor, the photon polarisations and the
     spin-0 and spin-2 contractions of the four components (every metric dot
@@ -565,14 +564,14 @@ def job_cov_ampgen(pwa, torch, stream, local, rank):
         host_step=lambda: L.covariant_amplitudes(waves, p3_h), sync=lambda: L.last_status,
         evals_per_step=1, launches_per_step=1, flush=False,
         metric="covariant amplitude passes/s (5M J/psi -> gamma K+ K- events x 12 waves x 4 "
-               "components); % FP64 peak",
+               "components); % HBM",
         unit="passes/s",
         workload="covariant tensor amplitudes of J/psi -> gamma X, X -> K+ K- (spins 0 and 2) for "
-                 "5M events x 12 waves x 4 components from device-resident 3-momenta (FP64 "
-                 "arithmetic, complex64 out to a device buffer)",
+                 "5M events x 12 waves x 4 components from device-resident 3-momenta (as rounded "
+                 "from FP64 to complex64, out to a device buffer)",
         config={"n_waves": N, "n_events": n, "components": 4,
                 "flops_per_event": cov_ampgen_flops(N)},
-        roof={"bound": "alu", "flops": float(cov_ampgen_flops(N)) * n},
+        roof={"bound": "hbm", "bytes": (72.0 + 32.0 * N) * n},
         dtype="f64", h2d=72 * n, d2h=32 * N * n, cpu_baseline=cpu_baseline,
         note="e2e passes host 3-momenta in (360 MB) and takes the amplitudes back (1.9 GB)")
 
@@ -945,12 +944,6 @@ def roofline(job, avg_s, peaks):
         if "flops" in job.roof:   # a contraction below the machine balance: tensor use for context
             tf = job.roof["flops"] / avg_s / 1e12
             roof.update({"tensor_achieved_tflops": tf, "tensor_frac": tf / peaks["bf16"]})
-    elif job.roof["bound"] == "alu":
-        achieved = job.roof["flops"] / avg_s / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": FP64_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_NOMINAL_TFLOPS, "algorithmic_flops_per_step": job.roof["flops"],
-                "peak_note": "nominal FP64 rate of the part (not measured); FP64 operations as "
-                             "counted per event in config.flops_per_event"}
     else:
         achieved = job.roof["flops"] / avg_s / 1e12
         roof = {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16"], "unit": "TFLOP/s",
@@ -958,7 +951,7 @@ def roofline(job, avg_s, peaks):
                 "peak_nominal": BF16_NOMINAL_TFLOPS, "frac_nominal": achieved / BF16_NOMINAL_TFLOPS,
                 "peak_note": "bf16 burst; the step time includes the small prep and final kernels"}
     roof.update({"traffic": TRAFFIC[job.name], "kernel": KERNELS[job.name],
-                 "peak_kind": "nominal" if job.roof["bound"] == "alu" else peaks["kind"]})
+                 "peak_kind": peaks["kind"]})
     return roof
 
 if __name__ == "__main__":
