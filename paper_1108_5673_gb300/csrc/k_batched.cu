@@ -90,8 +90,8 @@ constexpr int kHS = 32;         // parameter sets per half chunk (one block of R
 // Parameter sets per GEMM 1 / epilogue step: 32 (a half chunk), whose epilogue takes
 // all 16 warps; 16 for up to 16 sets, where two groups of eight warps take the tiles
 // in turn, each with accumulators of its own. 16 models of up to 1M events x 16
-// sets: 895 us a call with steps of 16, 936 with steps of 32 (half of whose products
-// and warps are padding then); 1M events x 32 waves x 256 sets 568 and 521 us.
+// sets: 895 us a call with steps of 16, 936 with steps of 32, half of whose products
+// and warps are padding then (632 now that a model's items share M V); 1M events x 32 waves x 256 sets 568 and 521 us.
 __host__ __device__ constexpr int step_sets(int K) { return K <= 16 ? 16 : 32; }
 constexpr int kXSMax = 6;       // X stages at most (as many as shared memory takes, at least 2)
 constexpr int kMaxSmem = 226 * 1024;

@@ -32,9 +32,9 @@
 // unit (seven warps per SM at 255 registers) 36% of the issue slots were used.
 // Twelve S warps and twelve gradient warps (72 registers) keep every sum's
 // order. Per call at 2M + 5M events x 20 waves, 4 free: 291 us (3.9 TB/s), 373
-// before; six and six warps 330, nine and six 315, fifteen and twelve 303 (these
-// with S warps that also waited for each other's tiles: 303). At 12 waves, 3 free
-// 214 (279), at 28 and 4, 1M + 2.5M events 255 (291). Splitting a
+// before; with S warps that also waited for each other's tiles 303, and then six and
+// six warps 330, nine and six 315, fifteen and twelve 303. At 12 waves, 3 free 214
+// (279), at 28 and 4, 1M + 2.5M events 255 (291). Splitting a
 // unit's waves over two warps in the S pass too changes the order of S's
 // remainders and with it the last digits of the gradients (3.6e-9).
 #include <numeric>
