@@ -78,6 +78,7 @@
 #include <cstring>
 #include <vector>
 
+#include "poll_limit.cuh"
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -469,8 +470,8 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
             const int c = ch / SPC;
             const int need = last ? g2_ready : ch % SPC == 0 ? c0 + c - 1 : 0;
             bool wx = !last && ch == 0, ws = !last && q >= NB;
-            unsigned long long t0 = 0;
-            for (unsigned it = 1;; ++it) {
+            PollLimit limit;
+            for (;;) {
                 if (g2 < g2_ready && test(&r_full, g2 & 1)) {
                     tc_fence_after();
                     const uint32_t xs = xbase + g2_s * kXBytes;
@@ -504,14 +505,10 @@ __device__ __forceinline__ void batched_body(const BatchArgs &a,
                     if (!wx && !ws)
                         break;
                 }
-                if ((it & 255) == 0) {
-                    const unsigned long long t = global_timer_ns();
-                    if (it == 256)
-                        t0 = t;
-                    if (__any_sync(0xffffffffu, t - t0 > kWaitLimitNs)) {
-                        ok = false;
-                        break;
-                    }
+                if (limit.due() &&
+                    __any_sync(0xffffffffu, limit.expired(global_timer_ns(), kWaitLimitNs))) {
+                    ok = false;
+                    break;
                 }
             }
             if (last || !ok)
