@@ -12,9 +12,11 @@
 // Exact digits. Each wave a gets one power of two 2^r_a > 2 max_j (|Re A_a| +
 // |Im A_a|) for the whole sample. Every float x of rows 2a, 2a+1 is written
 // as five fixed-point digits x = sum_{s=1..5} t_s + rest, t_s = c_s 2^(r_a -
-// 8s) with integers |c_s| <= 128 and |rest| <= 2^(r_a - 41): digit s is x's
-// remainder rounded to the nearest multiple of 2^(r_a - 8s) (by adding and
-// subtracting 1.5 2^(r_a - 8s + 23)), an exact float operation, and t_s has
+// 8s) with integers |c_s| <= 128 and |rest| <= 2^(r_a - 41). The kernel works on
+// x 2^-r_a (an exact product), so that every wave's digits lie at the same place
+// whatever its unit, and the sums get 2^(r_a + r_b) back in FP64 at the end. Digit s
+// is the remainder rounded to the nearest multiple of 2^-8s (by adding and
+// subtracting 1.5 2^(23 - 8s)), an exact float operation, and t_s has
 // at most 8 significant bits, so it is an exact BF16 value. Any x with |x| >=
 // 2^(r_a - 17) is a multiple of 2^(r_a - 40) and has rest = 0. A product of
 // digits s and t of rows p and q is c c' 2^(r_p + r_q - 8(s + t)): within one
@@ -185,17 +187,10 @@ __device__ __forceinline__ void two_sum2(f2 &hi, f2 &lo, f2 x)
 }
 
 // The scale of wave a's digits: r = floor(log2 amax) + 2 (so that every |x| <
-// 2^(r - 1)), clamped below at -35 (the quanta of the exact digit pairs stay
-// normal floats: r_p + r_q - 48 >= -118); a wave that is zero throughout gets
-// r = 0. Returns 1.5 2^(r + 15), the rounding constant of the first digit.
-__device__ __forceinline__ float first_digit_constant(float amax)
+// 2^(r - 1)); a wave that is zero throughout gets r = 0.
+__device__ __forceinline__ int wave_exponent(float amax)
 {
-    int r = 0;
-    if (amax > 0.f) {
-        const int ex = ((__float_as_int(amax) >> 23) & 0xff) - 127;  // subnormal: -127
-        r = max(ex + 2, -35);
-    }
-    return 1.5f * ldexpf(1.0f, r + 15);
+    return amax > 0.f ? ((__float_as_int(amax) >> 23) & 0xff) - 125 : 0;
 }
 
 // NW columns (this thread's half of a block) of its lane's row at `taddr`.
@@ -231,7 +226,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
     float *stages = reinterpret_cast<float *>(base + (size_t)NBUF * C::JBYTES);
     __shared__ uint64_t full[STAGES], empty[STAGES], jfull[NBUF], jempty[NBUF];
     __shared__ uint64_t accfull[2 * NACC], accempty[2 * NACC], g_done;
-    __shared__ float s_sig[R];
+    __shared__ float s_scale[R];   // 2^-r of the row's wave
     __shared__ uint32_t tmem_base;
     __shared__ int s_flags;
 
@@ -284,7 +279,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
     if (threadIdx.x < R) {
         const int w = threadIdx.x / 2;
         const int g = w < blocks.local() ? blocks.global(w) : n_waves;
-        s_sig[threadIdx.x] = g < n_waves ? first_digit_constant(amax[g]) : 1.5f * 32768.f;
+        s_scale[threadIdx.x] = g < n_waves ? __int_as_float((127 - wave_exponent(amax[g])) << 23) : 1.f;
     }
     if (warp == 1)
         tmem_alloc(&tmem_base, kNTmemCols);
@@ -530,16 +525,16 @@ __global__ void __launch_bounds__(kNThreads, 1)
                 const int rp = wg + it * C::WPG;
                 if (rp < NW) {
                     const int p = 2 * rp + half;
-                    const float sig = s_sig[p];
-                    const f2 S0 = pk2(sig, sig);
-                    f2 z0 = pk2(xs[it].x, xs[it].y), z1 = pk2(xs[it].z, xs[it].w);
+                    const float scale = s_scale[p], sig = 1.5f * 32768.f;
+                    const f2 S0 = pk2(sig, sig), SC = pk2(scale, scale);
+                    f2 z0 = mul2(pk2(xs[it].x, xs[it].y), SC), z1 = mul2(pk2(xs[it].z, xs[it].w), SC);
                     const uint32_t dst = jb + sw128(p, (uint32_t)l16 * 8);
                     float step = 1.0f;
 #pragma unroll
                     for (int d = 0; d < kNDigits; ++d) {
-                        // z rounded to a multiple of 2^(r - 8(d+1)): z + S - S with S =
-                        // S0 2^-8d (the products by powers of two are exact), and the
-                        // exact remainder
+                        // z rounded to a multiple of 2^-8(d+1): z + S - S with S = S0 2^-8d
+                        // (the products by powers of two are exact), and the exact
+                        // remainder
                         const f2 up = pk2(step, step), dn = pk2(-step, -step);
                         const f2 t0 = fma2(S0, dn, fma2(S0, up, z0));
                         const f2 t1 = fma2(S0, dn, fma2(S0, up, z1));
@@ -575,11 +570,12 @@ __global__ void __launch_bounds__(kNThreads, 1)
 
 // M from the CTAs' shares: one warp per (entry, part) of the launch's upper
 // triangle; lane k adds CTAs k, k + 32, ... (all loads issued first), then a
-// fixed shuffle tree; divided by N_gen, written to (a, b) and conjugated to
-// (b, a), the diagonal's imaginary part zero. With a timeout flagged, M is NaN.
+// fixed shuffle tree; scaled back by the two waves' 2^r, divided by N_gen, written
+// to (a, b) and conjugated to (b, a), the diagonal's imaginary part zero. With a
+// timeout flagged, M is NaN.
 __global__ void norm_tc_finalize(const double *__restrict__ part, int grid, int N,
-                                 NormBlocks blocks, double n_gen, const int *status,
-                                 double *__restrict__ M)
+                                 NormBlocks blocks, const float *__restrict__ amax, double n_gen,
+                                 const int *status, double *__restrict__ M)
 {
     const int ec = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int nl = blocks.local(), E = nl * (nl + 1) / 2;
@@ -607,7 +603,7 @@ __global__ void norm_tc_finalize(const double *__restrict__ part, int grid, int 
         v += x[k];
     v = warp_sum(v);
     if (lane == 0) {
-        double r = v / n_gen;
+        double r = ldexp(v, wave_exponent(amax[a]) + wave_exponent(amax[b])) / n_gen;
         if (*status & FLAG_TIMEOUT)
             r = NAN;
         if (a == b) {
@@ -639,7 +635,8 @@ cudaError_t norm_tc_nw(const CUtensorMap *map, const Planes &mc, const NormBlock
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     const int E2 = blocks.local() * (blocks.local() + 1);
-    norm_tc_finalize<<<(E2 + 7) / 8, 256, 0, s>>>(part, grid, mc.n_waves, blocks, n_gen, status, M);
+    norm_tc_finalize<<<(E2 + 7) / 8, 256, 0, s>>>(part, grid, mc.n_waves, blocks, amax, n_gen, status,
+                                                  M);
     return cudaGetLastError();
 }
 
@@ -676,9 +673,10 @@ int norm_tc_box_rows(int n_waves) { return 2 * norm_tc_block(n_waves); }
 
 bool norm_tc_scale_ok(float amax)
 {
-    // every kept quantum a normal float and every accumulator below 2^127:
-    // 2^r <= 2^55, i.e. amax < 2^53 (and finite)
-    return amax >= 0.f && amax < 0x1p53f;
+    // above, the FP64 kernel, whose error is the smaller one (the digits would serve up
+    // to 2^125: beyond, and below 2^-124, 2^-r is no normal float); far below, where
+    // amplitudes become subnormal, their own last bits limit the digits
+    return amax == 0.f || (amax >= 0x1p-100f && amax < 0x1p53f);
 }
 
 size_t norm_tc_partials_doubles(int n_waves, int grid)
