@@ -495,6 +495,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
         // A half warp holds one row of the tile (four events a lane); warp w of
         // the group takes row pairs w, w + WPG, ...
         const int cw = warp - kNFirstCons, g = cw / C::WPG, wg = cw % C::WPG;
+        const unsigned zero = (unsigned)blocks.n_box >> 4;  // what the compiler does not know
         const int half = lane >> 4, l16 = lane & 15;
         for (int j = g; j < n_my; j += C::GROUPS) {
             const int st = j % STAGES, b = j % NBUF, k = j / NBUF;
@@ -504,16 +505,24 @@ __global__ void __launch_bounds__(kNThreads, 1)
             }
             const float *T = stages + (size_t)st * (C::STAGE_BYTES / 4) + 4 * l16;
             float4 xs[C::ITERS];
+            unsigned seen = 0;
 #pragma unroll
             for (int it = 0; it < C::ITERS; ++it) {
                 const int rp = wg + it * C::WPG;
-                if (rp < NW)
+                if (rp < NW) {
                     xs[it] = *reinterpret_cast<const float4 *>(T + (2 * rp + half) * kNTE);
+                    seen |= __float_as_uint(xs[it].x);
+                }
             }
-            // the amplitudes are in registers: the stage may be refilled
+            // Once the amplitudes are in registers the stage may be refilled. The
+            // arrival's address depends on every load's result: loads that were only issued
+            // can be overtaken by it, since the products' operand reads, which can fill shared
+            // memory's bandwidth, hold them up for longer than a refill takes (single rows of a
+            // tile then came from the tile after: seen with three products of 128 columns
+            // a step).
             __syncwarp();
             if (lane == 0)
-                mbar_arrive(&empty[st]);
+                mbar_arrive(empty + st + (seen & zero));
             // the buffer is free once the products of its previous tile are done
             if (k > 0 && !mbar_wait(&jempty[b], (uint32_t)(k - 1) & 1)) {
                 flags |= FLAG_TIMEOUT;
