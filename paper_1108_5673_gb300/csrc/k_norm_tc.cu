@@ -24,25 +24,36 @@
 // multiples of one quantum and at most 2^14 of it, so the tensor cores' FP32
 // sum over 1024 events (at most 2^24 quanta) is exact.
 //
-// Digit blocks D_st[p][q] = sum_j t_s(p, j) t_t(q, j), R rows each, from at
-// most two MMAs per tile on the same digits in shared memory. The first takes
-// as many digits as fit M = 128 rows (S1 = 5 up to 12 waves, 3 up to 20, 2 up
-// to 32) against all five; the second the next two digits against the rest
-// (none, [X4; X5] against X4, [X3; X4] against [X3; X4; X5]). An M = 128 MMA
-// reads its 128 A rows whatever the number of columns, which is what a small
-// model's tile costs, hence one MMA where everything fits. With D_ts =
-// D_st^T these are all pairs (all but (5,5) beyond 12 waves), all exact,
-// drained every 1024 events:
+// Digit blocks D_st[p][q] = sum_j t_s(p, j) t_t(q, j), R rows each, from MMAs on
+// the same digits in shared memory. Up to 20 waves: one or two per tile, the first
+// with as many digits as fit M = 128 rows (S1 = 5 up to 12 waves, 3 up to 20) against
+// all five, the second [X4; X5] against X4. An M = 128 MMA reads its 128 A rows
+// whatever the number of columns, which is what a small model's tile costs, hence
+// one MMA where everything fits. With D_ts = D_st^T these are all pairs (all but
+// (5,5) beyond 12 waves), all exact, drained every 1024 events:
 //   G = T + U + U^T, T the products whose transposes are among them too (a
 //   symmetric sum), U the others,
 // so that one sum W = T/2 + U per (row, column) serves, G = W + W^T: float-
-// float for the first MMA's blocks, plain FP32 for the second's, which are
-// below 2^-32 of the leading one. Per event and real entry of G the error is
+// float for the first accumulator's blocks, plain FP32 for the second's, which are
+// below 2^-28 of the leading one. Per event and real entry of G the error is
 // at most 2^-41 (|x_p| 2^r_q [|x_q| < 2^(r_q - 17)] + |x_q| 2^r_p [|x_p| <
 // 2^(r_p - 17)]) + 2^(r_p + r_q - 61), with unbiased signs apart from the last
-// term. Measured against an exact Gram matrix (inputs on a 2^-22 grid): 0.6-
-// 1.5e-16 of M at 4-48 waves, 1-10M events; FP64 sums of the exact products
-// give 4-5e-16.
+// term.
+//
+// Beyond 20 waves, where M used to come from exact FP64 products, the rest is kept
+// too: Z = rest rounded to BF16 (a float: 8 bits of its own, whatever its size) is a
+// sixth row block, and the MMAs are [X1; X2] against [X1; X2; X3; X4] into the first
+// accumulator, [X1; X2] and [X3; X4] against [X5; Z] and [X3; X4] against [X3; X4]
+// into the second: every pair but (5,5), (5,Z) and (Z,Z). (The second's sums are
+// FP32 sums, no longer all exact: (1,5) and the products with Z are at most 2^-28 of
+// G.) The error above shrinks by 2^-9.
+//
+// Largest error of M relative to sqrt(M_aa M_bb), against double-double sums, for
+// uniform m and the harmonics and widths of the benchmark's waves (0.05 to 0.4 GeV),
+// 50k / 200k / 1M events: 20 waves 3e-14 / 2e-14 / 7e-15; 21 and more 2.7e-16 / 3e-16 /
+// 7e-16 (without Z 5e-14 / 3e-14 / 1e-14), FP64 sums of the exact products 1.5e-15 /
+// 1.4e-15 / 1.4e-15. Where a wave's largest amplitude is so far above its rms that this
+// would not hold (norm_tc_spread_ok), M is built again by the FP64 kernel.
 //
 // More than 32 waves: the accumulators no longer fit tensor memory, so the
 // waves are cut into three blocks and three launches take two blocks each
@@ -58,22 +69,26 @@
 // issues the MMAs (kind::f16, K = 16, four steps per tile); eight drain warps
 // (two per lane quarter, half of each block's columns) add the accumulators
 // into W. Up to 20 waves two accumulator sets alternate; beyond, one set, whose
-// two MMAs hand over separately, so that the first MMA of the next period
+// two accumulators hand over separately, so that the first MMA of the next period
 // runs while the second accumulator is drained. The CTA's share of M goes to
 // global memory with the CTA index innermost; norm_tc_finalize adds the CTAs
 // in a fixed order, divides by N_gen and fills the Hermitian matrix.
 //
 // Bound: the digit split (30 packed FP32 operations per two rows and four
-// events, on six warps) and the MMAs, about 1300 and 1024 cycles per tile at
+// events, on six warps) and the MMAs, about 1300 and 1280 cycles per tile at
 // 32 waves, overlapping in part; at few waves the fixed cost of a tile, ~600 cycles
 // (a copy 430, a step of the issuer). Producer and issuer run as converged warps
 // with one elected lane issuing, so that their addresses and descriptors stay in
 // uniform registers: as single lanes they took 5M x 4 from 183 to 207 us a call, 5M
-// x 16 from 305 to 340, 10M x 12 from 381 to 404, 5M x 20 from 334 to 352. Per call
-// of pwa_build_norm: 10M x 32 in 0.92 ms (2.8 TB/s of amplitudes), 5M x 20 in 0.33
-// ms, 10M x 12 in 0.38 ms, 4M x 48 in 1.16 ms; before, with one-warp consumers per
-// tile, 0.49 ms at 5M x 20 and 0.63 at 10M x 12, and on the FP64 pipe beyond 20
-// waves 81 ms at 10M x 32 and 69 ms at 4M x 48.
+// x 16 from 305 to 340, 10M x 12 from 381 to 404. Waiting for the loads before a stage
+// is released took 5M x 20 from 339 to 349. Per call of pwa_build_norm: 10M x 32 in
+// 0.99 ms (2.6 TB/s of amplitudes), 5M x 24 0.45, 5M x 20 0.35, 10M x 12 0.38, 4M x 48
+// 1.24; without Z 0.92, 0.39 and 1.15 at 32, 24 and 48 waves; on the FP64 pipe beyond 20
+// waves 81 ms at 10M x 32 and 69 ms at 4M x 48. Digit buffers and stages: with Z at 32
+// waves four buffers leave two stages; two buffers and eight stages 1.19 ms, three
+// two-warp groups with a buffer and a stage each 1.03, one group of six warps 1.03.
+#include <string.h>
+
 #include "pwa_internal.cuh"
 
 namespace pwa {
@@ -100,12 +115,16 @@ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 template <int NW>
 struct NormTcCfg {
     static constexpr int R = 2 * NW;                         // real rows (padded waves)
-    // digits in the first MMA's A operand; the second MMA takes digits S1 + 1
-    // and S1 + 2 against B2 digits from S1 + 1 on (none when S1 = 5)
+    // digits in the first MMA's A operand; B1 digits in its B operand; column
+    // blocks of the second accumulator (see the header); row blocks of a buffer
     static constexpr int S1 = NW <= 12 ? 5 : NW <= 20 ? 3 : 2;
-    static constexpr int B2 = S1 == 5 ? 0 : S1 == 3 ? 1 : 3;
-    static constexpr int N1 = round_up16(kNDigits * R);      // columns of the first MMA: digits 1-5
+    static constexpr bool REST = S1 == 2;                    // the rest of x as a sixth digit
+    static constexpr int B1 = REST ? 4 : kNDigits;
+    static constexpr int B2 = S1 == 5 ? 0 : S1 == 3 ? 1 : 4;
+    static constexpr int ROWBLOCKS = REST ? kNDigits + 1 : kNDigits;
+    static constexpr int N1 = round_up16(B1 * R);            // columns of the first accumulator
     static constexpr int N2 = round_up16(B2 * R);            // of the second
+    static constexpr int NI2 = REST ? 2 * R : N2;            // one instruction's columns in it
     static constexpr int NI1 = N1 > 256 ? N1 / 2 : N1;       // one instruction's columns
     static constexpr int WPG = NW <= 8 ? 1 : NW <= 12 ? 2 : 3;  // warps per consumer group
     static constexpr int GROUPS = kNCons / WPG;
@@ -115,7 +134,7 @@ struct NormTcCfg {
     // buffer rows: the digits, the B operands' padding, and the 128 rows that
     // each A operand reads
     static constexpr int BUFROWS =
-        cmax(cmax(N1, 128), B2 ? cmax(S1 * R + N2, S1 * R + 128) : 0);
+        REST ? ROWBLOCKS * R : cmax(cmax(N1, 128), B2 ? cmax(S1 * R + N2, S1 * R + 128) : 0);
     static constexpr uint32_t JBYTES = BUFROWS * 128;        // one 64-event K-atom of every row
     static constexpr uint32_t STAGE_BYTES = R * kNTE * 4;
     static constexpr int STAGES =
@@ -124,7 +143,9 @@ struct NormTcCfg {
     // the CTA's sums W[S1 R][R] as doubles reuse the digit buffers
     static constexpr size_t SUMS_BYTES = (size_t)S1 * R * R * sizeof(double);
     static_assert(S1 * R <= 128, "S1 digits of every row fit M = 128");
-    static_assert(NI1 % 16 == 0 && NI1 <= 256 && N2 <= 256 && N1 % NI1 == 0, "N of the MMA");
+    static_assert(NI1 % 16 == 0 && NI1 <= 256 && NI2 % 16 == 0 && NI2 <= 256 && N1 % NI1 == 0,
+                  "N of the MMA");
+    static_assert(!REST || BUFROWS >= S1 * R + 128, "rows of the second A operand");
     static_assert(NACC * (N1 + N2) <= (int)kNTmemCols, "tensor memory");
     static_assert(NW % 4 == 0, "drain in 4-column steps, 8-row swizzle atoms per digit");
     // Stages and buffers belong to one group each: a group's parity wait on
@@ -188,9 +209,11 @@ __device__ __forceinline__ void two_sum2(f2 &hi, f2 &lo, f2 x)
 
 // The scale of wave a's digits: r = floor(log2 amax) + 2 (so that every |x| <
 // 2^(r - 1)); a wave that is zero throughout gets r = 0.
-__device__ __forceinline__ int wave_exponent(float amax)
+__host__ __device__ __forceinline__ int wave_exponent(float amax)
 {
-    return amax > 0.f ? ((__float_as_int(amax) >> 23) & 0xff) - 125 : 0;
+    int bits;
+    memcpy(&bits, &amax, sizeof bits);
+    return amax > 0.f ? ((bits >> 23) & 0xff) - 125 : 0;
 }
 
 // NW columns (this thread's half of a block) of its lane's row at `taddr`.
@@ -274,7 +297,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
         for (int i = in_rows * kNTE + threadIdx.x; i < R * kNTE; i += blockDim.x)
             stages[(size_t)s * (C::STAGE_BYTES / 4) + i] = 0.f;
     for (int b = 0; b < NBUF; ++b)
-        for (uint32_t i = kNDigits * R * 32 + threadIdx.x; i < C::JBYTES / 4; i += blockDim.x)
+        for (uint32_t i = C::ROWBLOCKS * R * 32 + threadIdx.x; i < C::JBYTES / 4; i += blockDim.x)
             reinterpret_cast<uint32_t *>(base + (size_t)b * C::JBYTES)[i] = 0u;
     if (threadIdx.x < R) {
         const int w = threadIdx.x / 2;
@@ -311,7 +334,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
         // ---- MMA issuer: as the producer -----------------------------------
         const bool lead = elect_one();
         const uint32_t id1 = umma_idesc_bf16(128, C::NI1, 0, 0);
-        const uint32_t id2 = umma_idesc_bf16(128, C::N2, 0, 0);
+        const uint32_t id2 = umma_idesc_bf16(128, C::NI2, 0, 0);
         const uint64_t dK = umma_desc_sw128(0, 16, 1024);
         const uint32_t row2 = (uint32_t)(S1 * R) * 128u;  // byte offset of digit S1 + 1's rows
         bool ok = true;
@@ -357,7 +380,15 @@ __global__ void __launch_bounds__(kNThreads, 1)
 #pragma unroll
                     for (int ks = 0; ks < kNTE / 16; ++ks) {
                         const uint32_t a = jb + row2 + (uint32_t)ks * 32;
-                        umma_bf16(acc2, dK + (a >> 4), dK + (a >> 4), id2, (first && ks == 0) ? 0u : 1u);
+                        const uint32_t acc = (first && ks == 0) ? 0u : 1u;
+                        if constexpr (C::REST) {
+                            const uint32_t a1 = jb + (uint32_t)ks * 32, b5 = a1 + (uint32_t)(4 * R) * 128u;
+                            umma_bf16(acc2, dK + (a1 >> 4), dK + (b5 >> 4), id2, acc);
+                            umma_bf16(acc2, dK + (a >> 4), dK + (b5 >> 4), id2, 1u);
+                            umma_bf16(acc2 + (uint32_t)C::NI2, dK + (a >> 4), dK + (a >> 4), id2, acc);
+                        } else {
+                            umma_bf16(acc2, dK + (a >> 4), dK + (a >> 4), id2, acc);
+                        }
                     }
                 }
                 __syncwarp();
@@ -383,7 +414,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
         // Row m holds row p = m % R of digit m / R of each MMA's A operand;
         // block t of an accumulator is columns t R ... of it. Blocks whose
         // transpose is among the products too count half (T/2): t < S1 of the
-        // first MMA, the A digits' own of the second.
+        // first, the A digits' own of the second (its last two when there are four).
         const int q = warp & 3, h = (warp - kNFirstDrain) >> 2, m = q * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
         constexpr int HC = NW / 2;  // packed column pairs per thread and block (NW columns)
@@ -392,8 +423,8 @@ __global__ void __launch_bounds__(kNThreads, 1)
         // B2 = 1: D_44 counts half, D_54 (rows of the second A digit) in full
         const float w54 = m < R ? 0.5f : 1.0f;
         const f2 W54 = pk2(w54, w54);
-        // (wh, wl): the first MMA's blocks; w2: the second's, below 2^-32 of the
-        // leading one (2^-48 for B2 = 1), whose FP32 roundings are below 2^-56.
+        // (wh, wl): the first accumulator's blocks; w2: the second's, below 2^-28 of the
+        // leading one (2^-48 for B2 = 1), whose FP32 roundings are below 2^-52 of it.
         // Added to (wh, wl) they would fall below its last bit, one-sidedly.
         f2 wh[HC], wl[HC], w2[C::B2 > 0 ? HC : 1];
 #pragma unroll
@@ -416,7 +447,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
                 tc_fence_after();
                 const uint32_t acc = tmem + lane_addr + (uint32_t)set * (C::N1 + C::N2) +
                                      (half ? (uint32_t)C::N1 : 0u) + (uint32_t)(h * NW);
-                const int n_blocks = half ? C::B2 : kNDigits;
+                const int n_blocks = half ? C::B2 : C::B1;
 #pragma unroll
                 for (int t = 0; t < n_blocks; ++t) {
 #pragma unroll
@@ -440,7 +471,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
                             else if (C::B2 == 1)
                                 w2[c] = fma2(x, W54, w2[c]);
                             else
-                                w2[c] = t < 2 ? fma2(x, HALF, w2[c]) : add2(w2[c], x);
+                                w2[c] = t < 2 ? add2(w2[c], x) : fma2(x, HALF, w2[c]);
                         }
                     }
                 }
@@ -555,6 +586,13 @@ __global__ void __launch_bounds__(kNThreads, 1)
                         st_shared_v2(dst + (uint32_t)(d * R) * 128u, to_bf16x2(a0, a1),
                                      to_bf16x2(a2, a3));
                         step *= 0x1p-8f;
+                    }
+                    if constexpr (C::REST) {  // what is left, to 8 bits of its own
+                        float a0, a1, a2, a3;
+                        upk2(z0, a0, a1);
+                        upk2(z1, a2, a3);
+                        st_shared_v2(dst + (uint32_t)(kNDigits * R) * 128u, to_bf16x2(a0, a1),
+                                     to_bf16x2(a2, a3));
                     }
                 }
             }
@@ -686,6 +724,21 @@ bool norm_tc_scale_ok(float amax)
     // to 2^125: beyond, and below 2^-124, 2^-r is no normal float); far below, where
     // amplitudes become subnormal, their own last bits limit the digits
     return amax == 0.f || (amax >= 0x1p-100f && amax < 0x1p53f);
+}
+
+bool norm_tc_checks_spread(int n_waves) { return n_waves > 20; }
+
+bool norm_tc_spread_ok(int n_waves, const float *amax, int64_t n, double n_gen, const double *diag)
+{
+    // Beyond 20 waves the standard is the FP64 kernel's error. The dropped squares of
+    // the fifth digits add up to k^2 2^-67.6 of M_aa, k = 2^r_a / rms of the wave: k is
+    // at most 47 for widths of 0.05 GeV (error 3e-16 measured), 120 for 0.01 GeV
+    // (2e-15; FP64 1e-15), 900 for 1e-4 GeV (5e-14).
+    for (int a = 0; a < n_waves; ++a)
+        if (amax[a] > 0.f &&
+            !(ldexp((double)n / n_gen, 2 * wave_exponent(amax[a])) <= 0x1p14 * diag[a]))
+            return false;
+    return true;
 }
 
 size_t norm_tc_partials_doubles(int n_waves, int grid)

@@ -1660,6 +1660,58 @@ int pwa_load_events_incoherent(pwa_ctx *c, int n_lambda, const void *data_amp, i
                            });
 }
 
+static int build_norm_tc(pwa_ctx *c)
+{
+    CUtensorMap map;
+    CK(c, encode_planes_map(&map, c->mc.ptr, c->mc.n, c->mc.pitch, 2 * c->N,
+                            norm_tc_box_events(), norm_tc_box_rows(c->N)));
+    const int grid = c->num_sms;
+    const size_t nd = norm_tc_partials_doubles(c->N, grid);
+    double *scratch = nullptr;
+    int rc = dev_alloc(c, (void **)&scratch, (nd + 1) * sizeof(double), "norm scratch");
+    if (rc)
+        return rc;
+    int *dstat = reinterpret_cast<int *>(scratch + nd);
+    int flags = 0;
+    cudaError_t e = cudaMemsetAsync(dstat, 0, sizeof(int), c->stream);
+    if (e == cudaSuccess)
+        e = launch_build_norm_tc(&map, c->mc, c->mc_amax, c->n_gen, scratch, grid, dstat, c->M,
+                                 c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&flags, dstat, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess)
+        quiet(c);
+    dev_free(scratch);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
+    }
+    if (flags & FLAG_TIMEOUT)
+        return fail(c, PWA_ETIMEOUT, "build_norm: a device-side wait timed out");
+    return PWA_OK;
+}
+
+static int build_norm_fp64(pwa_ctx *c)
+{
+    double *scratch = nullptr;
+    int rc = dev_alloc(c, (void **)&scratch, norm_scratch_bytes(c->N, c->num_sms), "norm scratch");
+    if (rc)
+        return rc;
+    cudaError_t e = launch_build_norm(c->mc, c->n_gen, c->M, scratch, c->num_sms, c->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess)
+        quiet(c);
+    dev_free(scratch);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
+    }
+    return PWA_OK;
+}
+
 int pwa_build_norm(pwa_ctx *c, double *M_out)
 {
     if (!c)
@@ -1673,60 +1725,37 @@ int pwa_build_norm(pwa_ctx *c, double *M_out)
     if (const char *v = getenv("PWA_NORM_KERNEL"))
         if (strcmp(v, "fp64") == 0)
             tc = false;
+    const int N = c->N;
+    const size_t m_bytes = (size_t)2 * N * N * sizeof(double);
+    bool copied = false;
+    float am[kMaxWaves];
     if (tc) {
-        std::vector<float> am(c->N);
-        CK(c, cudaMemcpy(am.data(), c->mc_amax, c->N * sizeof(float), cudaMemcpyDeviceToHost));
-        for (float x : am)
-            tc = tc && norm_tc_scale_ok(x);
+        CK(c, cudaMemcpy(am, c->mc_amax, N * sizeof(float), cudaMemcpyDeviceToHost));
+        for (int a = 0; a < N; ++a)
+            tc = tc && norm_tc_scale_ok(am[a]);
     }
     if (tc) {
-        CUtensorMap map;
-        CK(c, encode_planes_map(&map, c->mc.ptr, c->mc.n, c->mc.pitch, 2 * c->N,
-                                norm_tc_box_events(), norm_tc_box_rows(c->N)));
-        const int grid = c->num_sms;
-        const size_t nd = norm_tc_partials_doubles(c->N, grid);
-        double *scratch = nullptr;
-        int rc = dev_alloc(c, (void **)&scratch, (nd + 1) * sizeof(double), "norm scratch");
-        if (rc)
+        if (int rc = build_norm_tc(c))
             return rc;
-        int *dstat = reinterpret_cast<int *>(scratch + nd);
-        int flags = 0;
-        cudaError_t e = cudaMemsetAsync(dstat, 0, sizeof(int), c->stream);
-        if (e == cudaSuccess)
-            e = launch_build_norm_tc(&map, c->mc, c->mc_amax, c->n_gen, scratch, grid, dstat, c->M,
-                                     c->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&flags, dstat, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess)
-            quiet(c);
-        dev_free(scratch);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
-        }
-        if (flags & FLAG_TIMEOUT)
-            return fail(c, PWA_ETIMEOUT, "build_norm: a device-side wait timed out");
-    } else {
-        double *scratch = nullptr;
-        int rc = dev_alloc(c, (void **)&scratch, norm_scratch_bytes(c->N, c->num_sms), "norm scratch");
-        if (rc)
-            return rc;
-        cudaError_t e = launch_build_norm(c->mc, c->n_gen, c->M, scratch, c->num_sms, c->stream);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess)
-            quiet(c);
-        dev_free(scratch);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(c, PWA_ECUDA, "build_norm: %s", cudaGetErrorString(e));
+        if (norm_tc_checks_spread(N)) {
+            double diag[kMaxWaves];  // the real parts of M_aa
+            if (M_out) {
+                CK(c, cudaMemcpy(M_out, c->M, m_bytes, cudaMemcpyDeviceToHost));
+                for (int a = 0; a < N; ++a)
+                    diag[a] = M_out[2 * ((size_t)a * N + a)];
+            } else {
+                CK(c, cudaMemcpy2D(diag, sizeof(double), c->M, 2 * (N + 1) * sizeof(double),
+                                   sizeof(double), N, cudaMemcpyDeviceToHost));
+            }
+            tc = norm_tc_spread_ok(N, am, c->mc.n, c->n_gen, diag);
+            copied = tc && M_out;
         }
     }
-    if (M_out)
-        CK(c, cudaMemcpy(M_out, c->M, (size_t)2 * c->N * c->N * sizeof(double),
-                         cudaMemcpyDeviceToHost));
+    if (!tc)
+        if (int rc = build_norm_fp64(c))
+            return rc;
+    if (M_out && !copied)
+        CK(c, cudaMemcpy(M_out, c->M, m_bytes, cudaMemcpyDeviceToHost));
     c->has_norm = true;
     return PWA_OK;
 }

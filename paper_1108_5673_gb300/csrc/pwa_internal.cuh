@@ -666,6 +666,11 @@ bool norm_tc_available(int n_waves);
 int norm_tc_box_events();
 int norm_tc_box_rows(int n_waves);
 bool norm_tc_scale_ok(float amax);
+// Where the FP64 kernel's accuracy is the standard, norm_tc_checks_spread(n_waves):
+// whether M as built from n events has it, by the amplitudes' spread (amax [N], diag
+// [N] = M_aa: host copies).
+bool norm_tc_checks_spread(int n_waves);
+bool norm_tc_spread_ok(int n_waves, const float *amax, int64_t n, double n_gen, const double *diag);
 size_t norm_tc_partials_doubles(int n_waves, int grid);
 cudaError_t launch_build_norm_tc(const CUtensorMap *map, const Planes &mc, const float *amax,
                                  double n_gen, double *partials, int grid, int *status, double *M,
