@@ -1147,8 +1147,17 @@ int pwa_create(pwa_ctx **out, int device, const pwa_config *cfg)
     c->work_bytes = nwork * sizeof(double);
     if ((rc = dev_alloc(c, (void **)&c->d_work, nwork * sizeof(double), "work")))
         return bail(rc);
-    if (cudaMemset(c->d_work, 0, nwork * sizeof(double)) != cudaSuccess)
-        return bail(fail(c, PWA_ECUDA, "memset"));
+    // Cleared on the context's own stream, ahead of everything the context does: a
+    // clear on the default stream waits for whatever others have queued there, and with
+    // kept memory no allocation in between waits for it. (A caller's stream that is being
+    // captured is refused: the clear would go into the graph.)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess ||
+        capture != cudaStreamCaptureStatusNone ||
+        cudaMemsetAsync(c->d_work, 0, nwork * sizeof(double), c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return bail(fail(c, PWA_ECUDA, "clearing the work area"));
+    }
     c->ticket = reinterpret_cast<unsigned *>(c->d_work + nwork - 4);
     c->async_status = reinterpret_cast<int *>(c->d_work + nwork - 2);
     c->zc_status = reinterpret_cast<int *>(c->d_work + nwork - 6);
