@@ -1356,6 +1356,34 @@ static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_
     return PWA_OK;
 }
 
+// Where the generators write the caller's amplitudes: the buffer itself if it is on
+// the device and takes whole complex numbers (the kernels store them 8 bytes at a
+// time), else one of their size.
+static int amplitude_buffer(pwa_ctx *c, void *out, size_t bytes, float **d)
+{
+    *d = static_cast<float *>(out);
+    if (is_device_pointer(out) && reinterpret_cast<uintptr_t>(out) % 8 == 0)
+        return PWA_OK;
+    return dev_alloc(c, (void **)d, bytes, "amplitudes");
+}
+
+// Ends a call that generated into amplitude_buffer's buffer with status rc.
+static int amplitude_result(pwa_ctx *c, int rc, void *out, size_t bytes, float *d)
+{
+    if (d == out)
+        return rc;
+    cudaError_t e = cudaSuccess;
+    if (!rc)
+        e = cudaMemcpyAsync(out, d, bytes, cudaMemcpyDefault, c->stream);
+    const cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    dev_free(d);
+    if (!rc && (e != cudaSuccess || e2 != cudaSuccess)) {
+        cudaGetLastError();
+        rc = fail(c, PWA_ECUDA, "amplitude copy: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
+    }
+    return rc;
+}
+
 int pwa_compute_amplitudes(pwa_ctx *c, const pwa_wave *waves, const double *kin, int64_t n,
                            void *out)
 {
@@ -1370,20 +1398,12 @@ int pwa_compute_amplitudes(pwa_ctx *c, const pwa_wave *waves, const double *kin,
     int rc = check_waves(c, waves, &table);
     if (rc)
         return rc;
-    const bool on_dev = is_device_pointer(out);
-    float *dout = static_cast<float *>(out);
-    if (!on_dev)
-        rc = dev_alloc(c, (void **)&dout, (size_t)n * c->N * 8, "amplitudes");
-    if (!rc)
-        rc = generate(c, table, kin, n, dout, false, 0);
-    if (!rc && !on_dev) {
-        cudaError_t e = cudaMemcpy(out, dout, (size_t)n * c->N * 8, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess)
-            rc = fail(c, PWA_ECUDA, "amplitude copy: %s", cudaGetErrorString(e));
-    }
-    if (!on_dev)
-        dev_free(dout);
-    return rc;
+    const size_t bytes = (size_t)n * c->N * 8;
+    float *dout = nullptr;
+    if ((rc = amplitude_buffer(c, out, bytes, &dout)))
+        return rc;
+    rc = generate(c, table, kin, n, dout, false, 0);
+    return amplitude_result(c, rc, out, bytes, dout);
 }
 
 int pwa_load_events_generated(pwa_ctx *c, const pwa_wave *waves, const double *data_kin,
@@ -1502,20 +1522,11 @@ int pwa_compute_covariant_amplitudes(pwa_ctx *c, const pwa_cov_wave *waves, cons
     if (rc)
         return rc;
     const size_t bytes = (size_t)n * 4 * c->N * 8;
-    const bool on_dev = is_device_pointer(out);
-    float *dout = static_cast<float *>(out);
-    if (!on_dev)
-        rc = dev_alloc(c, (void **)&dout, bytes, "amplitudes");
-    if (!rc)
-        rc = generate_cov(c, table, p3, n, dout, kCovEventMajor, 0, nullptr);
-    if (!rc && !on_dev) {
-        cudaError_t e = cudaMemcpy(out, dout, bytes, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess)
-            rc = fail(c, PWA_ECUDA, "amplitude copy: %s", cudaGetErrorString(e));
-    }
-    if (!on_dev)
-        dev_free(dout);
-    return rc;
+    float *dout = nullptr;
+    if ((rc = amplitude_buffer(c, out, bytes, &dout)))
+        return rc;
+    rc = generate_cov(c, table, p3, n, dout, kCovEventMajor, 0, nullptr);
+    return amplitude_result(c, rc, out, bytes, dout);
 }
 
 }  // extern "C"
