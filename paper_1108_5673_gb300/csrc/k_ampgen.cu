@@ -268,6 +268,10 @@ __global__ void __launch_bounds__(kGenThreads, 4)
                 Ei = ff_dot(D, ei, G, er);
             }
             const ff f = ff_mul(y, inv);
+            // below 2^-100 f's low part has lost bits, which the product with a large E shows
+            // in the result (in keV, MeV^2 and the like: 1 / (D^2 + G^2) is tiny there)
+            float f0, f1;
+            upk2(abs2(f.h), f0, f1);
             const ff re = ff_mul(Er, f), im = ff_mul(Ei, f);
             // error bound: y's, and D's rounding (2^-46 of M^2 + m^2, times |BW|)
             const f2 b = mul2(add2(abs2(D.h), abs2(G.h)), inv.h);
@@ -295,7 +299,8 @@ __global__ void __launch_bounds__(kGenThreads, 4)
             }
             // amplitudes in doubt wait for a warp's worth of them: FP64
             // instructions cost the same for one lane as for 32
-            const bool d0 = !(r0 && j0 && y0) && in0, d1 = !(r1 && j1 && y1) && in1;
+            const bool d0 = !(r0 && j0 && y0 && f0 >= 0x1p-100f) && in0,
+                       d1 = !(r1 && j1 && y1 && f1 >= 0x1p-100f) && in1;
             if (__any_sync(0xffffffffu, d0 || d1)) {
                 const unsigned below = (1u << lane) - 1;
                 unsigned doubt = __ballot_sync(0xffffffffu, d0);
