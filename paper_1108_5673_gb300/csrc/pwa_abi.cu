@@ -149,7 +149,8 @@ int dev_alloc(pwa_ctx *ctx, void **p, size_t bytes, const char *what)
 }
 
 // Whether the last wait of this thread before returning memory succeeded: it is
-// kept for another context only then (else cudaFree and the like decide).
+// kept for another context only then (else cudaFree and the like decide). Every
+// dev_free of memory that was in use follows a quiet() or a settle().
 thread_local bool t_quiet = true;
 
 // Before the memory of a context is returned: the work that may use it has
@@ -162,6 +163,17 @@ void quiet(pwa_ctx *c)
               (!c->captured || cudaDeviceSynchronize() == cudaSuccess);
     if (!t_quiet)
         cudaGetLastError();
+}
+
+// The wait for work that was enqueued on the context's stream with memory of the
+// call's own, before that is returned: the same rule.
+cudaError_t settle(pwa_ctx *c)
+{
+    const cudaError_t e = cudaStreamSynchronize(c->stream);
+    t_quiet = e == cudaSuccess;
+    if (!t_quiet)
+        cudaGetLastError();
+    return e;
 }
 
 // Notes that the context's work is being captured by the caller.
@@ -304,13 +316,13 @@ int pack_rows(pwa_ctx *c, const void *src, int64_t n, int dtype, int nw, float *
             e = launch_pack(staging, dtype, m, nw, dst + s, pitch, amax, n_max, c->num_sms,
                             c->stream);
         if (e != cudaSuccess) {
-            cudaStreamSynchronize(c->stream);
+            settle(c);
             dev_free(staging);
             cudaGetLastError();
             return fail(c, PWA_ECUDA, "loading amplitudes: %s", cudaGetErrorString(e));
         }
     }
-    cudaError_t e = cudaStreamSynchronize(c->stream);
+    const cudaError_t e = settle(c);
     dev_free(staging);
     if (e != cudaSuccess)
         return fail(c, PWA_ECUDA, "loading amplitudes: %s", cudaGetErrorString(e));
@@ -364,7 +376,7 @@ int load_floats(pwa_ctx *c, const double *src, int64_t n, float *dst)
         if (e == cudaSuccess)
             e = launch_to_float(staging, m, dst + s, c->stream);
     }
-    const cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    const cudaError_t e2 = settle(c);
     dev_free(staging);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         cudaGetLastError();
@@ -1016,6 +1028,8 @@ int pwa_mc_weights(pwa_ctx *c, const double *V, float *w)
     float *dw = w;
     if (!on_dev) {
         if (c->w_len < c->n_mc) {
+            if (c->d_w)
+                quiet(c);
             dev_free(c->d_w);
             c->w_len = 0;
             if ((rc = dev_alloc(c, (void **)&c->d_w, (size_t)c->n_mc * sizeof(float), "weights")))
@@ -1336,7 +1350,7 @@ static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_
         cudaError_t e = cudaMemcpyAsync(staging, kin, (size_t)n * 3 * sizeof(double),
                                         cudaMemcpyHostToDevice, c->stream);
         if (e != cudaSuccess) {
-            cudaStreamSynchronize(c->stream);
+            settle(c);
             dev_free(staging);
             return fail(c, PWA_ECUDA, "kinematics copy: %s", cudaGetErrorString(e));
         }
@@ -1345,7 +1359,7 @@ static int generate(pwa_ctx *c, const GenTable &table, const double *kin, int64_
     const char *kv = getenv("PWA_AMPGEN_KERNEL");
     cudaError_t e = launch_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, soa,
                                    pitch, c->num_sms, c->stream);
-    cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    const cudaError_t e2 = settle(c);
     dev_free(staging);
     if (e == cudaSuccess)
         e = e2;
@@ -1375,7 +1389,7 @@ static int amplitude_result(pwa_ctx *c, int rc, void *out, size_t bytes, float *
     cudaError_t e = cudaSuccess;
     if (!rc)
         e = cudaMemcpyAsync(out, d, bytes, cudaMemcpyDefault, c->stream);
-    const cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    const cudaError_t e2 = settle(c);
     dev_free(d);
     if (!rc && (e != cudaSuccess || e2 != cudaSuccess)) {
         cudaGetLastError();
@@ -1487,7 +1501,7 @@ static int generate_cov(pwa_ctx *c, const CovTable &table, const double *p3, int
         cudaError_t e = cudaMemcpyAsync(staging, p3, (size_t)n * 9 * sizeof(double),
                                         cudaMemcpyHostToDevice, c->stream);
         if (e != cudaSuccess) {
-            cudaStreamSynchronize(c->stream);
+            settle(c);
             dev_free(staging);
             return fail(c, PWA_ECUDA, "momenta copy: %s", cudaGetErrorString(e));
         }
@@ -1496,7 +1510,7 @@ static int generate_cov(pwa_ctx *c, const CovTable &table, const double *p3, int
     const char *kv = getenv("PWA_AMPGEN_KERNEL");
     cudaError_t e = launch_cov_amp_gen(dk, n, c->N, table, kv && strcmp(kv, "fp64") == 0, out, mode,
                                        pitch, amax, c->num_sms, c->stream);
-    cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    const cudaError_t e2 = settle(c);
     dev_free(staging);
     if (e == cudaSuccess)
         e = e2;
@@ -1699,10 +1713,9 @@ static int build_norm_tc(pwa_ctx *c)
                                  c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&flags, dstat, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    const cudaError_t e2 = settle(c);
     if (e == cudaSuccess)
-        e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess)
-        quiet(c);
+        e = e2;
     dev_free(scratch);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1720,10 +1733,9 @@ static int build_norm_fp64(pwa_ctx *c)
     if (rc)
         return rc;
     cudaError_t e = launch_build_norm(c->mc, c->n_gen, c->M, scratch, c->num_sms, c->stream);
+    const cudaError_t e2 = settle(c);
     if (e == cudaSuccess)
-        e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess)
-        quiet(c);
+        e = e2;
     dev_free(scratch);
     if (e != cudaSuccess) {
         cudaGetLastError();
