@@ -86,14 +86,25 @@ typedef struct pwa_config {
     void *stream;  /* cudaStream_t to run on; NULL = a stream the context owns */
 } pwa_config;
 
-/* Create a context on CUDA device `device`. On success *out owns all device
+/* Create a context on CUDA device `device`. On success *out holds all device
  * memory the library allocates for it; release it with pwa_destroy.
  * Errors: PWA_EINVAL (null out/cfg, n_waves or max_k out of range),
  * PWA_ECUDA (device not usable), PWA_ENOMEM. */
 int pwa_create(pwa_ctx **out, int device, const pwa_config *cfg);
 
-/* Free everything the context owns. Null is accepted. */
+/* Destroy the context. Its device and pinned memory is kept for the contexts that
+ * follow in this process: at most 1/32 of the device's memory and 64 MB of pinned
+ * memory per device; what exceeds that is freed at once, a block that eight sample
+ * loads did not take at the next load, everything when an allocation of the library
+ * fails, by pwa_trim, or at exit. PWA_POOL=0 in the environment keeps nothing. Null is
+ * accepted. */
 int pwa_destroy(pwa_ctx *ctx);
+
+/* Free the memory that destroyed contexts on `device` have left for the next ones, for
+ * instance before another library needs the device's memory; *bytes (may be null) is
+ * how much it was. Contexts that exist are not touched; any thread may call it.
+ * Errors: PWA_ECUDA (device not usable). */
+int pwa_trim(int device, int64_t *bytes);
 
 /* Load the data sample and the accepted MC sample (Eq. 2/3 and the text after
  * Eq. 2: the normalisation integral is a sum over the N_MC^Acc accepted events

@@ -16,7 +16,14 @@ from ._abi import (PWA_C64, PWA_C128, PWA_EDOMAIN, PWA_FORM_AMP, PWA_FORM_TABLE,
 
 __all__ = ["Likelihood", "ModelBatch", "PwaError", "PWA_FORM_AMP", "PWA_FORM_TABLE", "PWA_FORM_TC", "PWA_OK",
            "PWA_EDOMAIN", "PWA_C64", "PWA_C128", "PWA_PREC_DEFAULT", "PWA_PREC_BFP16",
-           "PWA_PREC_BFP8"]
+           "PWA_PREC_BFP8", "trim"]
+
+
+def trim(device=0):
+    """Free the device and pinned memory that closed Likelihoods and ModelBatches have left
+    for the next ones (at most 1/32 of the device); returns its bytes."""
+    from . import _abi
+    return _abi.pwa_trim(device)
 
 
 class Likelihood:

@@ -69,6 +69,7 @@ def load(path=LIB_PATH):
     sig = {
         "pwa_create": ([ctypes.POINTER(ctypes.c_void_p), I, ctypes.POINTER(pwa_config)], I),
         "pwa_destroy": ([P], I),
+        "pwa_trim": ([I, ctypes.POINTER(I64)], I),
         "pwa_load_events": ([P, P, I64, P, I64, D, I], I),
         "pwa_build_norm": ([P, P], I),
         "pwa_set_form": ([P, I], I),
@@ -140,6 +141,13 @@ def pwa_version():
 def pwa_table_bytes(n_waves, n_events):
     out = ctypes.c_int64()
     _check(None, load().pwa_table_bytes(n_waves, n_events, ctypes.byref(out)))
+    return out.value
+
+
+def pwa_trim(device=0):
+    """Bytes of kept memory that were given back."""
+    out = ctypes.c_int64()
+    _check(None, load().pwa_trim(device, ctypes.byref(out)))
     return out.value
 
 

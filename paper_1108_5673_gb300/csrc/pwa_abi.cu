@@ -1213,6 +1213,22 @@ int pwa_destroy(pwa_ctx *c)
     return PWA_OK;
 }
 
+int pwa_trim(int device, int64_t *bytes)
+{
+    if (bytes)
+        *bytes = 0;
+    int ndev = 0;
+    if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) {
+        cudaGetLastError();
+        return fail(nullptr, PWA_ECUDA, "device %d not available (%d devices)", device, ndev);
+    }
+    DeviceGuard g(device);
+    const size_t n = pool_trim();
+    if (bytes)
+        *bytes = (int64_t)n;
+    return PWA_OK;
+}
+
 int pwa_load_events(pwa_ctx *c, const void *data_amp, int64_t n_data, const void *mc_amp,
                     int64_t n_mc_acc, double n_mc_gen, int amp_dtype)
 {

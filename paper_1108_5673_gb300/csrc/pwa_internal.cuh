@@ -427,6 +427,7 @@ cudaError_t pool_alloc(void **p, size_t bytes);  // on the current device
 void pool_free(void *p, bool keep);              // likewise
 cudaError_t pool_host_alloc(void **p, size_t bytes);
 void pool_host_free(void *p, bool keep);
+size_t pool_trim();  // frees what is kept for the current device; returns its bytes
 void pool_loaded();  // a sample was loaded: blocks that many loads did not take are freed
 unsigned long long cuda_context_id();  // of the current CUDA context; changes with a device reset
 // Runs one of the configure functions below once per CUDA context.

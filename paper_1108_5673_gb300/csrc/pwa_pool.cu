@@ -8,14 +8,16 @@
 // blocks are therefore kept for the next context, within bounds:
 //  - at most 1/32 of the device's memory (64 MB of pinned memory) is kept; what
 //    exceeds it is freed at once, oldest first;
-//  - a block that the last 8 sample loads on its device did not take is freed
-//    at the next load;
+//  - a block, device or pinned, that the last 8 sample loads on its device did
+//    not take is freed at the next load;
 //  - an allocation that fails frees everything kept and is tried again;
 //  - PWA_POOL=0 keeps nothing.
+//  - pwa_trim gives back everything kept.
 // Blocks are put back only when the work that may use them has finished (the
-// callers wait for it), so that any stream may use them next. The lists are guarded by one mutex. A device reset
-// invalidates them: they belong to one CUDA context, whose id is compared at
-// each use, and are dropped with it.
+// callers wait for it), so that any stream may use them next. The lists are guarded
+// by one mutex, which is not held while CUDA allocates or frees (a free waits for the
+// device). A device reset invalidates them: they belong to one CUDA context, whose id
+// is compared at each use, and are dropped with it.
 #include <stdlib.h>
 #include <string.h>
 
@@ -70,19 +72,25 @@ bool enabled()
     return on;
 }
 
-void release(Block b, bool host)
-{
-    const cudaError_t e = host ? cudaFreeHost(b.p) : cudaFree(b.p);
-    if (e != cudaSuccess)
-        cudaGetLastError();
-}
+// Blocks that have left the lists, freed when this goes out of scope (after the lock).
+struct Released {
+    bool host;
+    std::vector<Block> blocks;
+    explicit Released(bool h) : host(h) {}
+    ~Released()
+    {
+        for (const Block &b : blocks)
+            if ((host ? cudaFreeHost(b.p) : cudaFree(b.p)) != cudaSuccess)
+                cudaGetLastError();
+    }
+};
 
-// Frees the first n kept blocks.
-void drop(Pool &p, size_t n, bool host)
+// Takes the first n kept blocks off the list.
+void drop(Pool &p, size_t n, Released *out)
 {
     for (size_t i = 0; i < n; ++i) {
         p.kept_bytes -= p.kept[i].size;
-        release(p.kept[i], host);
+        out->blocks.push_back(p.kept[i]);
     }
     p.kept.erase(p.kept.begin(), p.kept.begin() + n);
 }
@@ -126,17 +134,17 @@ void *take(Pool &p, size_t size)
     return b.p;
 }
 
-void put(Pool &p, void *q, bool host)
+void put(Pool &p, void *q, bool keep, Released *out)
 {
     const auto it = p.live.find(q);
-    if (it == p.live.end()) {  // of a context that was reset
-        release(Block{q, 0, 0}, host);
-        return;
+    Block b{q, 0, p.loads};
+    const bool known = it != p.live.end();  // else of a context that was reset
+    if (known) {
+        b.size = it->second;
+        p.live.erase(it);
     }
-    const Block b{q, it->second, p.loads};
-    p.live.erase(it);
-    if (!enabled() || b.size > p.cap) {
-        release(b, host);
+    if (!known || !keep || !enabled() || b.size > p.cap) {
+        out->blocks.push_back(b);
         return;
     }
     p.kept.push_back(b);
@@ -144,19 +152,36 @@ void put(Pool &p, void *q, bool host)
     size_t n = 0, bytes = p.kept_bytes;
     while (bytes > p.cap)
         bytes -= p.kept[n++].size;
-    drop(p, n, host);
+    drop(p, n, out);
 }
 
-Pool *current_pool(bool host)
+// Blocks that the last kKeepLoads loads did not take.
+void age(Pool &p, Released *out)
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+    ++p.loads;
+    size_t n = 0;  // stamps grow along the list
+    while (n < p.kept.size() && p.loads - p.kept[n].stamp > kKeepLoads)
+        ++n;
+    drop(p, n, out);
+}
+
+// The current device and the id of its context (false: no device).
+bool where(int *dev, unsigned long long *id)
+{
+    if (cudaGetDevice(dev) != cudaSuccess || *dev < 0 || *dev >= kMaxDevices) {
         cudaGetLastError();
-        return nullptr;
+        return false;
     }
+    *id = cuda_context_id();
+    return true;
+}
+
+// (with the lock held)
+Pool &pool_of(int dev, unsigned long long id, bool host)
+{
     Pool &p = host ? state().host[dev] : state().dev[dev];
-    renew(p, cuda_context_id());
-    return &p;
+    renew(p, id);
+    return p;
 }
 
 cudaError_t alloc(void **p, size_t bytes, bool host)
@@ -165,32 +190,49 @@ cudaError_t alloc(void **p, size_t bytes, bool host)
         return host ? cudaHostAlloc(p, size, cudaHostAllocMapped) : cudaMalloc(p, size);
     };
     const size_t size = rounded(bytes);
-    State &s = state();
-    std::lock_guard<std::mutex> g(s.lock);
-    Pool *pool = current_pool(host);
-    if (!pool)
+    int dev;
+    unsigned long long id;
+    if (!where(&dev, &id))
         return fresh(bytes);
-    if ((*p = take(*pool, size)))
-        return cudaSuccess;
-    cudaError_t e = fresh(size);
-    if (e == cudaErrorMemoryAllocation && !pool->kept.empty()) {
-        cudaGetLastError();
-        drop(*pool, pool->kept.size(), host);
-        e = fresh(size);
+    State &s = state();
+    size_t cap;
+    {
+        std::lock_guard<std::mutex> g(s.lock);
+        Pool &pool = pool_of(dev, id, host);
+        if ((*p = take(pool, size)))
+            return cudaSuccess;
+        cap = pool.cap;
     }
-    if (e != cudaSuccess) {
-        *p = nullptr;
-        return e;
-    }
-    if (!pool->cap) {
+    if (!cap) {
         size_t free_bytes = 0, total = 0;
         if (host)
             total = 32 * kHostCap;
         else if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess)
             cudaGetLastError();
-        pool->cap = total / 32;
+        cap = total / 32;
     }
-    pool->live[*p] = size;
+    cudaError_t e = fresh(size);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        bool any;
+        {
+            Released out(host);
+            std::lock_guard<std::mutex> g(s.lock);
+            Pool &pool = pool_of(dev, id, host);
+            any = !pool.kept.empty();
+            drop(pool, pool.kept.size(), &out);
+        }
+        if (any)
+            e = fresh(size);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        return e;
+    }
+    std::lock_guard<std::mutex> g(s.lock);
+    Pool &pool = pool_of(dev, id, host);
+    pool.cap = cap;
+    pool.live[*p] = size;
     return cudaSuccess;
 }
 
@@ -198,16 +240,15 @@ void give_back(void *p, bool host, bool keep)
 {
     if (!p)
         return;
-    State &s = state();
-    std::lock_guard<std::mutex> g(s.lock);
-    Pool *pool = current_pool(host);
-    if (pool && keep) {
-        put(*pool, p, host);
-    } else {
-        if (pool)
-            pool->live.erase(p);
-        release(Block{p, 0, 0}, host);
+    Released out(host);
+    int dev;
+    unsigned long long id;
+    if (!where(&dev, &id)) {
+        out.blocks.push_back(Block{p, 0, 0});
+        return;
     }
+    std::lock_guard<std::mutex> g(state().lock);
+    put(pool_of(dev, id, host), p, keep, &out);
 }
 
 }  // namespace
@@ -243,16 +284,29 @@ void pool_host_free(void *p, bool keep) { give_back(p, true, keep); }
 
 void pool_loaded()
 {
-    State &s = state();
-    std::lock_guard<std::mutex> g(s.lock);
-    Pool *pool = current_pool(false);
-    if (!pool)
+    Released dev_out(false), host_out(true);
+    int dev;
+    unsigned long long id;
+    if (!where(&dev, &id))
         return;
-    ++pool->loads;
-    size_t n = 0;  // stamps grow along the list
-    while (n < pool->kept.size() && pool->loads - pool->kept[n].stamp > kKeepLoads)
-        ++n;
-    drop(*pool, n, false);
+    std::lock_guard<std::mutex> g(state().lock);
+    age(pool_of(dev, id, false), &dev_out);
+    age(pool_of(dev, id, true), &host_out);
+}
+
+size_t pool_trim()
+{
+    Released dev_out(false), host_out(true);
+    int dev;
+    unsigned long long id;
+    if (!where(&dev, &id))
+        return 0;
+    std::lock_guard<std::mutex> g(state().lock);
+    Pool &d = pool_of(dev, id, false), &h = pool_of(dev, id, true);
+    const size_t bytes = d.kept_bytes + h.kept_bytes;
+    drop(d, d.kept.size(), &dev_out);
+    drop(h, h.kept.size(), &host_out);
+    return bytes;
 }
 
 cudaError_t configure_once(int which, cudaError_t (*configure)())
