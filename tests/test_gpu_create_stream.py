@@ -31,6 +31,7 @@ def test_default_stream_busy(pwa, fp64_norm):  # noqa: F811
             assert L._abi.load().pwa_build_norm(L.ctx, None) == 0
             return [L.nll_grad(V) for _ in range(50)]
 
+    pwa.trim()      # no block left by others to be freed, which would wait, meanwhile
     want = session()[0]
     session()
     for _ in range(3):
