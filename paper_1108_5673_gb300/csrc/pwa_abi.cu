@@ -1908,6 +1908,15 @@ static int bfail(pwa_batch *b, int code, const char *fmt, ...)
     return code;
 }
 
+// Waits for the batch's work; whether memory it used may be kept.
+static bool batch_quiet(pwa_batch *b)
+{
+    const bool ok = !b->stream || cudaStreamSynchronize(b->stream) == cudaSuccess;
+    if (!ok)
+        cudaGetLastError();
+    return ok;
+}
+
 static void batch_drop_graph(pwa_batch *b)
 {
     if (b->exec)
@@ -1915,7 +1924,7 @@ static void batch_drop_graph(pwa_batch *b)
     b->exec = nullptr;
     b->graph_k = 0;
     if (b->plan)
-        cudaFree(b->plan);
+        pool_free(b->plan, batch_quiet(b));
     b->plan = nullptr;
     b->plan_bytes = 0;
 }
@@ -1951,8 +1960,7 @@ int pwa_batch_destroy(pwa_batch *b)
     if (!b)
         return PWA_OK;
     DeviceGuard g(b->device);
-    if (b->stream)
-        cudaStreamSynchronize(b->stream);
+    const bool keep = batch_quiet(b);
     batch_drop_graph(b);
     for (pwa_ctx *c : b->models)
         pwa_destroy(c);
@@ -1964,10 +1972,8 @@ int pwa_batch_destroy(pwa_batch *b)
     }
     if (b->ev_fork)
         cudaEventDestroy(b->ev_fork);
-    if (b->d_buf)
-        cudaFree(b->d_buf);
-    if (b->h_buf)
-        cudaFreeHost(b->h_buf);
+    pool_free(b->d_buf, keep);
+    pool_host_free(b->h_buf, keep);
     if (b->own_stream && b->stream)
         cudaStreamDestroy(b->stream);
     delete b;
@@ -2039,8 +2045,8 @@ int pwa_batch_create(pwa_batch **out, int device, int n_models, const int *n_wav
         b->models.push_back(c);
     }
     const size_t nd = 4 * (size_t)max_k * b->sum_n + (size_t)n_models * max_k + n_models;
-    if (cudaMalloc((void **)&b->d_buf, nd * sizeof(double)) != cudaSuccess ||
-        cudaMallocHost((void **)&b->h_buf, nd * sizeof(double)) != cudaSuccess) {
+    if (pool_alloc((void **)&b->d_buf, nd * sizeof(double)) != cudaSuccess ||
+        pool_host_alloc((void **)&b->h_buf, nd * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return bail(bfail(b, PWA_ENOMEM, "batch io buffers (%zu doubles)", nd));
     }
@@ -2097,7 +2103,7 @@ static int batch_prepare(pwa_batch *b, int K)
             descs = batch_descs(b, K);
             b->plan_bytes = batched_plan_bytes(descs.data(), nm, xs, K, b->num_sms,
                                                b->items_per_sm, nullptr);
-            if (cudaMalloc(&b->plan, b->plan_bytes) != cudaSuccess) {
+            if (pool_alloc(&b->plan, b->plan_bytes) != cudaSuccess) {
                 cudaGetLastError();
                 b->plan = nullptr;
                 return bfail(b, PWA_ENOMEM, "batch plan (%zu bytes)", b->plan_bytes);

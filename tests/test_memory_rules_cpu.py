@@ -36,3 +36,11 @@ def test_buffers_of_a_context_go_back_after_a_wait():
                             r"cudaGraphExecDestroy|graphs", lines[k]):
                 k -= 1
             assert "quiet(c)" in lines[k], (i + 1, lines[k])
+
+
+def test_all_memory_is_the_pools():
+    """An allocation that fails frees everything kept and is tried again: only where it is
+    made through the pool, so all of them are, the model batch's plan and buffers too."""
+    for i, line in enumerate(code()):
+        assert not re.search(r"\b(cudaMalloc|cudaMallocHost|cudaHostAlloc|cudaFree|cudaFreeHost|cudaMallocAsync)\(",
+                             line), (i + 1, line)
