@@ -170,9 +170,10 @@ struct HessCfg {
 __device__ __forceinline__ constexpr int hess_place(int x, int sb) { return (x & 1) * sb + (x >> 1); }
 
 // The sums of many FP32 runs are float pairs (this part's FP64 pipe has 1/64 of
-// the FP32 rate: as doubles the conversions and sums of one block took 15 us),
-// scaled so that they overflow no earlier than the FP32 sums they are made of.
-constexpr float kSumScale = 0x1p-20f;
+// the FP32 rate: as doubles the conversions and sums of one block took 15 us). Every
+// FP32 sum is a multiple of 2^-149, so that a pair loses nothing to underflow that
+// its terms had not lost; a total that a float may not hold is added in FP64.
+__device__ __forceinline__ bool is_wide(float h) { return !(fabsf(h) < 0x1p100f); }
 
 __device__ __forceinline__ float half_of(f2 v, int odd)
 {
@@ -188,10 +189,21 @@ __device__ __forceinline__ void sum2(float &h, float &l, float x)
     h = t;
 }
 
+// The sum of n pairs, `stride` apart, in FP64. (A call, so that the kernels' own code
+// stays as it is without it.)
+__device__ __noinline__ double wide_sum(const float2 *v, int n, int stride)
+{
+    double d = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i)
+        d += (double)v[(size_t)i * stride].x + (double)v[(size_t)i * stride].y;
+    return d;
+}
+
 // Eight warps form J of the next tile (one event per thread, the tile after that
 // being loaded) while up to six add the products of the current one; two tile
-// buffers, one barrier per tile. Every kFlush tiles the FP32 sums go to FP64
-// sums in global scratch (they would take twice the registers of the products).
+// buffers, one barrier per tile. Every kFlush tiles the FP32 sums go to float pairs
+// in global scratch (they would take twice the registers of the products).
 //
 // Bound by instruction issue of the two parts together: at 32 waves the products
 // alone take 4.3 us a tile and SM (packed FMAs, two to an instruction; single
@@ -344,7 +356,7 @@ __global__ void __launch_bounds__(HessCfg<NP>::WARPS * 32, 1)
                         for (int q = 0; q < 8; ++q) {
                             float2 *x = acc + (size_t)(8 * r + q) * kHT;
                             float2 v = flushed ? *x : make_float2(0.f, 0.f);
-                            sum2(v.x, v.y, kSumScale * half_of(s[r][q >> 1], q & 1));
+                            sum2(v.x, v.y, half_of(s[r][q >> 1], q & 1));
                             *x = v;
                         }
 #pragma unroll
@@ -365,7 +377,7 @@ __global__ void __launch_bounds__(HessCfg<NP>::WARPS * 32, 1)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     float2 v = flushed ? acc[(size_t)(8 * r + q) * kHT] : make_float2(0.f, 0.f);
-                    sum2(v.x, v.y, kSumScale * half_of(s[r][q >> 1], q & 1));
+                    sum2(v.x, v.y, half_of(s[r][q >> 1], q & 1));
                     sums[(size_t)((half * C::R + r) * 8 + q) * C::NS] = v;
                 }
         }
@@ -382,20 +394,28 @@ __global__ void __launch_bounds__(HessCfg<NP>::WARPS * 32, 1)
             sum2(h, l, v.x);
             l += v.y;
         }
+        if (is_wide(h)) {  // in FP64 at the block's scratch, which is free now
+            reinterpret_cast<double *>(scratch)[(size_t)blockIdx.x * (64 * kHT) + q] =
+                wide_sum(sums + q, C::EG, 64 * C::NS);
+            h = INFINITY;
+            l = 0.f;
+        }
         out[q] = make_float2(h, l);
     }
 }
 
 // H[r][c] over the real parameters (Re V at 0..N-1, Im V at N..2N-1) from the
-// blocks' sums [grid][64][NS]: 32 entries per block, one per lane, its 8 warps
-// taking every eighth of the grid, then added in order, so that the order is the
-// same on every run; zero when a data intensity was not positive. With async_or
-// set, the status bits of the call are also OR-ed into *async_or.
+// blocks' sums [grid][64][NS] (infinite: a double in the block's scratch): 32 entries
+// per block, one per lane, its 8 warps taking every eighth of the grid, then added in
+// order, so that the order is the same on every run; zero when a data intensity was
+// not positive. With async_or set, the status bits of the call are also OR-ed into
+// *async_or.
 __global__ void __launch_bounds__(256)
-    hess_finalize(const float2 *partials, int grid, int NP, int N, const int *status, double *H,
-                  int *async_or)
+    hess_finalize(const float2 *partials, const float2 *scratch, int grid, int NP, int N,
+                  const int *status, double *H, int *async_or)
 {
     __shared__ float2 part[8][32];
+    __shared__ double part_wide[8][32];
     const int flags = *status;
     if (async_or && blockIdx.x == 0 && threadIdx.x == 0 && flags)
         atomicOr(async_or, flags);
@@ -409,6 +429,18 @@ __global__ void __launch_bounds__(256)
             sum2(h, l, v.x);
             l += v.y;
         }
+        if (!(fabsf(h) < INFINITY)) {  // a block's sum in FP64 was among them
+            double d = 0.0;
+#pragma unroll 1
+            for (int b = warp; b < grid; b += 8) {
+                const float2 v = partials[(size_t)b * NS * 64 + o];
+                d += isinf(v.x) ? reinterpret_cast<const double *>(scratch)[(size_t)b * (64 * kHT) + o]
+                                  : (double)v.x + (double)v.y;
+            }
+            part_wide[warp][lane] = d;
+            h = INFINITY;
+            l = 0.f;
+        }
     }
     part[warp][lane] = make_float2(h, l);
     __syncthreads();
@@ -417,6 +449,15 @@ __global__ void __launch_bounds__(256)
     for (int w = 1; w < 8; ++w) {
         sum2(h, l, part[w][lane].x);
         l += part[w][lane].y;
+    }
+    double total = (double)h + (double)l;
+    if (!(fabsf(h) < INFINITY)) {
+        total = 0.0;
+#pragma unroll 1
+        for (int w = 0; w < 8; ++w) {
+            const float2 v = part[w][lane];
+            total += isinf(v.x) ? part_wide[w][lane] : (double)v.x + (double)v.y;
+        }
     }
     int y = o % NS, x = 0;
     const int q = o / NS;
@@ -429,9 +470,7 @@ __global__ void __launch_bounds__(256)
     if (r >= N || c >= N || pr > pc)
         return;
     const int hr = pr < NP ? r : N + r, hc = pc < NP ? c : N + c, P = 2 * N;
-    const double v = (flags & FLAG_DOMAIN) ? 0.0
-                     : isfinite(h) ? ((double)h + (double)l) / (double)kSumScale
-                                   : (double)h;
+    const double v = (flags & FLAG_DOMAIN) ? 0.0 : total;
     H[hr * P + hc] = v;
     H[hc * P + hr] = v;
 }
@@ -504,7 +543,8 @@ cudaError_t hess_np(const Planes &d, const double *V, double *part, int grid, in
                                                    sums + (size_t)grid * C::NS * 64, status);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    hess_finalize<<<C::NS * 2, 256, 0, s>>>(sums, grid, NP, d.n_waves, status, H, async_or);
+    hess_finalize<<<C::NS * 2, 256, 0, s>>>(sums, sums + (size_t)grid * C::NS * 64, grid, NP, d.n_waves,
+                                            status, H, async_or);
     return cudaGetLastError();
 }
 
