@@ -24,8 +24,9 @@
 //    1.25 sum_a |V_a|_1 max |A_a|_1 over both samples, with |BW_r| <= 1/(M_r G_r)
 //    for the free waves;
 //  * ln I = e ln 2 + ln f, e and round(2^23 ln f) summed as integers; the MC
-//    sum of I and all gradients in FP32 per thread, float-float per warp and
-//    block, FP64 across blocks in a fixed order (the last CTA, atomic ticket).
+//    sum of I in float-float per thread, the gradients in FP32 per thread and
+//    warp, FP64 per block; across blocks the logarithms and intensities in FP64, the
+//    gradients as float pairs, in a fixed order (the last CTA, atomic ticket).
 // Every wait is bounded (FLAG_TIMEOUT) so a stalled pipeline returns.
 //
 // Bound by the FP32 pipe's latency before HBM: with both passes in one warp per
@@ -112,14 +113,22 @@ __device__ __forceinline__ f2 rcp2(f2 a)
 // A CTA's sum of value `item` of [2][P] (data, MC) for the last CTA, in a.partials
 // [grid][2 P]: the ln I, exponent and intensity sums (the first two of each P) as they
 // are, the gradients, which come from FP32 sums, as float pairs, since the FP64 pipe
-// (1/64 of the FP32 rate) was what the final sums took their time for.
+// (1/64 of the FP32 rate) was what the final sums took their time for. (Their terms are
+// multiples of 2^-149: nothing is lost to underflow.) A sum whose total a float may not
+// hold is kept as a double in a second [grid][2 P], its pair's high part infinite.
 __device__ __forceinline__ void res_partial(const ResArgs &a, int item, int P, double v)
 {
+    const size_t at = (size_t)blockIdx.x * 2 * P + item;
     if (item % P >= 2) {
-        const float h = (float)v, l = (float)(v - (double)h);
+        float h = (float)v, l = (float)(v - (double)h);
+        if (!(fabsf(h) < 0x1p100f)) {
+            a.partials[(size_t)gridDim.x * 2 * P + at] = v;
+            h = INFINITY;
+            l = 0.f;
+        }
         v = __hiloint2double(__float_as_int(l), __float_as_int(h));
     }
-    a.partials[(size_t)blockIdx.x * 2 * P + item] = v;
+    a.partials[at] = v;
 }
 
 template <int NP, int RP>
@@ -546,6 +555,7 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
         const int item = t % n, sl = t / n;
         double v = 0.0;
         dfloat f = {0.f, 0.f};
+        bool wide = false;
         for (int b0 = sl; b0 < n_cta; b0 += 8 * slices) {
             double r[8];
 #pragma unroll
@@ -555,14 +565,27 @@ __global__ void __launch_bounds__(ResTmaCfg<NP, RP>::THREADS, 1)
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                if (item % P < 2)
+                if (item % P < 2) {
                     v += r[q];
-                else
-                    f = df_add(f, dfloat{__int_as_float(__double2loint(r[q])),
-                                         __int_as_float(__double2hiint(r[q]))});
+                } else {
+                    const float h = __int_as_float(__double2loint(r[q]));
+                    wide = wide || h == INFINITY;
+                    f = df_add(f, dfloat{h, __int_as_float(__double2hiint(r[q]))});
+                }
             }
         }
-        fin[t] = item % P < 2 ? v : (double)f.hi + (double)f.lo;
+        if (item % P >= 2)
+            v = (double)f.hi + (double)f.lo;
+        if (wide) {
+            v = 0.0;
+            for (int b = sl; b < n_cta; b += slices) {
+                const double *x = a.partials + (size_t)b * n + item, r = __ldcg(x);
+                const float h = __int_as_float(__double2loint(r));
+                v += h == INFINITY ? __ldcg(x + (size_t)n_cta * n)
+                                   : (double)h + (double)__int_as_float(__double2hiint(r));
+            }
+        }
+        fin[t] = v;
     }
     __syncthreads();
     double tot = 0.0;

@@ -717,7 +717,7 @@ int pwa_version(void) { return 100; }
 
 const char *pwa_last_error(const pwa_ctx *ctx) { return ctx ? ctx->err : g_create_err; }
 
-constexpr int kResMaxBlocksPerSm = 3;
+constexpr int kResMaxBlocksPerSm = 3;  // (the TMA-fed kernel, one CTA per SM, takes scratch for two)
 static size_t res_grid(const pwa_ctx *c) { return (size_t)c->num_sms * c->tune_res_cps; }
 
 int pwa_load_resonance_events(pwa_ctx *c, int n_free, const double *m_data, const void *Y_data,

@@ -507,7 +507,7 @@ struct ResArgs {
     int64_t mc_pitch, n_mc;
     double inv_ngen;
     const double *V, *mass, *width;  // device
-    double *partials;    // 2 pstride grid (the order is the kernel's)
+    double *partials;    // 2 pstride grid (the order is the kernel's; the TMA-fed one: twice that)
     unsigned *ticket;    // zero on entry, left at zero
     int *status;         // status bits OR-ed here
     int *done;           // incremented once (may be null)
@@ -520,7 +520,7 @@ cudaError_t launch_nll_res(const ResArgs &a, int grid, cudaStream_t s);
 // k_nll_res_tma.cu: the same evaluation, TMA-fed (maps over the [1 + 2N]
 // planes of each sample with a box of res_tma_box_events() events x 1 + 2N
 // rows); amax[a] >= max over both samples of |Re| + |Im| of Y_a (free waves)
-// or A_a (fixed waves). Scratch as launch_nll_res with grid = one CTA per SM.
+// or A_a (fixed waves). Scratch as launch_nll_res with twice the grid.
 int res_tma_box_events();
 bool res_tma_available(int n_waves, int n_free);
 cudaError_t launch_nll_res_tma(const CUtensorMap *dmap, const CUtensorMap *mmap, const ResArgs &a,
