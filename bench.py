@@ -66,14 +66,14 @@ WORKLOAD = "1M data events x 20 waves (FP32 amplitudes, direct form), M from 5M 
 # capture of the current kernel, or None where there is none.
 TRAFFIC = {"direct": 160.139776e6 + 3.347968e6,
            "table": 1600.119e6 + 3.221760e6,
-           "tc": 2 * (1024.872e6 + 3.708160e6),        # a step is two launches of 128 sets
-           "res": 1148.176e6 + 3.313920e6,             # the same bytes since its S warps
+           "tc": 2 * (1024.895e6 + 3.099136e6),        # a step is two launches of 128 sets
+           "res": 1148.350e6 + 4.946432e6,
            "models": None,
-           "hessian": 160.091648e6 + 3.346944e6,
+           "hessian": 160.105216e6 + 2.952448e6,
            "weights": 800.125184e6 + 21.052672e6,
-           "incoh": None,          # kernel changed since its capture
+           "incoh": 320.117248e6 + 3.076608e6,
            "incoh_table": None,   # the table kernel's capture is of the coherent sample
-           "ampgen": None,         # kernel changed since its capture
+           "ampgen": 129.669376e6 + 740.991744e6,   # the last 60 MB of the output stay in L2
            "direct_4M_32": None,   # kernel changed since its capture (four-warp groups, amplitudes re-read)
            "cov_ampgen": None}     # kernel changed since its capture
 KERNELS = {"direct": "nll_amp_kernel<20, 2>", "table": "nll_table_kernel<20>",
@@ -528,7 +528,7 @@ def job_ampgen(pwa, torch, stream, local, rank):
                  "kinematics (as rounded from FP64 to complex64, out to a device buffer)",
         config={"n_waves": N_WAVES, "n_events": n, "flops_per_event": ampgen_flops(waves)},
         roof={"bound": "hbm", "bytes": (24.0 + 8.0 * N_WAVES) * n},
-        dtype="f64", h2d=24 * n, d2h=8 * N_WAVES * n, cpu_baseline=cpu_baseline,
+        dtype="f32 pairs, f64 where they cannot decide the rounding", h2d=24 * n, d2h=8 * N_WAVES * n, cpu_baseline=cpu_baseline,
         note="e2e passes host kinematics in (120 MB) and takes the amplitudes back (800 MB)")
 
 
@@ -572,7 +572,7 @@ def job_cov_ampgen(pwa, torch, stream, local, rank):
         config={"n_waves": N, "n_events": n, "components": 4,
                 "flops_per_event": cov_ampgen_flops(N)},
         roof={"bound": "hbm", "bytes": (72.0 + 32.0 * N) * n},
-        dtype="f64", h2d=72 * n, d2h=32 * N * n, cpu_baseline=cpu_baseline,
+        dtype="f32 pairs, f64 where they cannot decide the rounding", h2d=72 * n, d2h=32 * N * n, cpu_baseline=cpu_baseline,
         note="e2e passes host 3-momenta in (360 MB) and takes the amplitudes back (1.9 GB)")
 
 

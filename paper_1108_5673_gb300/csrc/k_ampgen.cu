@@ -10,13 +10,14 @@
 // and took 6.35 ms for 5M events x 20 waves. Here the values are formed in
 // float-float (ff.cuh, ~44 bits, two events per thread in packed FP32) with a
 // bound on their error, and rounded where the bound leaves no doubt which
-// float is nearest (Ziv's test). An amplitude in doubt (one in ~20 events),
-// and an event whose inputs leave the float-float range, go to a queue per
+// float is nearest (Ziv's test). An amplitude in doubt (one in 1240 at 20
+// waves with l up to 4, in 240 at 40 with l up to 10), and an event whose inputs or
+// products leave the float-float range, go to a queue per
 // warp and are evaluated in FP64 a warp's worth at a time: one by one, by the
 // lane concerned, they took as long as the rest (1.35 ms in all). Measured at
-// 5M x 20: 0.69 ms (1.3 TB/s of the 0.92 GB), at 2M x 40 with l up to 10: 0.98
+// 5M x 20: 0.69 ms (1.3 TB/s of the 0.92 GB), at 2M x 40 with l up to 10: 0.86
 // ms against 7.6, at 5M x 4: 0.22 ms against 1.48; bound by instruction issue
-// (57% of the slots, most of the rest packed FP32 instructions that take two).
+// (60% of the slots, most of the rest packed FP32 instructions that take two).
 //
 // The waves are visited in order of (|m|, l), so that
 // e^{i m phi}, P_m^m and the upward recurrence in l continue from wave to wave

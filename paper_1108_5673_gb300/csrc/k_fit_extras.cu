@@ -208,8 +208,8 @@ __device__ __noinline__ double wide_sum(const float2 *v, int n, int stride)
 // Bound by instruction issue of the two parts together: at 32 waves the products
 // alone take 4.3 us a tile and SM (packed FMAs, two to an instruction; single
 // ones made the call a third slower), forming J alone 4.3 to 5.8, both 6.9. One
-// call at 333k events x 29 waves 172 to 96 us, at 1M x 32 405 to 248 us, at 500k
-// x 48 499 to 210 us, against one 256-thread role that did both in turn, with
+// call at 333k events x 29 waves 172 to 98 us, at 1M x 32 404 to 245 us, at 500k
+// x 48 494 to 212 us, against one 256-thread role that did both in turn, with
 // 4x4 blocks (two 16-byte loads for 16 products, here four for 64).
 template <int NP>
 __global__ void __launch_bounds__(HessCfg<NP>::WARPS * 32, 1)

@@ -32,10 +32,12 @@
 // Bound by the FP32 pipe's latency before HBM: with both passes in one warp per
 // unit (seven warps per SM at 255 registers) 36% of the issue slots were used.
 // Twelve S warps and twelve gradient warps (72 registers) keep every sum's
-// order. Per call at 2M + 5M events x 20 waves, 4 free: 291 us (3.9 TB/s), 373
+// order. Per call at 2M + 5M events x 20 waves, 4 free: 287 us (4.0 TB/s), 372
 // before; with S warps that also waited for each other's tiles 303, and then six and
-// six warps 330, nine and six 315, fifteen and twelve 303. At 12 waves, 3 free 214
-// (279), at 28 and 4, 1M + 2.5M events 255 (291). Splitting a
+// six warps 330, nine and six 315, fifteen and twelve 303. At 12 waves, 3 free 213
+// (277); 1M + 2.5M events: 28 and 4 255 (288), 16 and 8 188 (250), 20 and 8 215 (274), 24
+// and 8 250 (301), 32 and 8 298 (434), although 72 registers make the larger ones spill
+// (20 and 4: 104 bytes a thread stored, 20 to 32 and 8: 356 to 384). Splitting a
 // unit's waves over two warps in the S pass too changes the order of S's
 // remainders and with it the last digits of the gradients (3.6e-9).
 #include <numeric>
